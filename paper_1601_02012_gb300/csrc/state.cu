@@ -6,16 +6,31 @@ namespace rr {
 namespace {
 
 // Rows [row0, row0 + nrows) of an nx x ny bundle; rid counts from row row0.
-__global__ void init_directions_kernel(int nx, int ny, int row0, int nrows, double fov_x, double fov_y,
-                                       double* dir, float4* dirh, float4* dirl)
+//
+// Bound by the FP64 pipe (sincos, a square root and two divisions a ray, on a
+// GPU whose FP64 rate is 1/64 of its FP32 rate), not by the 56 bytes a ray
+// writes. The angle grid of Eq. (txty) is antisymmetric, theta(n - 1 - i) =
+// -theta(i) exactly, and theta_x, theta_y enter theta only squared: one thread
+// computes |theta|, its sine and cosine and the two quotients once and writes
+// the four rays (+-theta_x, +-theta_y), whose components differ in sign only
+// (bit for bit what each ray's own evaluation gives). A thread's first ray is
+// (ix, iy) in the lower quarter of the whole bundle; of its rows only those in
+// the band are written. (kx, ky: fov / (2 (n - 1)), divided on the host.)
+// 2048^2 rays: 679 us with one evaluation a ray, 143 us now (1024^2: 171 -> 39).
+__global__ void init_directions_kernel(int nx, int ny, int row0, int nrows, double kx, double ky, double* dir,
+                                       float4* dirh, float4* dirl)
 {
-    const long long rid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (rid >= (long long)nx * nrows) return;
-    const int ix = (int)(rid % nx), iy = row0 + (int)(rid / nx);
+    const int hx = (nx + 1) / 2, hy = (ny + 1) / 2;
+    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= (long long)hx * hy) return;
+    const int ix = (int)(q % hx), iy = (int)(q / hx);
+    const int mx = nx - 1 - ix, my = ny - 1 - iy;
+    const bool lower = iy >= row0 && iy < row0 + nrows, upper = my != iy && my >= row0 && my < row0 + nrows;
+    if (!lower && !upper) return;
     // Eq. (txty) with 0-based pixel indices, as (2i - (N-1)) U / (2(N-1)): the
     // central pixel of an odd row is at exactly 0; a single ray per side sits at 0
-    const double tx = nx > 1 ? (double)(2 * ix - (nx - 1)) * (fov_x / (2.0 * (nx - 1))) : 0.0;
-    const double ty = ny > 1 ? (double)(2 * iy - (ny - 1)) * (fov_y / (2.0 * (ny - 1))) : 0.0;
+    const double tx = nx > 1 ? (double)(2 * ix - (nx - 1)) * kx : 0.0;
+    const double ty = ny > 1 ? (double)(2 * iy - (ny - 1)) * ky : 0.0;
     const double th = sqrt(tx * tx + ty * ty);
     double n0 = 0.0, n1 = 0.0, n2 = 1.0;
     if (th > 0.0) {
@@ -26,12 +41,25 @@ __global__ void init_directions_kernel(int nx, int ny, int row0, int nrows, doub
         n1 = s * (ty / th);
         n2 = c;
     }
-    dir[3 * rid] = n0;
-    dir[3 * rid + 1] = n1;
-    dir[3 * rid + 2] = n2;
     const float h0 = (float)n0, h1 = (float)n1, h2 = (float)n2;
-    dirh[rid] = make_float4(h0, h1, h2, 0.f);
-    dirl[rid] = make_float4((float)(n0 - (double)h0), (float)(n1 - (double)h1), (float)(n2 - (double)h2), 0.f);
+    const float l0 = (float)(n0 - (double)h0), l1 = (float)(n1 - (double)h1), l2 = (float)(n2 - (double)h2);
+    auto put = [&](int x, int y, bool fx, bool fy) {
+        const long long rid = (long long)(y - row0) * nx + x;
+        // (0 - v, not -v: a zero component stays +0, as in the ray's own evaluation)
+        dir[3 * rid] = fx ? 0.0 - n0 : n0;
+        dir[3 * rid + 1] = fy ? 0.0 - n1 : n1;
+        dir[3 * rid + 2] = n2;
+        dirh[rid] = make_float4(fx ? 0.f - h0 : h0, fy ? 0.f - h1 : h1, h2, 0.f);
+        dirl[rid] = make_float4(fx ? 0.f - l0 : l0, fy ? 0.f - l1 : l1, l2, 0.f);
+    };
+    if (lower) {
+        put(ix, iy, false, false);
+        if (mx != ix) put(mx, iy, true, false);
+    }
+    if (upper) {
+        put(ix, my, false, true);
+        if (mx != ix) put(mx, my, true, true);
+    }
 }
 
 __device__ __forceinline__ double ff(float2 v) { return (double)v.x + (double)v.y; }
@@ -128,10 +156,11 @@ cudaError_t launch_init_directions(const rr_bundle_desc& b, double* dir, float4*
                                    int row0, int nrows)
 {
     if (nrows < 0) nrows = b.ny;
-    const long long nr = (long long)b.nx * nrows;
+    const long long quarter = (long long)((b.nx + 1) / 2) * ((b.ny + 1) / 2);
+    const double kx = b.nx > 1 ? b.fov_x / (2.0 * (b.nx - 1)) : 0.0, ky = b.ny > 1 ? b.fov_y / (2.0 * (b.ny - 1)) : 0.0;
     const int nt = 256;
-    init_directions_kernel<<<(unsigned)((nr + nt - 1) / nt), nt, 0, s>>>(b.nx, b.ny, row0, nrows, b.fov_x, b.fov_y,
-                                                                          dir, dirh, dirl);
+    init_directions_kernel<<<(unsigned)((quarter + nt - 1) / nt), nt, 0, s>>>(b.nx, b.ny, row0, nrows, kx, ky, dir, dirh,
+                                                                             dirl);
     return cudaGetLastError();
 }
 
