@@ -115,10 +115,12 @@ TraceArgs make_trace_args(const rr_bundle_desc& b, const RayState& st, const rr_
     a.inv_chi_s_f = (float)(1.0 / b.chi_s);
     a.sub_len = (float)(32.0 * a.h);
     a.periodic = (b.flags & RR_PERIODIC) ? 1 : 0;
-    // flat addressing over the whole grid's records
+    // flat addressing over the whole grid's records (32-bit point indices: a
+    // grid of 2^31 points or more gets an empty box, which no sub-step lies in)
+    const bool small = (long long)grid->n[0] * grid->n[1] * grid->n[2] < (1LL << 31);
     for (int i = 0; i < 3; ++i) {
         a.fo[i] = 0;
-        a.fe[i] = grid->n[i];
+        a.fe[i] = small ? grid->n[i] : 0;
     }
     a.fs0 = grid->n[1] * grid->n[2];
     a.fs1 = grid->n[2];

@@ -208,7 +208,9 @@ rr_status rr_batch_trace(rr_batch* b, void* stream)
     a.counter = b->d_counter;
     a.chunk = b->chunk;
     a.tile = b->tile;
-    return status_of_cuda(launch_trace_batch(a, b->interp, b->fp64, grid_blocks(b), s));
+    bool small = true;
+    for (int i = 0; i < n; ++i) small = small && b->h_args[i].fe[0] > 0;
+    return status_of_cuda(launch_trace_batch(a, b->interp, b->fp64, grid_blocks(b), s, small));
 }
 
 rr_status rr_batch_finalize(rr_batch* b, double* const* kappa, double* const* kappa_born, void* stream)

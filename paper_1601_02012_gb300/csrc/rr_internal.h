@@ -146,13 +146,14 @@ cudaError_t launch_trace(const TraceArgs& a, int interp, bool fp64_dda, cudaStre
 // Forms of the FP32 walk's sums.
 enum { kFormKahan = 0, kFormPlain = 1, kFormMoments = 2, kFormShear = 3, kFormMethodA = 4, kFormGeneric = 5 };
 // Record addressing of the trilinear walk (see trace.cu).
-enum { kAddrIndex = 0, kAddrPlanes = 1, kAddrFlat = 2 };
+enum { kAddrIndex = 0, kAddrPlanes = 1, kAddrFlat = 2, kAddrAuto = 3 };
 // flat: the caller has checked that no ray of the step comes within a cell of
 // the periodic seam and that the grid has fewer than 2^31 points (used by the
 // default FP32 trilinear periodic form only; ignored otherwise).
 cudaError_t launch_trace(const TraceArgs& a, int interp, bool fp64_dda, cudaStream_t s, const TileCfg& t,
                          int form = kFormKahan, bool flat = false);
-cudaError_t launch_trace_batch(const BatchArgs& b, int interp, bool fp64_dda, int blocks, cudaStream_t s);
+// small: every bundle's grid has fewer than 2^31 points
+cudaError_t launch_trace_batch(const BatchArgs& b, int interp, bool fp64_dda, int blocks, cudaStream_t s, bool small);
 // Steps b.s[0 .. b.n) of an FP32 compensated form (kFormKahan, kFormShear,
 // kFormMoments, kFormMethodA, kFormGeneric) in one launch; a holds the shared
 // fields. flat: every step passed the flat-addressing check (trilinear).

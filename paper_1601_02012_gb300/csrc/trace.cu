@@ -69,6 +69,36 @@ __device__ __forceinline__ void shift_corners(float2 q[8], const float2 p[4], in
     }
 }
 
+// What the sub-steps of one ray's step accumulate and hand on.
+template <class R>
+struct PieceState {
+    // per-step sums of (kappa, Born kappa): packed Kahan pairs (FP32) or FP64
+    Acc2 s2;
+    Acc2 s2m;   // moments form: the B moments; shear form: (gamma1, gamma2)
+    Acc<R> sk, sb;
+    // Method A: n . grad Phi and g at the start and at the end of the interval
+    float qa = 0.f, ga = 0.f, qb = 0.f, gb = 0.f;
+    uint32_t cnt = 0;
+    int pc0 = -1, pc1 = -1, pc2 = -1;   // cell where the previous sub-step ended
+    bool overflow = false;
+};
+
+// The form's own per-ray constants.
+struct RayWeights {
+    float w1[6], w2[6];   // shear form: the Q weights of gamma1, gamma2
+    float4 nd;            // Method A: the direction, for n . grad Phi
+};
+
+template <int FORM>
+__device__ __forceinline__ void ray_weights(const TraceArgs& A, long long rid, RayWeights& V)
+{
+    if constexpr (FORM == kFormShear) shear_weights(A.dirh[rid], V.w1, V.w2);
+    if constexpr (FORM == kFormMethodA) V.nd = A.dirh[rid];
+}
+
+// The FP32 walk's slivers, in units of the path: 4 ulp (see walk_piece).
+constexpr float kSliver = 4.76837158203125e-07f;
+
 // One ray over one step. INTERP: RR_NGP or RR_TRILINEAR. R: float
 // (compensated FP32 walk) or double (plain FP64 walk). FORM (FP32 only):
 // kFormKahan (default), kFormPlain (uncompensated FP32 sums within and across
@@ -93,6 +123,17 @@ __device__ __forceinline__ void shift_corners(float2 q[8], const float2 p[4], in
 //               which also holds its staged arguments, and the forms with
 //               more per-segment state (moments, shear, Method A, generic)
 //               measured 1.5-4 % slower with them and keep indices.
+//  kAddrAuto:   kAddrFlat for the sub-steps whose own cells and vertex planes
+//               lie inside the grid without a wrap (counted exactly as the walk
+//               will cross them, so a ray that ends on the box face z = 0 still
+//               qualifies), kAddrIndex out of line for the others. Whole-grid
+//               records of steps the host cannot clear: steps that reach the
+//               observer on the box face, bounded boxes, batches. Grids of
+//               fewer than 2^31 points. (One step of 1024^2 rays through 256
+//               cells down to z = 0: 3.13 ms by vertex planes, 2.55 ms; a batch
+//               of 16 cones 12.30 ms by vertex indices, 9.87 ms. With both
+//               loops inlined the rare one's registers spill into the common
+//               one: 10.5 ms; with one loop that branches per crossing 12.4 ms.)
 //  kAddrFlat:   no wrap: a 32-bit point index B of the mirrored cell's entry
 //               corner and a constant signed stride d_a per axis (the next
 //               vertex plane along the motion), so the 8 corners are B plus
@@ -101,10 +142,10 @@ __device__ __forceinline__ void shift_corners(float2 q[8], const float2 p[4], in
 //               seam and the grid has fewer than 2^31 points: the host checks
 //               the step's footprint box; each sub-step checks its own cell
 //               range first and, outside it, flags kErrRange and reads nothing.
-template <int INTERP, class R, int FORM = kFormKahan, int ADDR = kAddrPlanes, bool REGACC = false>
-__device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, RayAcc* acc = nullptr)
+template <int INTERP, class R, int FORM, int ADDR>
+__device__ __forceinline__ void walk_piece(const TraceArgs& A, Walk<R>& W, const RayWeights& V, int j, bool resume,
+                                           int fB, const int fd[3], PieceState<R>& S)
 {
-    static_assert(!REGACC || (FORM != kFormPlain && sizeof(R) == 4), "register accumulators: FP32 compensated forms");
     using OT = unsigned long long;
     constexpr bool PLANES = ADDR == kAddrPlanes;
     constexpr bool FLAT = ADDR == kAddrFlat;
@@ -116,46 +157,10 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
     // one record per point: 2 float4 of the tidal tensor, 1 gradient float4
     // (Method A) or a float2 scalar pair (generic form)
     using PR = typename std::conditional<MA, float4, typename std::conditional<GEN, float2, Rec>::type>::type;
-    const long long rid = (long long)iy * A.nx + ix;
     const int nn[3] = {A.n0, A.n1, A.n2};
-    RayRange rg;
-    if (!ray_range(A, rid, rg)) return;
-    if (!REGACC || !acc->loaded) {
-        prefetch_l2(A.kacc + rid);
-        prefetch_l2(A.bacc + rid);
-        prefetch_l2(A.nseg + rid);
-        if constexpr (SH) {
-            prefetch_l2(A.g1acc + rid);
-            prefetch_l2(A.g2acc + rid);
-        }
-    }
+    const long long sx = (long long)A.n1 * A.n2, sy = A.n2;
     const R chis = (R)A.chi_s;
     const R ichis = F64 ? (R)(1.0 / A.chi_s) : (R)A.inv_chi_s_f;
-    const long long sx = (long long)A.n1 * A.n2, sy = A.n2;
-    // FP32: sub-steps of at most sub_len, so that the path variable stays small
-    const int nsub = F64 ? 1 : max(1, (int)ceilf(rg.Lf / A.sub_len));
-    const float dsub = rg.Lf / (float)nsub;
-
-    // per-step sums of (kappa, Born kappa): packed Kahan pairs (FP32) or FP64
-    Acc2 s2;
-    Acc2 s2m;   // moments form: the B moments; shear form: (gamma1, gamma2)
-    float w1[6], w2[6];   // shear form: the Q weights of gamma1, gamma2
-    if constexpr (SH) shear_weights(A.dirh[rid], w1, w2);
-    float4 nd;            // Method A: the direction, for n . grad Phi
-    if constexpr (MA) nd = A.dirh[rid];
-    // Method A: n . grad Phi and g at the start and at the end of the interval
-    float qa = 0.f, ga = 0.f, qb = 0.f, gb = 0.f;
-    Acc<R> sk, sb;
-    uint32_t cnt = 0;
-    int iter = 0;
-    bool overflow = false;
-    int pc0 = -1, pc1 = -1, pc2 = -1;   // cell where the previous sub-step ended
-    int pB = -1;                        // FLAT: entry corner where the previous sub-step ended
-    for (int j = 0; j < nsub && !overflow; ++j) {
-    float bh, bl, Lj, D0j;
-    sub_step(rg, j, nsub, dsub, bh, bl, Lj, D0j);
-    Walk<R> W;
-    walk_setup<R>(A, rid, bh, bl, Lj, D0j, rg.hi, rg.lo, W);
     int* c = W.c;
     const int* sgn = W.sgn;
     int* k = W.k;
@@ -178,39 +183,16 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
     const R* cu = W.cu;
     const float* w = W.w;
     const R L = W.L, chiA0 = W.chiA0, D0 = W.D0;
+    // Crossings closer together than the walk resolves are one crossing: a
+    // crossing within eps_rel * L of the step's end, and a segment shorter
+    // than eps_rel * (its end), are rounding slivers at an edge or corner the
+    // ray passes through; they are neither integrated nor counted. FP32: 4 ulp
+    // of the path. FP64: 2^-36, above the error the FP64 start point carries
+    // into a crossing distance (ulp(|p|) / |n_a|) for rays 1e-4 rad off an axis.
+    const R eps_rel = F64 ? (R)1.4551915228366852e-11 : (R)kSliver;
+    const R eps_end = L * eps_rel;
     const int max_iter = W.max_iter;
-    // FLAT: entry corner B, strides d, crossing counts as floats
-    int fB = 0, fd[3] = {0, 0, 0};
-    float kf[3] = {0.f, 0.f, 0.f};
-    if constexpr (FLAT) {
-        bool inside = true;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            // box-local vertex and cell coordinates (the records' box starts
-            // at fo, periodically)
-            const int sa = a == 0 ? A.fs0 : (a == 1 ? A.fs1 : 1);
-            int vl = vlo[a] - A.fo[a];
-            if (vl < 0) vl += nn[a];
-            int cl = c[a] - A.fo[a];
-            if (cl < 0) cl += nn[a];
-            fB += vl * sa;
-            fd[a] = sgn[a] * sa;
-            // crossings this sub-step can make on axis a (2 more than the path
-            // allows, for rounding); cells c .. c + sgn K, vertex planes one further
-            int K = 0;
-            if (T0[a] < L) {
-                const float x = (L - T0[a]) * v[a];
-                if (x < 4194304.f) K = f2i_exact(x) + 2;
-                else inside = false;
-            }
-            const int lo = sgn[a] > 0 ? cl : cl - K, hi = sgn[a] > 0 ? cl + K + 1 : cl + 1;
-            if (lo < 0 || hi > A.fe[a] - 1) inside = false;
-        }
-        if (!inside) {
-            atomicOr(A.err, kErrRange);
-            break;
-        }
-    }
+    float kf[3] = {0.f, 0.f, 0.f};   // FLAT: crossing counts as floats
     auto fetch = [&](long long i) -> PR {
         if constexpr (MA) return load_grad_rec(A.rec, i);
         else if constexpr (GEN) return __ldg(reinterpret_cast<const float2*>(A.rec) + i);
@@ -219,16 +201,11 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
     };
     // (the channel pair the walk integrates) of a record
     auto pair = [&](const PR& r) -> float2 {
-        if constexpr (MA) return radial_pair(nd, r);
+        if constexpr (MA) return radial_pair(V.nd, r);
         else if constexpr (GEN) return r;
         else return make_float2(project(w, r), r.b.z);
     };
-    // a sub-step that resumes inside the previous one's last cell does not
-    // start a new cell segment
-    bool resume;
-    if constexpr (FLAT) resume = j > 0 && fB == pB;
-    else resume = j > 0 && c[0] == pc0 && c[1] == pc1 && c[2] == pc2;
-    iter = 0;
+    int iter = 0;
 
     // Field cache: (projected kappa value, delta) at the 8 mirrored corners
     // (trilinear) or at the cell centre (NGP); the shear form also keeps
@@ -252,24 +229,16 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
             }
             const PR r = fetch(o);
             q2[m] = pair(r);
-            if constexpr (SH) g2[m] = make_float2(project(w1, r), project(w2, r));
+            if constexpr (SH) g2[m] = make_float2(project(V.w1, r), project(V.w2, r));
         }
     } else {
         const PR r = fetch(c[0] * sx + c[1] * sy + c[2]);
         q2[0] = pair(r);
-        if constexpr (SH) g2[0] = make_float2(project(w1, r), project(w2, r));
+        if constexpr (SH) g2[0] = make_float2(project(V.w1, r), project(V.w2, r));
     }
 
     R sig = 0;                       // path from the sub-step start to the segment entry
     R T[3] = {T0[0], T0[1], T0[2]};  // path to the next face crossing per axis
-    // Crossings closer together than the walk resolves are one crossing: a
-    // crossing within eps_rel * L of the step's end, and a segment shorter
-    // than eps_rel * (its end), are rounding slivers at an edge or corner the
-    // ray passes through; they are neither integrated nor counted. FP32: 4 ulp
-    // of the path. FP64: 2^-36, above the error the FP64 start point carries
-    // into a crossing distance (ulp(|p|) / |n_a|) for rays 1e-4 rad off an axis.
-    const R eps_rel = F64 ? (R)1.4551915228366852e-11 : (R)4.76837158203125e-07;
-    const R eps_end = L * eps_rel;
     while (true) {
         // exit plane: the nearest face crossing (lowest axis on ties)
         R tend = T[0];
@@ -349,21 +318,21 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
             // (the exit of the segment that ends the interval: the last one,
             // or, without wrap, the one leaving the box)
             if (j == 0 && iter == 0) {
-                qa = INTERP == RR_TRILINEAR ? trilinear_x(q2, u[0], u[1], u[2]) : q2[0].x;
-                ga = D0 * chiA0 * ichis;
+                S.qa = INTERP == RR_TRILINEAR ? trilinear_x(q2, u[0], u[1], u[2]) : q2[0].x;
+                S.ga = D0 * chiA0 * ichis;
             }
             if (last || (!A.periodic && (ncell < 0 || ncell >= ne))) {
                 if (INTERP == RR_TRILINEAR) {
                     float ue[3];
 #pragma unroll
                     for (int a = 0; a < 3; ++a) ue[a] = fminf(fmaxf(fmaf(t, v[a], u[a]), 0.f), 1.f);
-                    qb = trilinear_x(q2, ue[0], ue[1], ue[2]);
+                    S.qb = trilinear_x(q2, ue[0], ue[1], ue[2]);
                 } else {
-                    qb = q2[0].x;
+                    S.qb = q2[0].x;
                 }
                 float G0, G1, G2;
                 kernel_coeffs(t, sig, chiA0, D0, chis, ichis, G0, G1, G2);
-                gb = fmaf(t, fmaf(t, G2, G1), G0);
+                S.gb = fmaf(t, fmaf(t, G2, G1), G0);
             }
         }
 
@@ -373,11 +342,11 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
                 if (INTERP == RR_TRILINEAR) {
                     float2 e2[4];
                     line_cubic2(q2, bc2(u[0]), bc2(u[1]), bc2(u[2]), bc2(v[0]), bc2(v[1]), bc2(v[2]), e2);
-                    s2.add(dot_kernel(e2, t, chiA, -1.f, 0.f));
-                    s2m.add(dot_kernel(e2, t, chiA * chiA, -2.f * chiA, 1.f));
+                    S.s2.add(dot_kernel(e2, t, chiA, -1.f, 0.f));
+                    S.s2m.add(dot_kernel(e2, t, chiA * chiA, -2.f * chiA, 1.f));
                 } else {
-                    s2.add(segment_ngp(q2[0], t, chiA, -1.f, 0.f));
-                    s2m.add(segment_ngp(q2[0], t, chiA * chiA, -2.f * chiA, 1.f));
+                    S.s2.add(segment_ngp(q2[0], t, chiA, -1.f, 0.f));
+                    S.s2m.add(segment_ngp(q2[0], t, chiA * chiA, -2.f * chiA, 1.f));
                 }
             } else if constexpr (GEN) {
                 // each channel's kernel about the entry point: K(chi_A - s) =
@@ -390,17 +359,17 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
                 if (INTERP == RR_TRILINEAR) {
                     float2 e2[4];
                     line_cubic2(q2, bc2(u[0]), bc2(u[1]), bc2(u[2]), bc2(v[0]), bc2(v[1]), bc2(v[2]), e2);
-                    s2.add(dot_kernel_pair(e2, t, G0, G1, G2));
+                    S.s2.add(dot_kernel_pair(e2, t, G0, G1, G2));
                 } else {
                     const float2 tt = bc2(t);
                     const float2 J1 = __fmul2_rn(tt, __ffma2_rn(tt, __ffma2_rn(tt, __fmul2_rn(G2, bc2(1.f / 3.f)),
                                                                               __fmul2_rn(G1, bc2(0.5f))), G0));
-                    s2.add(__fmul2_rn(q2[0], J1));
+                    S.s2.add(__fmul2_rn(q2[0], J1));
                 }
             } else if constexpr (MA) {
                 float G0, G1, G2;
                 kernel_coeffs(t, sig, chiA0, D0, chis, ichis, G0, G1, G2);
-                s2.add(INTERP == RR_TRILINEAR
+                S.s2.add(INTERP == RR_TRILINEAR
                            ? segment_trilinear_a(q2, u[0], u[1], u[2], v[0], v[1], v[2], t, G0, G1, G2)
                            : segment_ngp_a(q2[0], t, G0, G1, G2));
             } else if constexpr (!F64) {
@@ -409,10 +378,10 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
                 const float2 x = INTERP == RR_TRILINEAR
                                      ? segment_trilinear(q2, u[0], u[1], u[2], v[0], v[1], v[2], t, G0, G1, G2)
                                      : segment_ngp(q2[0], t, G0, G1, G2);
-                if constexpr (FORM == kFormPlain) s2.s = __fadd2_rn(s2.s, x);
-                else s2.add(x);
+                if constexpr (FORM == kFormPlain) S.s2.s = __fadd2_rn(S.s2.s, x);
+                else S.s2.add(x);
                 if constexpr (SH)
-                    s2m.add(INTERP == RR_TRILINEAR
+                    S.s2m.add(INTERP == RR_TRILINEAR
                                 ? segment_trilinear(g2, u[0], u[1], u[2], v[0], v[1], v[2], t, G0, G1, G2)
                                 : segment_ngp(g2[0], t, G0, G1, G2));
             } else {
@@ -443,15 +412,15 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
                         xk = __fma_rn((double)e2[n].x, J[n], xk);
                         xb = __fma_rn((double)e2[n].y, J[n], xb);
                     }
-                    sk.add((R)xk);
-                    sb.add((R)xb);
+                    S.sk.add((R)xk);
+                    S.sb.add((R)xb);
                 } else {
-                    sk.add((R)__dmul_rn((double)q2[0].x, J[0]));
-                    sb.add((R)__dmul_rn((double)q2[0].y, J[0]));
+                    S.sk.add((R)__dmul_rn((double)q2[0].x, J[0]));
+                    S.sb.add((R)__dmul_rn((double)q2[0].y, J[0]));
                 }
             }
             if (resume) resume = false;
-            else ++cnt;
+            else ++S.cnt;
         }
         sig = tend;
         if (last) break;
@@ -491,32 +460,146 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
             shift_corners(q2, p2, e);
             if constexpr (SH) {
 #pragma unroll
-                for (int r = 0; r < 4; ++r) p2[r] = make_float2(project(w1, nr[r]), project(w2, nr[r]));
+                for (int r = 0; r < 4; ++r) p2[r] = make_float2(project(V.w1, nr[r]), project(V.w2, nr[r]));
                 shift_corners<true>(g2, p2, e);
             }
         } else {
             q2[0] = pair(nr[0]);
-            if constexpr (SH) g2[0] = make_float2(project(w1, nr[0]), project(w2, nr[0]));
+            if constexpr (SH) g2[0] = make_float2(project(V.w1, nr[0]), project(V.w2, nr[0]));
         }
         if (++iter > max_iter) {
-            overflow = true;
+            S.overflow = true;
             break;
         }
     }
-    pc0 = c[0]; pc1 = c[1]; pc2 = c[2];
-    pB = fB;
+    if constexpr (FLAT) {
+        // the cell the walk ended in (a box-local walk may have passed the seam, once)
+        S.pc0 = wrap_once(c[0] + sgn[0] * f2i_exact(kf[0]), nn[0]);
+        S.pc1 = wrap_once(c[1] + sgn[1] * f2i_exact(kf[1]), nn[1]);
+        S.pc2 = wrap_once(c[2] + sgn[2] * f2i_exact(kf[2]), nn[2]);
+    } else {
+        S.pc0 = c[0]; S.pc1 = c[1]; S.pc2 = c[2];
+    }
+}
+
+// A sub-step by wrapped vertex indices, out of line: kAddrAuto's rare path. It
+// sets the walk up again, so that nothing of the caller's loop outlives the
+// call in registers but what PieceState holds.
+template <int FORM>
+__device__ __noinline__ void index_piece(const TraceArgs& A, long long rid, float bh, float bl, float Lj, float D0j,
+                                         int j, bool resume, PieceState<float>& S)
+{
+    RayWeights V;
+    ray_weights<FORM>(A, rid, V);
+    Walk<float> W;
+    walk_setup<float>(A, rid, bh, bl, Lj, D0j, 0.0, 0.0, W);
+    const int fd[3] = {0, 0, 0};
+    walk_piece<RR_TRILINEAR, float, FORM, kAddrIndex>(A, W, V, j, resume, 0, fd, S);
+}
+
+template <int INTERP, class R, int FORM = kFormKahan, int ADDR = kAddrPlanes, bool REGACC = false>
+__device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, RayAcc* acc = nullptr)
+{
+    static_assert(!REGACC || (FORM != kFormPlain && sizeof(R) == 4), "register accumulators: FP32 compensated forms");
+    constexpr bool AUTO = ADDR == kAddrAuto;
+    constexpr bool FLAT = ADDR == kAddrFlat || AUTO;
+    static_assert(!FLAT || (INTERP == RR_TRILINEAR && sizeof(R) == 4), "flat addressing: FP32 trilinear walk");
+    constexpr bool F64 = sizeof(R) == 8;
+    constexpr bool SH = !F64 && FORM == kFormShear;
+    constexpr bool MA = !F64 && FORM == kFormMethodA;
+    const long long rid = (long long)iy * A.nx + ix;
+    const int nn[3] = {A.n0, A.n1, A.n2};
+    RayRange rg;
+    if (!ray_range(A, rid, rg)) return;
+    if (!REGACC || !acc->loaded) {
+        prefetch_l2(A.kacc + rid);
+        prefetch_l2(A.bacc + rid);
+        prefetch_l2(A.nseg + rid);
+        if constexpr (SH) {
+            prefetch_l2(A.g1acc + rid);
+            prefetch_l2(A.g2acc + rid);
+        }
+    }
+    // FP32: sub-steps of at most sub_len, so that the path variable stays small
+    const int nsub = F64 ? 1 : max(1, (int)ceilf(rg.Lf / A.sub_len));
+    const float dsub = rg.Lf / (float)nsub;
+
+    RayWeights V;
+    ray_weights<FORM>(A, rid, V);
+    PieceState<R> S;
+    for (int j = 0; j < nsub && !S.overflow; ++j) {
+    float bh, bl, Lj, D0j;
+    sub_step(rg, j, nsub, dsub, bh, bl, Lj, D0j);
+    Walk<R> W;
+    walk_setup<R>(A, rid, bh, bl, Lj, D0j, rg.hi, rg.lo, W);
+    // FLAT: entry corner B, strides d
+    int fB = 0, fd[3] = {0, 0, 0};
+    bool inside = true;
+    if constexpr (FLAT) {
+        const int* c = W.c;
+        const int* sgn = W.sgn;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            // box-local vertex and cell coordinates (the records' box starts
+            // at fo, periodically)
+            const int sa = a == 0 ? A.fs0 : (a == 1 ? A.fs1 : 1);
+            int vl = W.vlo[a] - A.fo[a];
+            if (vl < 0) vl += nn[a];
+            int cl = c[a] - A.fo[a];
+            if (cl < 0) cl += nn[a];
+            fB += vl * sa;
+            fd[a] = sgn[a] * sa;
+            // crossings this sub-step can make on axis a (2 more than the path
+            // allows, for rounding); cells c .. c + sgn K, vertex planes one further
+            int K = 0;
+            if (W.T0[a] < W.L) {
+                const float x = (W.L - W.T0[a]) * W.v[a];
+                if (x < 4194304.f) K = f2i_exact(x) + 2;
+                else inside = false;
+                if constexpr (AUTO) {
+                    // the walk crosses face k (k = 0, 1, ...) on this axis while
+                    // T_k = T0 + k td < L - eps_end, and T_k never decreases with
+                    // k: drop the margin that the walk's own test rules out
+                    const float lim = W.L - W.L * kSliver;
+#pragma unroll
+                    for (int r = 0; r < 3; ++r)
+                        if (K > 0 && !(fmaf((float)(K - 1), W.td[a], W.T0[a]) < lim)) --K;
+                }
+            }
+            const int lo = sgn[a] > 0 ? cl : cl - K, hi = sgn[a] > 0 ? cl + K + 1 : cl + 1;
+            if (lo < 0 || hi > A.fe[a] - 1) inside = false;
+        }
+        if (!AUTO && !inside) {
+            atomicOr(A.err, kErrRange);
+            break;
+        }
+    }
+    // a sub-step that resumes inside the previous one's last cell does not
+    // start a new cell segment
+    const bool resume = j > 0 && W.c[0] == S.pc0 && W.c[1] == S.pc1 && W.c[2] == S.pc2;
+    if constexpr (AUTO) {
+        if (inside) {
+            walk_piece<INTERP, R, FORM, kAddrFlat>(A, W, V, j, resume, fB, fd, S);
+        } else {
+            PieceState<R> Q = S;
+            index_piece<FORM>(A, rid, bh, bl, Lj, D0j, j, resume, Q);
+            S = Q;
+        }
+    } else {
+        walk_piece<INTERP, R, FORM, ADDR>(A, W, V, j, resume, fB, fd, S);
+    }
     }
 
     if constexpr (MA) {
-        s2.add(make_float2(-ga * qa, 0.f));
-        s2.add(make_float2(gb * qb, 0.f));
+        S.s2.add(make_float2(-S.ga * S.qa, 0.f));
+        S.s2.add(make_float2(S.gb * S.qb, 0.f));
     }
     if constexpr (!F64) {
-        sk.s = s2.s.x; sk.c = s2.c.x;
-        sb.s = s2.s.y; sb.c = s2.c.y;
+        S.sk.s = S.s2.s.x; S.sk.c = S.s2.c.x;
+        S.sb.s = S.s2.s.y; S.sb.c = S.s2.c.y;
     }
-    if (overflow) atomicOr(A.err, kErrStepLimit);
-    if (!sk.finite() || !sb.finite()) atomicOr(A.err, kErrNonFinite);
+    if (S.overflow) atomicOr(A.err, kErrStepLimit);
+    if (!S.sk.finite() || !S.sb.finite()) atomicOr(A.err, kErrNonFinite);
     if constexpr (REGACC) {
         // the first step of the launch: the ray's state from memory
         if (!acc->loaded) {
@@ -536,48 +619,48 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
     }
     if constexpr (SH) {
         float gh, gl;
-        if (!s2m.finite()) atomicOr(A.err, kErrNonFinite);
-        two_sum(s2m.s.x, -s2m.c.x, gh, gl);
+        if (!S.s2m.finite()) atomicOr(A.err, kErrNonFinite);
+        two_sum(S.s2m.s.x, -S.s2m.c.x, gh, gl);
         if constexpr (REGACC) acc->x1 = ff_mul_add(acc->x1, gh, gl, A.sch, A.scl);
         else A.g1acc[rid] = ff_mul_add(A.g1acc[rid], gh, gl, A.sch, A.scl);
-        two_sum(s2m.s.y, -s2m.c.y, gh, gl);
+        two_sum(S.s2m.s.y, -S.s2m.c.y, gh, gl);
         if constexpr (REGACC) acc->x2 = ff_mul_add(acc->x2, gh, gl, A.sch, A.scl);
         else A.g2acc[rid] = ff_mul_add(A.g2acc[rid], gh, gl, A.sch, A.scl);
     }
     if constexpr (FORM == kFormMoments) {
         float mh, ml;
-        if (!s2m.finite()) atomicOr(A.err, kErrNonFinite);
-        two_sum(s2m.s.x, -s2m.c.x, mh, ml);
+        if (!S.s2m.finite()) atomicOr(A.err, kErrNonFinite);
+        two_sum(S.s2m.s.x, -S.s2m.c.x, mh, ml);
         if constexpr (REGACC) acc->x1 = ff_mul_add(acc->x1, mh, ml, A.sch, A.scl);
         else A.kmom[rid] = ff_mul_add(A.kmom[rid], mh, ml, A.sch, A.scl);
-        two_sum(s2m.s.y, -s2m.c.y, mh, ml);
+        two_sum(S.s2m.s.y, -S.s2m.c.y, mh, ml);
         if constexpr (REGACC) acc->x2 = ff_mul_add(acc->x2, mh, ml, A.bsh, A.bsl);
         else A.bmom[rid] = ff_mul_add(A.bmom[rid], mh, ml, A.bsh, A.bsl);
     }
     if constexpr (FORM == kFormPlain) {
         // plain FP32 across steps too: the high word only
-        A.kacc[rid] = make_float2(fmaf(sk.s, A.sch, A.kacc[rid].x), 0.f);
-        A.bacc[rid] = make_float2(fmaf(sb.s, A.bsh, A.bacc[rid].x), 0.f);
-        A.nseg[rid] += cnt;
+        A.kacc[rid] = make_float2(fmaf(S.sk.s, A.sch, A.kacc[rid].x), 0.f);
+        A.bacc[rid] = make_float2(fmaf(S.sb.s, A.bsh, A.bacc[rid].x), 0.f);
+        A.nseg[rid] += S.cnt;
         return;
     }
     float kh, kl, bh, bl;
-    sk.pair(kh, kl);
-    sb.pair(bh, bl);
+    S.sk.pair(kh, kl);
+    S.sb.pair(bh, bl);
     if constexpr (REGACC) {
         acc->k = ff_mul_add(acc->k, kh, kl, A.sch, A.scl);
         acc->b = ff_mul_add(acc->b, bh, bl, A.bsh, A.bsl);
-        acc->n += cnt;
+        acc->n += S.cnt;
         return;
     }
     A.kacc[rid] = ff_mul_add(A.kacc[rid], kh, kl, A.sch, A.scl);
     A.bacc[rid] = ff_mul_add(A.bacc[rid], bh, bl, A.bsh, A.bsl);
-    A.nseg[rid] += cnt;
+    A.nseg[rid] += S.cnt;
 }
 
 
 template <int INTERP, class R, int FORM = kFormKahan, int ADDR = (FORM == kFormKahan ? kAddrPlanes : kAddrIndex)>
-__global__ void __launch_bounds__(NT_MAX, 2) trace_kernel(const TraceArgs A, const TileCfg t)
+__global__ void __launch_bounds__(NT_MAX, 2) trace_kernel(const __grid_constant__ TraceArgs A, const TileCfg t)
 {
     prefetch_ahead(A, t);
     int ix, iy;
@@ -636,7 +719,7 @@ __global__ void __launch_bounds__(NT_MAX, 2)
 // block takes `chunk` consecutive tiles from a global counter (monotonic, no
 // waiting), finds the bundle by binary search in the tile offsets, stages that
 // bundle's arguments in shared memory and traces the tile.
-template <int INTERP, class R>
+template <int INTERP, class R, int ADDR>
 __global__ void __launch_bounds__(NT_MAX, 2) trace_batch_kernel(const BatchArgs B)
 {
     __shared__ TraceArgs sA;
@@ -673,7 +756,7 @@ __global__ void __launch_bounds__(NT_MAX, 2) trace_batch_kernel(const BatchArgs 
             const int ntx = B.tiles_x[cone];
             int ix, iy;
             tile_ray(B.tile, local % ntx, local / ntx, ix, iy);
-            if (ix < sA.nx && iy < sA.ny) trace_ray<INTERP, R, kFormKahan, kAddrIndex>(sA, ix, iy);
+            if (ix < sA.nx && iy < sA.ny) trace_ray<INTERP, R, kFormKahan, ADDR>(sA, ix, iy);
             __syncthreads();
         }
     }
@@ -698,6 +781,12 @@ namespace {
 template <int INTERP, class R, int FORM>
 cudaError_t launch_one(const TraceArgs& a, const dim3& grid, int nt, cudaStream_t s, const TileCfg& t)
 {
+    if constexpr (INTERP == RR_TRILINEAR && sizeof(R) == 4) {
+        if (a.fe[0] > 0) {   // fewer than 2^31 points
+            trace_kernel<INTERP, R, FORM, kAddrAuto><<<grid, nt, 0, s>>>(a, t);
+            return cudaGetLastError();
+        }
+    }
     trace_kernel<INTERP, R, FORM><<<grid, nt, 0, s>>>(a, t);
     return cudaGetLastError();
 }
@@ -782,21 +871,28 @@ cudaError_t launch_trace(const TraceArgs& a, int interp, bool fp64_dda, cudaStre
     return launch_trace(a, interp, fp64_dda, s, TileCfg{});
 }
 
-cudaError_t launch_trace_batch(const BatchArgs& b, int interp, bool fp64_dda, int blocks, cudaStream_t s)
+namespace {
+
+using BatchKernel = void (*)(const BatchArgs);
+
+// small: every bundle's grid has fewer than 2^31 points
+BatchKernel batch_kernel(int interp, bool fp64_dda, bool small)
+{
+    if (interp == RR_TRILINEAR) {
+        if (fp64_dda) return trace_batch_kernel<RR_TRILINEAR, double, kAddrIndex>;
+        return small ? trace_batch_kernel<RR_TRILINEAR, float, kAddrAuto>
+                     : trace_batch_kernel<RR_TRILINEAR, float, kAddrIndex>;
+    }
+    return fp64_dda ? trace_batch_kernel<RR_NGP, double, kAddrIndex> : trace_batch_kernel<RR_NGP, float, kAddrIndex>;
+}
+
+}  // namespace
+
+cudaError_t launch_trace_batch(const BatchArgs& b, int interp, bool fp64_dda, int blocks, cudaStream_t s, bool small)
 {
     if (!tile_ok(b.tile) || b.chunk < 1 || blocks < 1) return cudaErrorInvalidValue;
     const int nt = 32 * b.tile.bwx * b.tile.bwy;
-    if (interp == RR_TRILINEAR) {
-        if (fp64_dda)
-            trace_batch_kernel<RR_TRILINEAR, double><<<blocks, nt, 0, s>>>(b);
-        else
-            trace_batch_kernel<RR_TRILINEAR, float><<<blocks, nt, 0, s>>>(b);
-    } else {
-        if (fp64_dda)
-            trace_batch_kernel<RR_NGP, double><<<blocks, nt, 0, s>>>(b);
-        else
-            trace_batch_kernel<RR_NGP, float><<<blocks, nt, 0, s>>>(b);
-    }
+    batch_kernel(interp, fp64_dda, small)<<<blocks, nt, 0, s>>>(b);
     return cudaGetLastError();
 }
 
@@ -804,14 +900,8 @@ int batch_blocks_per_sm(int interp, bool fp64_dda, const TileCfg& t)
 {
     const int nt = 32 * t.bwx * t.bwy;
     int n = 0;
-    cudaError_t e;
-    if (interp == RR_TRILINEAR)
-        e = fp64_dda ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, trace_batch_kernel<RR_TRILINEAR, double>, nt, 0)
-                     : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, trace_batch_kernel<RR_TRILINEAR, float>, nt, 0);
-    else
-        e = fp64_dda ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, trace_batch_kernel<RR_NGP, double>, nt, 0)
-                     : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, trace_batch_kernel<RR_NGP, float>, nt, 0);
+    const cudaError_t e =
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel(interp, fp64_dda, true), nt, 0);
     return (e == cudaSuccess && n > 0) ? n : 1;
 }
 }  // namespace rr
-
