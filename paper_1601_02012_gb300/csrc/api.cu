@@ -105,7 +105,11 @@ TraceArgs make_trace_args(const rr_bundle_desc& b, const RayState& st, const rr_
     split_ff(a.inv_h, a.ihh, a.ihl);
     a.nx = b.nx; a.ny = b.ny;
     a.obs0 = obs[0]; a.obs1 = obs[1]; a.obs2 = obs[2];
-    for (int i = 0; i < 3; ++i) split_ff(obs[i], a.oh[i], a.ol[i]);
+    for (int i = 0; i < 3; ++i) {
+        split_ff(obs[i], a.oh[i], a.ol[i]);
+        a.face0[i] = (float)-obs[i];
+        a.face1[i] = (float)(grid->n[i] * a.h - obs[i]);
+    }
     a.chi_s = b.chi_s;
     a.chi_a = chi_a;
     a.chi_b = chi_b;

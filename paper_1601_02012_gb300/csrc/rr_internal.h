@@ -63,6 +63,7 @@ struct TraceArgs {
     int nx, ny;                 // rays
     double obs0, obs1, obs2;
     float oh[3], ol[3];         // observer as float-float
+    float face0[3], face1[3];   // the box faces relative to the observer, rounded to FP32 (bounded walks)
     double chi_s, chi_a, chi_b;
     float cah, cal;             // chi_a as float-float
     float Lf;                   // chi_a - chi_b rounded to FP32
