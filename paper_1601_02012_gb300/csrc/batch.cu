@@ -22,6 +22,7 @@ struct rr_batch {
     std::vector<rr_ctx*> cones;
     int interp = RR_TRILINEAR;
     bool fp64 = false;
+    bool periodic = true;        // every bundle is
     TileCfg tile;
     int chunk = 1;
     int blocks_per_sm = 0;       // 0: as many as fit (occupancy)
@@ -67,7 +68,7 @@ void build_tiles(rr_batch* b)
 
 int grid_blocks(const rr_batch* b)
 {
-    const int per_sm = b->blocks_per_sm > 0 ? b->blocks_per_sm : batch_blocks_per_sm(b->interp, b->fp64, b->tile);
+    const int per_sm = b->blocks_per_sm > 0 ? b->blocks_per_sm : batch_blocks_per_sm(b->interp, b->fp64, b->periodic, b->tile);
     long long blocks = (long long)per_sm * b->sms;
     if (blocks > b->total_tiles) blocks = b->total_tiles;
     return blocks < 1 ? 1 : (int)blocks;
@@ -91,6 +92,7 @@ rr_status rr_batch_create(int32_t n, const rr_bundle_desc* bundles, rr_batch** o
     if (!b) return RR_ERR_OOM;
     b->interp = bundles[0].interp;
     b->fp64 = (bundles[0].flags & RR_FP64_DDA) != 0;
+    for (int i = 0; i < n; ++i) b->periodic = b->periodic && (bundles[i].flags & RR_PERIODIC);
     b->cones.assign((size_t)n, nullptr);
     b->staged.assign((size_t)n, false);
     for (int i = 0; i < n; ++i) {
@@ -210,7 +212,7 @@ rr_status rr_batch_trace(rr_batch* b, void* stream)
     a.tile = b->tile;
     bool small = true;
     for (int i = 0; i < n; ++i) small = small && b->h_args[i].fe[0] > 0;
-    return status_of_cuda(launch_trace_batch(a, b->interp, b->fp64, grid_blocks(b), s, small));
+    return status_of_cuda(launch_trace_batch(a, b->interp, b->fp64, grid_blocks(b), s, small, b->periodic));
 }
 
 rr_status rr_batch_finalize(rr_batch* b, double* const* kappa, double* const* kappa_born, void* stream)

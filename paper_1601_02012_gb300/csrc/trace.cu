@@ -237,6 +237,9 @@ __device__ __forceinline__ void walk_piece(const TraceArgs& A, Walk<R>& W, const
         if constexpr (SH) g2[0] = make_float2(project(V.w1, r), project(V.w2, r));
     }
 
+    // (a resumed first segment is not a new one; it is integrated below unless
+    // the walk starts on its exit face)
+    if (resume && T0[0] > (R)0 && T0[1] > (R)0 && T0[2] > (R)0) --S.cnt;
     R sig = 0;                       // path from the sub-step start to the segment entry
     R T[3] = {T0[0], T0[1], T0[2]};  // path to the next face crossing per axis
     while (true) {
@@ -419,14 +422,12 @@ __device__ __forceinline__ void walk_piece(const TraceArgs& A, Walk<R>& W, const
                     S.sb.add((R)__dmul_rn((double)q2[0].y, J[0]));
                 }
             }
-            if (resume) resume = false;
-            else ++S.cnt;
+            ++S.cnt;
         }
         sig = tend;
         if (last) break;
 
         // cross the exit face e
-        resume = false;
         if constexpr (FLAT) {
             fB += fde;
 #pragma unroll
@@ -497,7 +498,8 @@ __device__ __noinline__ void index_piece(const TraceArgs& A, long long rid, floa
     walk_piece<RR_TRILINEAR, float, FORM, kAddrIndex>(A, W, V, j, resume, 0, fd, S);
 }
 
-template <int INTERP, class R, int FORM = kFormKahan, int ADDR = kAddrPlanes, bool REGACC = false>
+// PER: periodic bundles only.
+template <int INTERP, class R, int FORM, int ADDR, bool PER, bool REGACC = false>
 __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, RayAcc* acc = nullptr)
 {
     static_assert(!REGACC || (FORM != kFormPlain && sizeof(R) == 4), "register accumulators: FP32 compensated forms");
@@ -510,7 +512,7 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
     const long long rid = (long long)iy * A.nx + ix;
     const int nn[3] = {A.n0, A.n1, A.n2};
     RayRange rg;
-    if (!ray_range(A, rid, rg)) return;
+    if (!ray_range<PER>(A, rid, rg)) return;
     if (!REGACC || !acc->loaded) {
         prefetch_l2(A.kacc + rid);
         prefetch_l2(A.bacc + rid);
@@ -581,7 +583,16 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
         if (inside) {
             walk_piece<INTERP, R, FORM, kAddrFlat>(A, W, V, j, resume, fB, fd, S);
         } else {
-            PieceState<R> Q = S;
+            // (only what the form carries: each further word costs the common
+            // path registers around the call)
+            PieceState<R> Q;
+            Q.s2 = S.s2;
+            Q.cnt = S.cnt;
+            if constexpr (SH || FORM == kFormMoments) Q.s2m = S.s2m;
+            if constexpr (MA) {
+                Q.qa = S.qa; Q.ga = S.ga;
+                Q.qb = S.qb; Q.gb = S.gb;
+            }
             index_piece<FORM>(A, rid, bh, bl, Lj, D0j, j, resume, Q);
             S = Q;
         }
@@ -659,13 +670,13 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
 }
 
 
-template <int INTERP, class R, int FORM = kFormKahan, int ADDR = (FORM == kFormKahan ? kAddrPlanes : kAddrIndex)>
+template <int INTERP, class R, int FORM, int ADDR, bool PER>
 __global__ void __launch_bounds__(NT_MAX, 2) trace_kernel(const __grid_constant__ TraceArgs A, const TileCfg t)
 {
     prefetch_ahead(A, t);
     int ix, iy;
     tile_ray(t, blockIdx.x, blockIdx.y, ix, iy);
-    if (ix < A.nx && iy < A.ny) trace_ray<INTERP, R, FORM, ADDR>(A, ix, iy);
+    if (ix < A.nx && iy < A.ny) trace_ray<INTERP, R, FORM, ADDR, PER>(A, ix, iy);
 }
 
 // Consecutive steps of one bundle in one launch (the default FP32 form): each
@@ -675,7 +686,7 @@ __global__ void __launch_bounds__(NT_MAX, 2) trace_kernel(const __grid_constant_
 // the result equals one trace_kernel launch per step bit for bit; what goes
 // is the per-launch and per-step traffic of the ray state (directions,
 // accumulators) and all launches but one.
-template <int INTERP, int ADDR, int FORM>
+template <int INTERP, int ADDR, int FORM, bool PER>
 __global__ void __launch_bounds__(NT_MAX, 2)
     trace_steps_kernel(const TraceArgs A, const __grid_constant__ StepBlock S, const TileCfg t)
 {
@@ -697,7 +708,7 @@ __global__ void __launch_bounds__(NT_MAX, 2)
         As.fo[0] = st.fo[0]; As.fo[1] = st.fo[1]; As.fo[2] = st.fo[2];
         As.fe[0] = st.fe[0]; As.fe[1] = st.fe[1]; As.fe[2] = st.fe[2];
         As.fs0 = st.fs0; As.fs1 = st.fs1;
-        trace_ray<INTERP, float, FORM, ADDR, true>(As, ix, iy, &acc);
+        trace_ray<INTERP, float, FORM, ADDR, PER, true>(As, ix, iy, &acc);
     }
     if (acc.loaded) {
         const long long rid = (long long)iy * A.nx + ix;
@@ -719,7 +730,7 @@ __global__ void __launch_bounds__(NT_MAX, 2)
 // block takes `chunk` consecutive tiles from a global counter (monotonic, no
 // waiting), finds the bundle by binary search in the tile offsets, stages that
 // bundle's arguments in shared memory and traces the tile.
-template <int INTERP, class R, int ADDR>
+template <int INTERP, class R, int ADDR, bool PER>
 __global__ void __launch_bounds__(NT_MAX, 2) trace_batch_kernel(const BatchArgs B)
 {
     __shared__ TraceArgs sA;
@@ -756,7 +767,7 @@ __global__ void __launch_bounds__(NT_MAX, 2) trace_batch_kernel(const BatchArgs 
             const int ntx = B.tiles_x[cone];
             int ix, iy;
             tile_ray(B.tile, local % ntx, local / ntx, ix, iy);
-            if (ix < sA.nx && iy < sA.ny) trace_ray<INTERP, R, kFormKahan, ADDR>(sA, ix, iy);
+            if (ix < sA.nx && iy < sA.ny) trace_ray<INTERP, R, kFormKahan, ADDR, PER>(sA, ix, iy);
             __syncthreads();
         }
     }
@@ -778,17 +789,22 @@ bool tile_ok(const TileCfg& t)
 
 namespace {
 
+template <int INTERP, class R, int FORM, int ADDR>
+cudaError_t launch_addr(const TraceArgs& a, const dim3& grid, int nt, cudaStream_t s, const TileCfg& t)
+{
+    if (a.periodic) trace_kernel<INTERP, R, FORM, ADDR, true><<<grid, nt, 0, s>>>(a, t);
+    else trace_kernel<INTERP, R, FORM, ADDR, false><<<grid, nt, 0, s>>>(a, t);
+    return cudaGetLastError();
+}
+
 template <int INTERP, class R, int FORM>
 cudaError_t launch_one(const TraceArgs& a, const dim3& grid, int nt, cudaStream_t s, const TileCfg& t)
 {
     if constexpr (INTERP == RR_TRILINEAR && sizeof(R) == 4) {
-        if (a.fe[0] > 0) {   // fewer than 2^31 points
-            trace_kernel<INTERP, R, FORM, kAddrAuto><<<grid, nt, 0, s>>>(a, t);
-            return cudaGetLastError();
-        }
+        // fewer than 2^31 points
+        if (a.fe[0] > 0) return launch_addr<INTERP, R, FORM, kAddrAuto>(a, grid, nt, s, t);
     }
-    trace_kernel<INTERP, R, FORM><<<grid, nt, 0, s>>>(a, t);
-    return cudaGetLastError();
+    return launch_addr<INTERP, R, FORM, FORM == kFormKahan ? kAddrPlanes : kAddrIndex>(a, grid, nt, s, t);
 }
 
 template <int FORM>
@@ -808,12 +824,12 @@ cudaError_t launch_trace(const TraceArgs& a, int interp, bool fp64_dda, cudaStre
     const int nt = 32 * t.bwx * t.bwy;
     if (flat && !fp64_dda && interp == RR_TRILINEAR && a.periodic) {
         switch (form) {
-        case kFormPlain: trace_kernel<RR_TRILINEAR, float, kFormPlain, kAddrFlat><<<grid, nt, 0, s>>>(a, t); break;
-        case kFormMoments: trace_kernel<RR_TRILINEAR, float, kFormMoments, kAddrFlat><<<grid, nt, 0, s>>>(a, t); break;
-        case kFormGeneric: trace_kernel<RR_TRILINEAR, float, kFormGeneric, kAddrFlat><<<grid, nt, 0, s>>>(a, t); break;
-        case kFormMethodA: trace_kernel<RR_TRILINEAR, float, kFormMethodA, kAddrFlat><<<grid, nt, 0, s>>>(a, t); break;
-        case kFormShear: trace_kernel<RR_TRILINEAR, float, kFormShear, kAddrFlat><<<grid, nt, 0, s>>>(a, t); break;
-        default: trace_kernel<RR_TRILINEAR, float, kFormKahan, kAddrFlat><<<grid, nt, 0, s>>>(a, t); break;
+        case kFormPlain: trace_kernel<RR_TRILINEAR, float, kFormPlain, kAddrFlat, true><<<grid, nt, 0, s>>>(a, t); break;
+        case kFormMoments: trace_kernel<RR_TRILINEAR, float, kFormMoments, kAddrFlat, true><<<grid, nt, 0, s>>>(a, t); break;
+        case kFormGeneric: trace_kernel<RR_TRILINEAR, float, kFormGeneric, kAddrFlat, true><<<grid, nt, 0, s>>>(a, t); break;
+        case kFormMethodA: trace_kernel<RR_TRILINEAR, float, kFormMethodA, kAddrFlat, true><<<grid, nt, 0, s>>>(a, t); break;
+        case kFormShear: trace_kernel<RR_TRILINEAR, float, kFormShear, kAddrFlat, true><<<grid, nt, 0, s>>>(a, t); break;
+        default: trace_kernel<RR_TRILINEAR, float, kFormKahan, kAddrFlat, true><<<grid, nt, 0, s>>>(a, t); break;
         }
         return cudaGetLastError();
     }
@@ -833,19 +849,19 @@ cudaError_t launch_trace(const TraceArgs& a, int interp, bool fp64_dda, cudaStre
 }
 
 template <int FORM>
-static void launch_steps_form(const TraceArgs& a, const StepBlock& b, int interp, bool flat, dim3 grid, int nt,
+static cudaError_t launch_steps_form(const TraceArgs& a, const StepBlock& b, int interp, bool flat, dim3 grid, int nt,
                               const TileCfg& t, cudaStream_t s)
 {
-    // the addressing of each form's single-step kernel: flat for trilinear
-    // steps clear of the seam (or box-local records); otherwise vertex-plane
-    // offsets for the default form and vertex indices for the others
-    constexpr int ADDR = FORM == kFormKahan ? kAddrPlanes : kAddrIndex;
+    // trilinear: steps that all take the flat addressing (periodic); NGP: any
     if (interp == RR_TRILINEAR) {
-        if (flat && a.periodic) trace_steps_kernel<RR_TRILINEAR, kAddrFlat, FORM><<<grid, nt, 0, s>>>(a, b, t);
-        else trace_steps_kernel<RR_TRILINEAR, ADDR, FORM><<<grid, nt, 0, s>>>(a, b, t);
+        if (!flat || !a.periodic) return cudaErrorInvalidValue;
+        trace_steps_kernel<RR_TRILINEAR, kAddrFlat, FORM, true><<<grid, nt, 0, s>>>(a, b, t);
     } else {
-        trace_steps_kernel<RR_NGP, ADDR, FORM><<<grid, nt, 0, s>>>(a, b, t);
+        constexpr int ADDR = FORM == kFormKahan ? kAddrPlanes : kAddrIndex;
+        if (a.periodic) trace_steps_kernel<RR_NGP, ADDR, FORM, true><<<grid, nt, 0, s>>>(a, b, t);
+        else trace_steps_kernel<RR_NGP, ADDR, FORM, false><<<grid, nt, 0, s>>>(a, b, t);
     }
+    return cudaGetLastError();
 }
 
 cudaError_t launch_trace_steps(const TraceArgs& a, const StepBlock& b, int interp, bool flat, cudaStream_t s,
@@ -856,14 +872,13 @@ cudaError_t launch_trace_steps(const TraceArgs& a, const StepBlock& b, int inter
     const dim3 grid = tile_grid(t, a.nx, a.ny);
     const int nt = 32 * t.bwx * t.bwy;
     switch (form) {
-    case kFormKahan: launch_steps_form<kFormKahan>(a, b, interp, flat, grid, nt, t, s); break;
-    case kFormShear: launch_steps_form<kFormShear>(a, b, interp, flat, grid, nt, t, s); break;
-    case kFormMoments: launch_steps_form<kFormMoments>(a, b, interp, flat, grid, nt, t, s); break;
-    case kFormMethodA: launch_steps_form<kFormMethodA>(a, b, interp, flat, grid, nt, t, s); break;
-    case kFormGeneric: launch_steps_form<kFormGeneric>(a, b, interp, flat, grid, nt, t, s); break;
+    case kFormKahan: return launch_steps_form<kFormKahan>(a, b, interp, flat, grid, nt, t, s);
+    case kFormShear: return launch_steps_form<kFormShear>(a, b, interp, flat, grid, nt, t, s);
+    case kFormMoments: return launch_steps_form<kFormMoments>(a, b, interp, flat, grid, nt, t, s);
+    case kFormMethodA: return launch_steps_form<kFormMethodA>(a, b, interp, flat, grid, nt, t, s);
+    case kFormGeneric: return launch_steps_form<kFormGeneric>(a, b, interp, flat, grid, nt, t, s);
     default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_trace(const TraceArgs& a, int interp, bool fp64_dda, cudaStream_t s)
@@ -875,33 +890,41 @@ namespace {
 
 using BatchKernel = void (*)(const BatchArgs);
 
-// small: every bundle's grid has fewer than 2^31 points
-BatchKernel batch_kernel(int interp, bool fp64_dda, bool small)
+// small: every bundle's grid has fewer than 2^31 points; periodic: every bundle is
+template <bool PER>
+BatchKernel batch_kernel_of(int interp, bool fp64_dda, bool small)
 {
     if (interp == RR_TRILINEAR) {
-        if (fp64_dda) return trace_batch_kernel<RR_TRILINEAR, double, kAddrIndex>;
-        return small ? trace_batch_kernel<RR_TRILINEAR, float, kAddrAuto>
-                     : trace_batch_kernel<RR_TRILINEAR, float, kAddrIndex>;
+        if (fp64_dda) return trace_batch_kernel<RR_TRILINEAR, double, kAddrIndex, PER>;
+        return small ? trace_batch_kernel<RR_TRILINEAR, float, kAddrAuto, PER>
+                     : trace_batch_kernel<RR_TRILINEAR, float, kAddrIndex, PER>;
     }
-    return fp64_dda ? trace_batch_kernel<RR_NGP, double, kAddrIndex> : trace_batch_kernel<RR_NGP, float, kAddrIndex>;
+    return fp64_dda ? trace_batch_kernel<RR_NGP, double, kAddrIndex, PER>
+                    : trace_batch_kernel<RR_NGP, float, kAddrIndex, PER>;
+}
+
+BatchKernel batch_kernel(int interp, bool fp64_dda, bool small, bool periodic)
+{
+    return periodic ? batch_kernel_of<true>(interp, fp64_dda, small) : batch_kernel_of<false>(interp, fp64_dda, small);
 }
 
 }  // namespace
 
-cudaError_t launch_trace_batch(const BatchArgs& b, int interp, bool fp64_dda, int blocks, cudaStream_t s, bool small)
+cudaError_t launch_trace_batch(const BatchArgs& b, int interp, bool fp64_dda, int blocks, cudaStream_t s, bool small,
+                               bool periodic)
 {
     if (!tile_ok(b.tile) || b.chunk < 1 || blocks < 1) return cudaErrorInvalidValue;
     const int nt = 32 * b.tile.bwx * b.tile.bwy;
-    batch_kernel(interp, fp64_dda, small)<<<blocks, nt, 0, s>>>(b);
+    batch_kernel(interp, fp64_dda, small, periodic)<<<blocks, nt, 0, s>>>(b);
     return cudaGetLastError();
 }
 
-int batch_blocks_per_sm(int interp, bool fp64_dda, const TileCfg& t)
+int batch_blocks_per_sm(int interp, bool fp64_dda, bool periodic, const TileCfg& t)
 {
     const int nt = 32 * t.bwx * t.bwy;
     int n = 0;
     const cudaError_t e =
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel(interp, fp64_dda, true), nt, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel(interp, fp64_dda, true, periodic), nt, 0);
     return (e == cudaSuccess && n > 0) ? n : 1;
 }
 }  // namespace rr

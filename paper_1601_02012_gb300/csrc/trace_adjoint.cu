@@ -205,7 +205,7 @@ __device__ __forceinline__ void flush_face(double* __restrict__ grad, const long
 // The FP32 trilinear form is capped at 128 registers (4 blocks of kAdjWarps
 // warps per SM): uncapped it takes more and runs slower, and at 96 registers
 // (5 blocks) its spills cost more than the occupancy gains.
-template <int INTERP, class R>
+template <int INTERP, class R, bool PER>
 __global__ void __launch_bounds__(32 * kAdjWarps, (INTERP == RR_TRILINEAR && sizeof(R) == 4) ? 4 : 1)
     trace_adjoint_kernel(const TraceArgs A, const AdjArgs B, const TileCfg tc)
 {
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(32 * kAdjWarps, (INTERP == RR_TRILINEAR && siz
     if (gk == 0.f && gb == 0.f) return;
     const int nn[3] = {A.n0, A.n1, A.n2};
     RayRange rg;
-    if (!ray_range(A, rid, rg)) return;
+    if (!ray_range<PER>(A, rid, rg)) return;
     const R chis = (R)A.chi_s;
     const R ichis = F64 ? (R)(1.0 / A.chi_s) : (R)A.inv_chi_s_f;
     const long long sx = (long long)A.n1 * A.n2, sy = A.n2;
@@ -365,15 +365,21 @@ cudaError_t launch_trace_adjoint(const TraceArgs& a, const AdjArgs& b, int inter
     const int nt = 32 * t.bwx * t.bwy;
     if (nt > 32 * kAdjWarps) return cudaErrorInvalidConfiguration;   // the face-flush staging holds kAdjWarps warps
     if (interp == RR_TRILINEAR) {
-        if (fp64_dda)
-            trace_adjoint_kernel<RR_TRILINEAR, double><<<grid, nt, 0, s>>>(a, b, t);
-        else
-            trace_adjoint_kernel<RR_TRILINEAR, float><<<grid, nt, 0, s>>>(a, b, t);
+        if (fp64_dda) {
+            if (a.periodic) trace_adjoint_kernel<RR_TRILINEAR, double, true><<<grid, nt, 0, s>>>(a, b, t);
+            else trace_adjoint_kernel<RR_TRILINEAR, double, false><<<grid, nt, 0, s>>>(a, b, t);
+        } else {
+            if (a.periodic) trace_adjoint_kernel<RR_TRILINEAR, float, true><<<grid, nt, 0, s>>>(a, b, t);
+            else trace_adjoint_kernel<RR_TRILINEAR, float, false><<<grid, nt, 0, s>>>(a, b, t);
+        }
     } else {
-        if (fp64_dda)
-            trace_adjoint_kernel<RR_NGP, double><<<grid, nt, 0, s>>>(a, b, t);
-        else
-            trace_adjoint_kernel<RR_NGP, float><<<grid, nt, 0, s>>>(a, b, t);
+        if (fp64_dda) {
+            if (a.periodic) trace_adjoint_kernel<RR_NGP, double, true><<<grid, nt, 0, s>>>(a, b, t);
+            else trace_adjoint_kernel<RR_NGP, double, false><<<grid, nt, 0, s>>>(a, b, t);
+        } else {
+            if (a.periodic) trace_adjoint_kernel<RR_NGP, float, true><<<grid, nt, 0, s>>>(a, b, t);
+            else trace_adjoint_kernel<RR_NGP, float, false><<<grid, nt, 0, s>>>(a, b, t);
+        }
     }
     return cudaGetLastError();
 }

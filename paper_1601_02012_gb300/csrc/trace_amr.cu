@@ -51,7 +51,8 @@ __device__ __forceinline__ int amr_locate(const AmrDevice& M, const int q[3], in
     return v < 0 ? -1 : v;
 }
 
-template <int INTERP, int FORM, bool REGACC = false>
+// PER: periodic bundles only.
+template <int INTERP, int FORM, bool PER, bool REGACC = false>
 __device__ __forceinline__ void trace_ray_amr(const TraceArgs& A, const AmrDevice& M, int ix, int iy,
                                               RayAcc* acc = nullptr)
 {
@@ -69,7 +70,7 @@ __device__ __forceinline__ void trace_ray_amr(const TraceArgs& A, const AmrDevic
     const long long rid = (long long)iy * A.nx + ix;
     const int NF = A.n0;   // finest cells per side
     RayRange rg;
-    if (!ray_range(A, rid, rg)) return;
+    if (!ray_range<PER>(A, rid, rg)) return;
     if (!REGACC || !acc->loaded) {
         prefetch_l2(A.kacc + rid);
         prefetch_l2(A.bacc + rid);
@@ -350,12 +351,12 @@ __device__ __forceinline__ void trace_ray_amr(const TraceArgs& A, const AmrDevic
     }
 }
 
-template <int INTERP, int FORM>
+template <int INTERP, int FORM, bool PER>
 __global__ void __launch_bounds__(NT_MAX, 2) trace_amr_kernel(const TraceArgs A, const AmrDevice M, const TileCfg t)
 {
     int ix, iy;
     tile_ray(t, blockIdx.x, blockIdx.y, ix, iy);
-    if (ix < A.nx && iy < A.ny) trace_ray_amr<INTERP, FORM>(A, M, ix, iy);
+    if (ix < A.nx && iy < A.ny) trace_ray_amr<INTERP, FORM, PER>(A, M, ix, iy);
 }
 
 // Consecutive steps over the adaptive mesh in one launch, as
@@ -363,7 +364,7 @@ __global__ void __launch_bounds__(NT_MAX, 2) trace_amr_kernel(const TraceArgs A,
 // records, interval and scales, the ray's sums (and its shear pair) in
 // registers in between; per step the arithmetic of trace_amr_kernel, so the
 // same results bit for bit.
-template <int INTERP, int FORM>
+template <int INTERP, int FORM, bool PER>
 __global__ void __launch_bounds__(NT_MAX, 2)
     trace_amr_steps_kernel(const TraceArgs A, const AmrDevice M, const __grid_constant__ StepBlock S, const TileCfg t)
 {
@@ -381,7 +382,7 @@ __global__ void __launch_bounds__(NT_MAX, 2)
         As.Lf = st.Lf; As.D0f = st.D0f;
         As.sch = st.sch; As.scl = st.scl;
         As.bsh = st.bsh; As.bsl = st.bsl;
-        trace_ray_amr<INTERP, FORM, true>(As, M, ix, iy, &acc);
+        trace_ray_amr<INTERP, FORM, PER, true>(As, M, ix, iy, &acc);
     }
     if (acc.loaded) {
         const long long rid = (long long)iy * A.nx + ix;
@@ -397,49 +398,57 @@ __global__ void __launch_bounds__(NT_MAX, 2)
 
 }  // namespace
 
+namespace {
+
+using AmrKernel = void (*)(const TraceArgs, const AmrDevice, const TileCfg);
+using AmrStepsKernel = void (*)(const TraceArgs, const AmrDevice, const StepBlock, const TileCfg);
+
+template <int INTERP, bool PER>
+AmrKernel amr_kernel(int form)
+{
+    switch (form) {
+    case kFormShear: return trace_amr_kernel<INTERP, kFormShear, PER>;
+    case kFormMethodA: return trace_amr_kernel<INTERP, kFormMethodA, PER>;
+    case kFormGeneric: return trace_amr_kernel<INTERP, kFormGeneric, PER>;
+    default: return trace_amr_kernel<INTERP, kFormKahan, PER>;
+    }
+}
+
+template <int INTERP, bool PER>
+AmrStepsKernel amr_steps_kernel(int form)
+{
+    switch (form) {
+    case kFormKahan: return trace_amr_steps_kernel<INTERP, kFormKahan, PER>;
+    case kFormShear: return trace_amr_steps_kernel<INTERP, kFormShear, PER>;
+    case kFormMethodA: return trace_amr_steps_kernel<INTERP, kFormMethodA, PER>;
+    case kFormGeneric: return trace_amr_steps_kernel<INTERP, kFormGeneric, PER>;
+    default: return nullptr;
+    }
+}
+
+}  // namespace
+
 cudaError_t launch_trace_amr_steps(const TraceArgs& a, const AmrDevice& m, const StepBlock& b, int interp,
                                    cudaStream_t s, int form)
 {
-    if (b.n < 1 || b.n > kMaxStepBlock) return cudaErrorInvalidValue;
+    const AmrStepsKernel k = interp == RR_TRILINEAR
+                                 ? (a.periodic ? amr_steps_kernel<RR_TRILINEAR, true>(form)
+                                               : amr_steps_kernel<RR_TRILINEAR, false>(form))
+                                 : (a.periodic ? amr_steps_kernel<RR_NGP, true>(form)
+                                               : amr_steps_kernel<RR_NGP, false>(form));
+    if (!k || b.n < 1 || b.n > kMaxStepBlock) return cudaErrorInvalidValue;
     const TileCfg t;
-    const dim3 grid = tile_grid(t, a.nx, a.ny);
-    const dim3 block(32 * t.bwx * t.bwy);
-    const bool tri = interp == RR_TRILINEAR;
-#define RR_AMR_STEPS(F)                                                                              \
-    do {                                                                                              \
-        if (tri) trace_amr_steps_kernel<RR_TRILINEAR, F><<<grid, block, 0, s>>>(a, m, b, t);          \
-        else trace_amr_steps_kernel<RR_NGP, F><<<grid, block, 0, s>>>(a, m, b, t);                   \
-    } while (0)
-    switch (form) {
-    case kFormKahan: RR_AMR_STEPS(kFormKahan); break;
-    case kFormShear: RR_AMR_STEPS(kFormShear); break;
-    case kFormMethodA: RR_AMR_STEPS(kFormMethodA); break;
-    case kFormGeneric: RR_AMR_STEPS(kFormGeneric); break;
-    default: return cudaErrorInvalidValue;
-    }
-#undef RR_AMR_STEPS
+    k<<<tile_grid(t, a.nx, a.ny), 32 * t.bwx * t.bwy, 0, s>>>(a, m, b, t);
     return cudaGetLastError();
 }
 
 cudaError_t launch_trace_amr(const TraceArgs& a, const AmrDevice& m, int interp, cudaStream_t s, int form)
 {
+    const AmrKernel k = interp == RR_TRILINEAR
+                            ? (a.periodic ? amr_kernel<RR_TRILINEAR, true>(form) : amr_kernel<RR_TRILINEAR, false>(form))
+                            : (a.periodic ? amr_kernel<RR_NGP, true>(form) : amr_kernel<RR_NGP, false>(form));
     const TileCfg t;
-    const dim3 grid = tile_grid(t, a.nx, a.ny);
-    const dim3 block(32 * t.bwx * t.bwy);
-    const bool tri = interp == RR_TRILINEAR;
-    if (form == kFormShear) {
-        if (tri) trace_amr_kernel<RR_TRILINEAR, kFormShear><<<grid, block, 0, s>>>(a, m, t);
-        else trace_amr_kernel<RR_NGP, kFormShear><<<grid, block, 0, s>>>(a, m, t);
-    } else if (form == kFormGeneric) {
-        if (tri) trace_amr_kernel<RR_TRILINEAR, kFormGeneric><<<grid, block, 0, s>>>(a, m, t);
-        else trace_amr_kernel<RR_NGP, kFormGeneric><<<grid, block, 0, s>>>(a, m, t);
-    } else if (form == kFormMethodA) {
-        if (tri) trace_amr_kernel<RR_TRILINEAR, kFormMethodA><<<grid, block, 0, s>>>(a, m, t);
-        else trace_amr_kernel<RR_NGP, kFormMethodA><<<grid, block, 0, s>>>(a, m, t);
-    } else {
-        if (tri) trace_amr_kernel<RR_TRILINEAR, kFormKahan><<<grid, block, 0, s>>>(a, m, t);
-        else trace_amr_kernel<RR_NGP, kFormKahan><<<grid, block, 0, s>>>(a, m, t);
-    }
+    k<<<tile_grid(t, a.nx, a.ny), 32 * t.bwx * t.bwy, 0, s>>>(a, m, t);
     return cudaGetLastError();
 }
 

@@ -434,57 +434,60 @@ struct RayRange {
     double hi, lo;
 };
 
+// PER: periodic walks only (their kernels carry no clipping code; the others
+// are instantiated apart).
+template <bool PER>
 __device__ __forceinline__ bool ray_range(const TraceArgs& A, long long rid, RayRange& g)
 {
     g.ch = A.cah; g.cl = A.cal; g.Lf = A.Lf; g.D0f = A.D0f;
     g.hi = A.chi_a; g.lo = A.chi_b;
-    if (!A.periodic) {
-        // FP64 divisions only for the axes whose faces may lie in the step: an
-        // FP32 estimate of the distances to both faces, good to a few ulp, with
-        // a margin of 1e-5 first settles the axes that do not clip the step and
-        // the rays that miss the box (a face that the observer lies on is at 0
-        // exactly; a NaN or an infinity settles nothing). Six FP64 divisions a
-        // ray and step were half of a bounded walk of few cells: three tiles of
-        // 128^3 in 12 steps, 512^2 rays: 4.10 -> 3.07 ms per call.
-        const float4 nf4 = A.dirh[rid];
-        const float nf[3] = {nf4.x, nf4.y, nf4.z};
-        const float cb = (float)g.lo;
-        bool clip[3];
+    if constexpr (PER) return true;
+    if (A.periodic) return true;
+    // FP64 divisions only for the axes whose faces may lie in the step: an
+    // FP32 estimate of the distances to both faces, good to a few ulp, with
+    // a margin of 1e-5 first settles the axes that do not clip the step and
+    // the rays that miss the box (a face that the observer lies on is at 0
+    // exactly; a NaN or an infinity settles nothing). Six FP64 divisions a
+    // ray and step were half of a bounded walk of few cells: three tiles of
+    // 128^3 in 12 steps, 512^2 rays: 4.10 -> 3.07 ms per call.
+    const float4 nf4 = A.dirh[rid];
+    const float nf[3] = {nf4.x, nf4.y, nf4.z};
+    const float cb = (float)g.lo;
+    bool clip[3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const float r = __fdividef(1.f, nf[a]);
-            const float c0 = A.face0[a] == 0.f ? 0.f : A.face0[a] * r, c1 = A.face1[a] * r;
-            const float far = fmaxf(c0, c1), near = fminf(c0, c1);
-            const float mfar = 1e-5f * (fabsf(far) + g.ch), mnear = 1e-5f * (fabsf(near) + g.ch);
-            const bool ok = fabsf(nf[a]) > 1e-30f && fabsf(nf[a]) <= 1.f;
-            if (ok && (far + mfar < cb || near - mnear > g.ch)) return false;
-            clip[a] = !(ok && far - mfar > g.ch && (near + mnear < cb || near == 0.f));
-        }
-        if (!(clip[0] || clip[1] || clip[2])) return true;
-        const int nn[3] = {A.n0, A.n1, A.n2};
-        const double obs[3] = {A.obs0, A.obs1, A.obs2};
-        double hi = g.hi, lo = g.lo;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            if (!clip[a]) continue;
-            const double nd = A.dir[3 * rid + a];
-            const double ext = nn[a] * A.h;
-            if (nd == 0.0) {
-                if (obs[a] < 0.0 || obs[a] > ext) hi = lo;
-            } else {
-                const double c0 = -obs[a] / nd, c1 = (ext - obs[a]) / nd;
-                hi = fmin(hi, fmax(c0, c1));
-                lo = fmax(lo, fmin(c0, c1));
-            }
-        }
-        if (!(hi > lo)) return false;
-        g.hi = hi;
-        g.lo = lo;
-        g.ch = (float)hi;
-        g.cl = (float)(hi - (double)g.ch);
-        g.Lf = (float)(hi - lo);
-        g.D0f = (float)(A.chi_s - hi);
+    for (int a = 0; a < 3; ++a) {
+        const float r = __fdividef(1.f, nf[a]);
+        const float c0 = A.face0[a] == 0.f ? 0.f : A.face0[a] * r, c1 = A.face1[a] * r;
+        const float far = fmaxf(c0, c1), near = fminf(c0, c1);
+        const float mfar = 1e-5f * (fabsf(far) + g.ch), mnear = 1e-5f * (fabsf(near) + g.ch);
+        const bool ok = fabsf(nf[a]) > 1e-30f && fabsf(nf[a]) <= 1.f;
+        if (ok && (far + mfar < cb || near - mnear > g.ch)) return false;
+        clip[a] = !(ok && far - mfar > g.ch && (near + mnear < cb || near == 0.f));
     }
+    if (!(clip[0] || clip[1] || clip[2])) return true;
+    const int nn[3] = {A.n0, A.n1, A.n2};
+    const double obs[3] = {A.obs0, A.obs1, A.obs2};
+    double hi = g.hi, lo = g.lo;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        if (!clip[a]) continue;
+        const double nd = A.dir[3 * rid + a];
+        const double ext = nn[a] * A.h;
+        if (nd == 0.0) {
+            if (obs[a] < 0.0 || obs[a] > ext) hi = lo;
+        } else {
+            const double c0 = -obs[a] / nd, c1 = (ext - obs[a]) / nd;
+            hi = fmin(hi, fmax(c0, c1));
+            lo = fmax(lo, fmin(c0, c1));
+        }
+    }
+    if (!(hi > lo)) return false;
+    g.hi = hi;
+    g.lo = lo;
+    g.ch = (float)hi;
+    g.cl = (float)(hi - (double)g.ch);
+    g.Lf = (float)(hi - lo);
+    g.D0f = (float)(A.chi_s - hi);
     return true;
 }
 
