@@ -118,6 +118,9 @@ TraceArgs make_trace_args(const rr_bundle_desc& b, const RayState& st, const rr_
     a.D0f = (float)(b.chi_s - chi_a);
     a.inv_chi_s_f = (float)(1.0 / b.chi_s);
     a.sub_len = (float)(32.0 * a.h);
+    // (as a ray divides its own clipped path)
+    a.nsub = (int)std::max(1.f, std::min(ceilf(a.Lf / a.sub_len), 1e9f));
+    a.dsub = a.Lf / (float)a.nsub;
     a.periodic = (b.flags & RR_PERIODIC) ? 1 : 0;
     // flat addressing over the whole grid's records (32-bit point indices: a
     // grid of 2^31 points or more gets an empty box, which no sub-step lies in)
@@ -660,6 +663,8 @@ rr_status rr_trace_steps(rr_ctx* ctx, const rr_grid_desc* grid, int32_t nsteps, 
             st.rec = a.rec;
             st.chi_a = a.chi_a; st.chi_b = a.chi_b;
             st.cah = a.cah; st.cal = a.cal; st.Lf = a.Lf; st.D0f = a.D0f;
+            st.nsub = a.nsub;
+            st.dsub = a.dsub;
             st.sch = a.sch; st.scl = a.scl; st.bsh = a.bsh; st.bsl = a.bsl;
             for (int q = 0; q < 3; ++q) {
                 st.fo[q] = a.fo[q];

@@ -70,6 +70,8 @@ struct TraceArgs {
     float D0f;                  // chi_s - chi_a rounded to FP32
     float inv_chi_s_f;          // 1/chi_s rounded to FP32
     float sub_len;              // FP32 walk: longest sub-step (32 cell sizes)
+    int nsub;                   // the whole step's sub-steps and their equal length
+    float dsub;
     int periodic;
     const double* dir;
     const float4* dirh;
@@ -98,6 +100,8 @@ struct StepArgs {
     const float4* rec;
     double chi_a, chi_b;
     float cah, cal, Lf, D0f;
+    int nsub;
+    float dsub;
     float sch, scl, bsh, bsl;
     int fo[3], fe[3];
     int fs0, fs1;

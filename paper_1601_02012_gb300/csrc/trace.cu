@@ -36,37 +36,23 @@ namespace rr {
 namespace {
 
 // Crossing face e of the mirrored cell: the 4 corners on the exit side become
-// the entry side and the 4 new corner values p come in on the exit side.
-// SEL: the same moves as selects on e (no divergent branches), slot by slot
-// the value it takes for e = 0, 1, 2. Selects are used everywhere: faster in
-// the shear and Method A forms and in the multi-step kernels (2 % on the
-// production pass), the same as the branches for one default step per launch.
-template <bool SEL = true>
-__device__ __forceinline__ void shift_corners(float2 q[8], const float2 p[4], int e)
+// the entry side and the 4 new corner values p come in on the exit side, slot
+// by slot as selects on e (e0: e = 0, e1: e = 1): the rays of a warp rarely
+// cross the same face at the same iteration, and branches would diverge (2 %
+// slower on the production pass).
+__device__ __forceinline__ void shift_corners(float2 q[8], const float2 p[4], bool e0, bool e1)
 {
-    if constexpr (SEL) {
-        const bool e0 = e == 0, e1 = e == 1;
-        float2 n[8];
-        n[0] = e0 ? q[1] : (e1 ? q[2] : q[4]);
-        n[1] = e0 ? p[0] : (e1 ? q[3] : q[5]);
-        n[2] = e0 ? q[3] : (e1 ? p[0] : q[6]);
-        n[3] = (e0 || e1) ? p[1] : q[7];
-        n[4] = e0 ? q[5] : (e1 ? q[6] : p[0]);
-        n[5] = e0 ? p[2] : (e1 ? q[7] : p[1]);
-        n[6] = e0 ? q[7] : p[2];
-        n[7] = p[3];
+    float2 n[8];
+    n[0] = e0 ? q[1] : (e1 ? q[2] : q[4]);
+    n[1] = e0 ? p[0] : (e1 ? q[3] : q[5]);
+    n[2] = e0 ? q[3] : (e1 ? p[0] : q[6]);
+    n[3] = (e0 || e1) ? p[1] : q[7];
+    n[4] = e0 ? q[5] : (e1 ? q[6] : p[0]);
+    n[5] = e0 ? p[2] : (e1 ? q[7] : p[1]);
+    n[6] = e0 ? q[7] : p[2];
+    n[7] = p[3];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) q[i] = n[i];
-    } else if (e == 0) {
-        q[0] = q[1]; q[2] = q[3]; q[4] = q[5]; q[6] = q[7];
-        q[1] = p[0]; q[3] = p[1]; q[5] = p[2]; q[7] = p[3];
-    } else if (e == 1) {
-        q[0] = q[2]; q[1] = q[3]; q[4] = q[6]; q[5] = q[7];
-        q[2] = p[0]; q[3] = p[1]; q[6] = p[2]; q[7] = p[3];
-    } else {
-        q[0] = q[4]; q[1] = q[5]; q[2] = q[6]; q[3] = q[7];
-        q[4] = p[0]; q[5] = p[1]; q[6] = p[2]; q[7] = p[3];
-    }
+    for (int i = 0; i < 8; ++i) q[i] = n[i];
 }
 
 // What the sub-steps of one ray's step accumulate and hand on.
@@ -144,12 +130,10 @@ constexpr float kSliver = 4.76837158203125e-07f;
 //               range first and, outside it, flags kErrRange and reads nothing.
 template <int INTERP, class R, int FORM, int ADDR>
 __device__ __forceinline__ void walk_piece(const TraceArgs& A, Walk<R>& W, const RayWeights& V, int j, bool resume,
-                                           int fB, const int fd[3], PieceState<R>& S)
+                                           PieceState<R>& S)
 {
     using OT = unsigned long long;
     constexpr bool PLANES = ADDR == kAddrPlanes;
-    constexpr bool FLAT = ADDR == kAddrFlat;
-    static_assert(!FLAT || (INTERP == RR_TRILINEAR && sizeof(R) == 4), "flat addressing: FP32 trilinear walk");
     constexpr bool F64 = sizeof(R) == 8;
     constexpr bool SH = !F64 && FORM == kFormShear;
     constexpr bool MA = !F64 && FORM == kFormMethodA;
@@ -192,11 +176,9 @@ __device__ __forceinline__ void walk_piece(const TraceArgs& A, Walk<R>& W, const
     const R eps_rel = F64 ? (R)1.4551915228366852e-11 : (R)kSliver;
     const R eps_end = L * eps_rel;
     const int max_iter = W.max_iter;
-    float kf[3] = {0.f, 0.f, 0.f};   // FLAT: crossing counts as floats
     auto fetch = [&](long long i) -> PR {
         if constexpr (MA) return load_grad_rec(A.rec, i);
         else if constexpr (GEN) return __ldg(reinterpret_cast<const float2*>(A.rec) + i);
-        else if constexpr (FLAT) return load_rec32(A.rec, i);
         else return load_rec(A.rec, i);
     };
     // (the channel pair the walk integrates) of a record
@@ -216,9 +198,7 @@ __device__ __forceinline__ void walk_piece(const TraceArgs& A, Walk<R>& W, const
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
             long long o;
-            if constexpr (FLAT) {
-                o = (unsigned)(fB + ((m & 1) ? fd[0] : 0) + ((m & 2) ? fd[1] : 0) + ((m & 4) ? fd[2] : 0));
-            } else if constexpr (PLANES) {
+            if constexpr (PLANES) {
                 o = (long long)(((m & 1) ? phi[0] : plo[0]) + ((m & 2) ? phi[1] : plo[1]) +
                                 ((m & 4) ? phi[2] : plo[2]));
             } else {
@@ -255,8 +235,7 @@ __device__ __forceinline__ void walk_piece(const TraceArgs& A, Walk<R>& W, const
         R u[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            if constexpr (FLAT) u[a] = __saturatef(fmaf(sig - T[a], v[a], cu[a]));
-            else u[a] = fmin(fmax(fma(sig - T[a], v[a], cu[a]), (R)0), (R)1);
+            u[a] = fmin(fmax(fma(sig - T[a], v[a], cu[a]), (R)0), (R)1);
         }
 
         // Prefetch the next cell's new records before this segment's arithmetic.
@@ -265,19 +244,7 @@ __device__ __forceinline__ void walk_piece(const TraceArgs& A, Walk<R>& W, const
         OT nph = 0;     // offset of the vertex plane beyond the exit face (PLANES)
         int nvhi = 0;   // its vertex index (otherwise)
         PR nr[4];
-        // FLAT: the stride along the exit axis
-        const int fde = e == 0 ? fd[0] : (e == 1 ? fd[1] : fd[2]);
-        if (FLAT && !last) {
-            // the new exit-side corners: B + 2 d_e plus 0, d_A, d_B, d_A + d_B
-            // over the other two axes A < B
-            const int P = fB + 2 * fde;
-            const int dA = e == 0 ? fd[1] : fd[0];
-            const int dB = e == 2 ? fd[1] : fd[2];
-            nr[0] = fetch((unsigned)P);
-            nr[1] = fetch((unsigned)(P + dA));
-            nr[2] = fetch((unsigned)(P + dB));
-            nr[3] = fetch((unsigned)(P + dA + dB));
-        } else if (!last) {
+        if (!last) {
 #pragma unroll
             for (int a = 0; a < 3; ++a)
                 if (a == e) {
@@ -428,15 +395,6 @@ __device__ __forceinline__ void walk_piece(const TraceArgs& A, Walk<R>& W, const
         if (last) break;
 
         // cross the exit face e
-        if constexpr (FLAT) {
-            fB += fde;
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-                if (a == e) {
-                    kf[a] += 1.f;
-                    T[a] = fmaf(kf[a], td[a], T0[a]);
-                }
-        } else {
         if (!A.periodic && (ncell < 0 || ncell >= ne)) break;
 #pragma unroll
         for (int a = 0; a < 3; ++a)
@@ -453,16 +411,15 @@ __device__ __forceinline__ void walk_piece(const TraceArgs& A, Walk<R>& W, const
                 if constexpr (F64) T[a] = fma((R)k[a], td[a], T0[a]);
                 else T[a] = fmaf(i2f_exact(k[a]), td[a], T0[a]);
             }
-        }
         if (INTERP == RR_TRILINEAR) {
             float2 p2[4];
 #pragma unroll
             for (int r = 0; r < 4; ++r) p2[r] = pair(nr[r]);
-            shift_corners(q2, p2, e);
+            shift_corners(q2, p2, e == 0, e == 1);
             if constexpr (SH) {
 #pragma unroll
                 for (int r = 0; r < 4; ++r) p2[r] = make_float2(project(V.w1, nr[r]), project(V.w2, nr[r]));
-                shift_corners<true>(g2, p2, e);
+                shift_corners(g2, p2, e == 0, e == 1);
             }
         } else {
             q2[0] = pair(nr[0]);
@@ -473,13 +430,163 @@ __device__ __forceinline__ void walk_piece(const TraceArgs& A, Walk<R>& W, const
             break;
         }
     }
-    if constexpr (FLAT) {
-        // the cell the walk ended in (a box-local walk may have passed the seam, once)
-        S.pc0 = wrap_once(c[0] + sgn[0] * f2i_exact(kf[0]), nn[0]);
-        S.pc1 = wrap_once(c[1] + sgn[1] * f2i_exact(kf[1]), nn[1]);
-        S.pc2 = wrap_once(c[2] + sgn[2] * f2i_exact(kf[2]), nn[2]);
+    S.pc0 = c[0]; S.pc1 = c[1]; S.pc2 = c[2];
+}
+
+// The contribution of one segment of the FP32 trilinear walk (path sig .. tend
+// of the sub-step, corner pairs q and, for the shear, g) to the step's sums;
+// slivers are skipped. SELECT: by selecting the old sums afterwards instead of
+// branching around the arithmetic (three control instructions a segment):
+// default form 21.52 -> 21.23 ms per production pass; the forms with more sums
+// or fewer registers to spare keep the branch.
+template <int FORM, bool SELECT>
+__device__ __forceinline__ void add_segment(const TraceArgs& A, const Walk<float>& W, const float2 q[8],
+                                            const float2* g, const float T[3], float sig, float tend,
+                                            PieceState<float>& S)
+{
+    const float t = tend - sig;
+    // mirrored entry point of this segment
+    float u[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) u[a] = __saturatef(fmaf(sig - T[a], W.v[a], W.cu[a]));
+    const bool live = t > tend * kSliver;
+    if (!SELECT && !live) return;
+    const PieceState<float> S0 = S;
+    const float chis = (float)A.chi_s, ichis = A.inv_chi_s_f;
+    float2 e[4];
+    line_cubic2(q, bc2(u[0]), bc2(u[1]), bc2(u[2]), bc2(W.v[0]), bc2(W.v[1]), bc2(W.v[2]), e);
+    const float chiA = W.chiA0 - sig;
+    if constexpr (FORM == kFormMoments) {
+        S.s2.add(dot_kernel(e, t, chiA, -1.f, 0.f));
+        S.s2m.add(dot_kernel(e, t, chiA * chiA, -2.f * chiA, 1.f));
+    } else if constexpr (FORM == kFormGeneric) {
+        // each channel's kernel about the entry point: K(chi_A - s) = K(chi_A) -
+        // K'(chi_A) s + k2 s^2
+        const float2 G0 = make_float2(fmaf(chiA, fmaf(chiA, A.kq[2], A.kq[1]), A.kq[0]),
+                                      fmaf(chiA, fmaf(chiA, A.kq[5], A.kq[4]), A.kq[3]));
+        const float2 G1 = make_float2(-fmaf(2.f * A.kq[2], chiA, A.kq[1]), -fmaf(2.f * A.kq[5], chiA, A.kq[4]));
+        S.s2.add(dot_kernel_pair(e, t, G0, G1, make_float2(A.kq[2], A.kq[5])));
     } else {
-        S.pc0 = c[0]; S.pc1 = c[1]; S.pc2 = c[2];
+        float G0, G1, G2;
+        kernel_coeffs(t, sig, W.chiA0, W.D0, chis, ichis, G0, G1, G2);
+        const float2 x = FORM == kFormMethodA ? dot_kernel_a(e, t, G0, G1, G2) : dot_kernel(e, t, G0, G1, G2);
+        if constexpr (FORM == kFormPlain) S.s2.s = __fadd2_rn(S.s2.s, x);
+        else S.s2.add(x);
+        if constexpr (FORM == kFormShear)
+            S.s2m.add(segment_trilinear(g, u[0], u[1], u[2], W.v[0], W.v[1], W.v[2], t, G0, G1, G2));
+    }
+    ++S.cnt;
+    if (SELECT && !live) S = S0;
+}
+
+// walk_piece with flat addressing (FP32 trilinear): the same segments with the
+// same arithmetic. The loop holds crossings only; the segment that ends the
+// sub-step follows it, once for the whole warp, without the loads, the
+// projections and the corner shift that a crossing needs, and one test ends the
+// loop on the last segment and on the cap alike. Bound by issue slots (FMA pipes
+// 58 % and ALU 47 % busy at 75 % issue); production pass, trace kernels 22.62 ->
+// 21.52 ms without the last segment in the loop, 20.83 ms with one test.
+// (B: point index of the entry corner, fd: index step per axis along the
+// motion; more: another sub-step follows)
+template <int FORM, bool SELECT>
+__device__ __forceinline__ void walk_flat(const TraceArgs& A, const Walk<float>& W, const RayWeights& V, bool first,
+                                          bool more, bool resume, int B, const int fd[3], PieceState<float>& S)
+{
+    constexpr bool SH = FORM == kFormShear;
+    constexpr bool MA = FORM == kFormMethodA;
+    constexpr bool GEN = FORM == kFormGeneric;
+    using PR = typename std::conditional<MA, float4, typename std::conditional<GEN, float2, Rec>::type>::type;
+    auto fetch = [&](int i) -> PR {
+        if constexpr (MA) return load_grad_rec(A.rec, (unsigned)i);
+        else if constexpr (GEN) return __ldg(reinterpret_cast<const float2*>(A.rec) + (unsigned)i);
+        else return load_rec32(A.rec, (unsigned)i);
+    };
+    auto pair = [&](const PR& r) -> float2 {
+        if constexpr (MA) return radial_pair(V.nd, r);
+        else if constexpr (GEN) return r;
+        else return make_float2(project(W.w, r), r.b.z);
+    };
+    float2 q[8], g[SH ? 8 : 1];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+        const PR r = fetch(B + ((m & 1) ? fd[0] : 0) + ((m & 2) ? fd[1] : 0) + ((m & 4) ? fd[2] : 0));
+        q[m] = pair(r);
+        if constexpr (SH) g[m] = make_float2(project(V.w1, r), project(V.w2, r));
+    }
+    float sig = 0.f;                          // path from the sub-step start to the segment entry
+    float T[3] = {W.T0[0], W.T0[1], W.T0[2]};   // path to the next face crossing per axis
+    float kf[3] = {0.f, 0.f, 0.f};            // crossings so far
+    const float lim = W.L - W.L * kSliver;
+    int left = W.max_iter + 1;
+    // (a resumed first segment is not a new one; it is integrated unless the
+    // walk starts on its exit face)
+    if (resume && T[0] > 0.f && T[1] > 0.f && T[2] > 0.f) --S.cnt;
+    if constexpr (MA) {
+        // the surface term of Eq. (2nterm) at the start of the traced interval
+        if (first) {
+            float u[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) u[a] = __saturatef(fmaf(sig - T[a], W.v[a], W.cu[a]));
+            S.qa = trilinear_x(q, u[0], u[1], u[2]);
+            S.ga = W.D0 * W.chiA0 * A.inv_chi_s_f;
+        }
+    }
+    while (true) {
+        // exit plane: the nearest face crossing (lowest axis on ties)
+        const bool p1 = T[1] < T[0];
+        const float t01 = p1 ? T[1] : T[0];
+        const bool e2 = T[2] < t01;
+        const float tend = e2 ? T[2] : t01;
+        if (!(tend < lim) | (left == 0)) break;
+        --left;
+        const bool e0 = !e2 && !p1, e1 = !e2 && p1;
+        // the new exit-side corners, loaded ahead of this segment's arithmetic:
+        // B + 2 d_e plus 0, d_A, d_B, d_A + d_B over the other two axes A < B
+        const int fde = e2 ? fd[2] : (p1 ? fd[1] : fd[0]);
+        const int P = B + 2 * fde;
+        const int dA = e0 ? fd[1] : fd[0];
+        const int dB = e2 ? fd[1] : fd[2];
+        const PR r[4] = {fetch(P), fetch(P + dA), fetch(P + dB), fetch(P + dA + dB)};
+        add_segment<FORM, SELECT>(A, W, q, g, T, sig, tend, S);
+        // cross the exit face
+        sig = tend;
+        B += fde;
+        if (e0) { kf[0] += 1.f; T[0] = fmaf(kf[0], W.td[0], W.T0[0]); }
+        if (e1) { kf[1] += 1.f; T[1] = fmaf(kf[1], W.td[1], W.T0[1]); }
+        if (e2) { kf[2] += 1.f; T[2] = fmaf(kf[2], W.td[2], W.T0[2]); }
+        float2 p[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) p[i] = pair(r[i]);
+        shift_corners(q, p, e0, e1);
+        if constexpr (SH) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) p[i] = make_float2(project(V.w1, r[i]), project(V.w2, r[i]));
+            shift_corners(g, p, e0, e1);
+        }
+    }
+    // (no crossing left: the cap ended the walk, or it ended on its last allowed one)
+    if (left == 0 && fminf(fminf(T[0], T[1]), T[2]) < lim) {
+        S.overflow = true;
+        return;
+    }
+    add_segment<FORM, SELECT>(A, W, q, g, T, sig, W.L, S);
+    if constexpr (MA) {
+        // the surface term at the end of the interval (the last sub-step's stays)
+        const float t = W.L - sig;
+        float u[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            u[a] = __saturatef(fmaf(t, W.v[a], __saturatef(fmaf(sig - T[a], W.v[a], W.cu[a]))));
+        S.qb = trilinear_x(q, u[0], u[1], u[2]);
+        float G0, G1, G2;
+        kernel_coeffs(t, sig, W.chiA0, W.D0, (float)A.chi_s, A.inv_chi_s_f, G0, G1, G2);
+        S.gb = fmaf(t, fmaf(t, G2, G1), G0);
+    }
+    if (more) {
+        // the cell the walk ended in (a box-local walk may have passed the seam, once)
+        S.pc0 = wrap_once(W.c[0] + W.sgn[0] * f2i_exact(kf[0]), A.n0);
+        S.pc1 = wrap_once(W.c[1] + W.sgn[1] * f2i_exact(kf[1]), A.n1);
+        S.pc2 = wrap_once(W.c[2] + W.sgn[2] * f2i_exact(kf[2]), A.n2);
     }
 }
 
@@ -494,13 +601,23 @@ __device__ __noinline__ void index_piece(const TraceArgs& A, long long rid, floa
     ray_weights<FORM>(A, rid, V);
     Walk<float> W;
     walk_setup<float>(A, rid, bh, bl, Lj, D0j, 0.0, 0.0, W);
-    const int fd[3] = {0, 0, 0};
-    walk_piece<RR_TRILINEAR, float, FORM, kAddrIndex>(A, W, V, j, resume, 0, fd, S);
+    walk_piece<RR_TRILINEAR, float, FORM, kAddrIndex>(A, W, V, j, resume, S);
 }
 
-// PER: periodic bundles only.
+// Whether a multi-step kernel sets a ray's constants up once, outside its loop
+// over the steps, and takes the sub-steps' division from the host. Production
+// pass, trace kernels: default form 20.83 -> 20.33 ms, shear (256^3, 1024^2 rays,
+// 20 steps) 4.46 -> 4.37 ms; the moments, Method A and the index walks spill or
+// gain nothing (3.00 -> 3.08, 2.57 -> 2.63, NGP 1.73 -> 1.78 ms) and keep both
+// inside.
+template <int FORM, int ADDR>
+constexpr bool kHoist = ADDR == kAddrFlat && (FORM == kFormKahan || FORM == kFormShear);
+
+// PER: periodic bundles only. REGACC: one of several steps of a launch; acc and
+// W0 (the ray's constants) live across them.
 template <int INTERP, class R, int FORM, int ADDR, bool PER, bool REGACC = false>
-__device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, RayAcc* acc = nullptr)
+__device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, RayAcc* acc = nullptr,
+                                          const Walk<R>* W0 = nullptr)
 {
     static_assert(!REGACC || (FORM != kFormPlain && sizeof(R) == 4), "register accumulators: FP32 compensated forms");
     constexpr bool AUTO = ADDR == kAddrAuto;
@@ -523,17 +640,19 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
         }
     }
     // FP32: sub-steps of at most sub_len, so that the path variable stays small
-    const int nsub = F64 ? 1 : max(1, (int)ceilf(rg.Lf / A.sub_len));
-    const float dsub = rg.Lf / (float)nsub;
+    constexpr bool HOIST = REGACC && kHoist<FORM, ADDR>;
+    const int nsub = F64 ? 1 : (HOIST ? A.nsub : max(1, (int)ceilf(rg.Lf / A.sub_len)));
+    const float dsub = HOIST ? A.dsub : rg.Lf / (float)nsub;
 
     RayWeights V;
     ray_weights<FORM>(A, rid, V);
+    Walk<R> W;
+    if constexpr (HOIST) W = *W0;
     PieceState<R> S;
     for (int j = 0; j < nsub && !S.overflow; ++j) {
     float bh, bl, Lj, D0j;
     sub_step(rg, j, nsub, dsub, bh, bl, Lj, D0j);
-    Walk<R> W;
-    walk_setup<R>(A, rid, bh, bl, Lj, D0j, rg.hi, rg.lo, W);
+    walk_setup<R, false, !HOIST>(A, rid, bh, bl, Lj, D0j, rg.hi, rg.lo, W);
     // FLAT: entry corner B, strides d
     int fB = 0, fd[3] = {0, 0, 0};
     bool inside = true;
@@ -581,7 +700,7 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
     const bool resume = j > 0 && W.c[0] == S.pc0 && W.c[1] == S.pc1 && W.c[2] == S.pc2;
     if constexpr (AUTO) {
         if (inside) {
-            walk_piece<INTERP, R, FORM, kAddrFlat>(A, W, V, j, resume, fB, fd, S);
+            walk_flat<FORM, false>(A, W, V, j == 0, j + 1 < nsub, resume, fB, fd, S);
         } else {
             // (only what the form carries: each further word costs the common
             // path registers around the call)
@@ -597,7 +716,8 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
             S = Q;
         }
     } else {
-        walk_piece<INTERP, R, FORM, ADDR>(A, W, V, j, resume, fB, fd, S);
+        if constexpr (FLAT) walk_flat<FORM, FORM == kFormKahan || FORM == kFormPlain || FORM == kFormMoments>(A, W, V, j == 0, j + 1 < nsub, resume, fB, fd, S);
+        else walk_piece<INTERP, R, FORM, ADDR>(A, W, V, j, resume, S);
     }
     }
 
@@ -696,6 +816,8 @@ __global__ void __launch_bounds__(NT_MAX, 2)
     if (ix >= A.nx || iy >= A.ny) return;
     RayAcc acc;
     acc.loaded = false;
+    Walk<float> W0;
+    if constexpr (kHoist<FORM, ADDR>) ray_consts<float>(A, (long long)iy * A.nx + ix, W0);
     for (int g = 0; g < S.n; ++g) {
         const StepArgs& st = S.s[g];
         TraceArgs As = A;
@@ -703,12 +825,13 @@ __global__ void __launch_bounds__(NT_MAX, 2)
         As.chi_a = st.chi_a; As.chi_b = st.chi_b;
         As.cah = st.cah; As.cal = st.cal;
         As.Lf = st.Lf; As.D0f = st.D0f;
+        As.nsub = st.nsub; As.dsub = st.dsub;
         As.sch = st.sch; As.scl = st.scl;
         As.bsh = st.bsh; As.bsl = st.bsl;
         As.fo[0] = st.fo[0]; As.fo[1] = st.fo[1]; As.fo[2] = st.fo[2];
         As.fe[0] = st.fe[0]; As.fe[1] = st.fe[1]; As.fe[2] = st.fe[2];
         As.fs0 = st.fs0; As.fs1 = st.fs1;
-        trace_ray<INTERP, float, FORM, ADDR, PER, true>(As, ix, iy, &acc);
+        trace_ray<INTERP, float, FORM, ADDR, PER, true>(As, ix, iy, &acc, &W0);
     }
     if (acc.loaded) {
         const long long rid = (long long)iy * A.nx + ix;

@@ -521,19 +521,48 @@ __device__ __forceinline__ void sub_step(const RayRange& g, int j, int nsub, flo
 // ray `rid` for a walk of length Lf (see the file comment). EXACT: as for
 // sub_step (the start cell through the exact bit pattern, the periodic wrap
 // only for cells outside [0, n)).
-template <class R, bool EXACT = false>
+//
+// The part that does not change along a ray (motion signs, crossing rates, Q
+// weights) is ray_consts, which a kernel that walks a ray through many steps
+// runs once per ray (three divisions and the nine operations of w): CONSTS
+// false.
+template <class R>
+__device__ __forceinline__ void ray_consts(const TraceArgs& A, long long rid, Walk<R>& W)
+{
+    constexpr bool F64 = sizeof(R) == 8;
+    const float4 nh4 = A.dirh[rid];
+    const float nh[3] = {nh4.x, nh4.y, nh4.z};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        W.sgn[a] = nh[a] > 0.f ? -1 : 1;   // motion along a is -n_a
+        if constexpr (F64) W.v[a] = (R)(fabs(A.dir[3 * rid + a]) * A.inv_h);
+        else W.v[a] = fabsf(nh[a]) * A.inv_hf;
+        W.td[a] = W.v[a] > (R)0 ? (R)1 / W.v[a] : (R)0;
+    }
+    // (sums of products rounded as written: every kernel gets the same weights)
+    W.w[0] = __fadd_rn(__fmul_rn(nh[1], nh[1]), __fmul_rn(nh[2], nh[2]));
+    W.w[1] = __fadd_rn(__fmul_rn(nh[0], nh[0]), __fmul_rn(nh[2], nh[2]));
+    W.w[2] = __fadd_rn(__fmul_rn(nh[0], nh[0]), __fmul_rn(nh[1], nh[1]));
+    W.w[3] = -2.f * nh[0] * nh[1];
+    W.w[4] = -2.f * nh[0] * nh[2];
+    W.w[5] = -2.f * nh[1] * nh[2];
+}
+
+template <class R, bool EXACT = false, bool CONSTS = true>
 __device__ __forceinline__ void walk_setup(const TraceArgs& A, long long rid, float ch, float cl, float Lf,
                                            float D0f, double hi, double lo, Walk<R>& W)
 {
     constexpr bool F64 = sizeof(R) == 8;
+    if constexpr (CONSTS) ray_consts<R>(A, rid, W);
     const int nn[3] = {A.n0, A.n1, A.n2};
     const float4 nh4 = A.dirh[rid];
     const float nh[3] = {nh4.x, nh4.y, nh4.z};
 
     // Start cell; distances (in cells) from the start point to the lower and
     // upper face on each axis.
-    int* c = W.c; int* sgn = W.sgn; int* k = W.k;
-    R* T0 = W.T0; R* td = W.td; R* v = W.v; R* cu = W.cu;
+    int* c = W.c; int* k = W.k;
+    const int* sgn = W.sgn;
+    R* T0 = W.T0; R* cu = W.cu;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         R flo, fhi;   // distance to the lower / upper face
@@ -596,22 +625,15 @@ __device__ __forceinline__ void walk_setup(const TraceArgs& A, long long rid, fl
             ci = nn[a] - 1; flo = (R)1; fhi = (R)0;
         }
         c[a] = ci;
-        sgn[a] = nh[a] > 0.f ? -1 : 1;   // motion along a is -n_a
         const R u0 = sgn[a] > 0 ? flo : fhi;      // mirrored: grows along the motion
         const R e0 = sgn[a] > 0 ? fhi : flo;      // distance to the exit face
-        R va;
-        if constexpr (F64) va = (R)(fabs(A.dir[3 * rid + a]) * A.inv_h);
-        else va = fabsf(nh[a]) * A.inv_hf;
-        v[a] = va;
         k[a] = 0;
-        if (va > (R)0) {
+        if (W.v[a] > (R)0) {
             // path to the k-th face crossing on this axis: T0 + k td (one rounding)
-            td[a] = (R)1 / va;
-            T0[a] = e0 * td[a];
+            T0[a] = e0 * W.td[a];
             cu[a] = (R)1;
         } else {
             T0[a] = (R)1e30;   // never crosses; u stays u0
-            td[a] = (R)0;
             cu[a] = u0;
         }
     }
@@ -623,15 +645,6 @@ __device__ __forceinline__ void walk_setup(const TraceArgs& A, long long rid, fl
         vlo[a] = sgn[a] > 0 ? c[a] : up;
         vhi[a] = sgn[a] > 0 ? up : c[a];
     }
-    float* w = W.w;
-    // (sums of products rounded as written: every kernel gets the same weights)
-    w[0] = __fadd_rn(__fmul_rn(nh[1], nh[1]), __fmul_rn(nh[2], nh[2]));
-    w[1] = __fadd_rn(__fmul_rn(nh[0], nh[0]), __fmul_rn(nh[2], nh[2]));
-    w[2] = __fadd_rn(__fmul_rn(nh[0], nh[0]), __fmul_rn(nh[1], nh[1]));
-    w[3] = -2.f * nh[0] * nh[1];
-    w[4] = -2.f * nh[0] * nh[2];
-    w[5] = -2.f * nh[1] * nh[2];
-
     W.L = F64 ? (R)(hi - lo) : (R)Lf;
     W.chiA0 = F64 ? (R)hi : (R)ch;
     W.D0 = F64 ? (R)(A.chi_s - hi) : (R)D0f;
