@@ -642,14 +642,16 @@ rr_status rr_trace_steps(rr_ctx* ctx, const rr_grid_desc* grid, int32_t nsteps, 
     const TraceArgs a0 = make_trace_args(ctx, grid, rec[0], chi_a[0], chi_b[0], scale[0], a_step[0]);
     cudaStream_t s = (cudaStream_t)stream;
     cudaError_t e = cudaSuccess;
-    // blocks of up to kMaxStepBlock steps that all take the flat addressing
-    // (trilinear) or any steps (NGP) go to one launch each; a trilinear step
-    // outside the flat range is launched on its own
+    // blocks of up to kMaxStepBlock steps go to one launch each: steps that all
+    // take the flat addressing, or all choose it per sub-step (trilinear), or
+    // any (NGP); a step on a grid of 2^31 points is launched on its own
+    const bool small = a0.fe[0] > 0;
     int32_t i = 0;
     while (i < nsteps && e == cudaSuccess) {
         const bool tri = b.interp == RR_TRILINEAR;
         auto flat_at = [&](int32_t k) { return boxes || flat_ok(whole, b.obs, *grid, chi_a[k], chi_b[k]); };
-        if (tri && !flat_at(i)) {
+        const bool flat = tri && flat_at(i);
+        if (tri && !flat && !small) {
             const TraceArgs a = make_trace_args(ctx, grid, rec[i], chi_a[i], chi_b[i], scale[i], a_step[i]);
             e = launch_trace(a, b.interp, false, s, TileCfg{}, form, false);
             ++i;
@@ -657,7 +659,7 @@ rr_status rr_trace_steps(rr_ctx* ctx, const rr_grid_desc* grid, int32_t nsteps, 
         }
         StepBlock blk{};
         blk.n = 0;
-        while (i < nsteps && blk.n < kMaxStepBlock && (!tri || flat_at(i))) {
+        while (i < nsteps && blk.n < kMaxStepBlock && (!tri || flat_at(i) == flat)) {
             const TraceArgs a = make_trace_args(ctx, grid, rec[i], chi_a[i], chi_b[i], scale[i], a_step[i]);
             StepArgs& st = blk.s[blk.n++];
             st.rec = a.rec;
@@ -683,7 +685,14 @@ rr_status rr_trace_steps(rr_ctx* ctx, const rr_grid_desc* grid, int32_t nsteps, 
             }
             ++i;
         }
-        e = launch_trace_steps(a0, blk, b.interp, tri, s, form);
+        if (tri && !flat && blk.n == 1) {
+            // (the single-step kernel spills less than the multi-step one)
+            const int32_t k = i - 1;
+            const TraceArgs a = make_trace_args(ctx, grid, rec[k], chi_a[k], chi_b[k], scale[k], a_step[k]);
+            e = launch_trace(a, b.interp, false, s, TileCfg{}, form, false);
+        } else {
+            e = launch_trace_steps(a0, blk, b.interp, flat, s, form);
+        }
     }
     return from_cuda(e);
 }

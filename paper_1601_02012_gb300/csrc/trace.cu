@@ -129,8 +129,8 @@ constexpr float kSliver = 4.76837158203125e-07f;
 //               the step's footprint box; each sub-step checks its own cell
 //               range first and, outside it, flags kErrRange and reads nothing.
 template <int INTERP, class R, int FORM, int ADDR>
-__device__ __forceinline__ void walk_piece(const TraceArgs& A, Walk<R>& W, const RayWeights& V, int j, bool resume,
-                                           PieceState<R>& S)
+__device__ __forceinline__ void walk_piece(const TraceArgs& A, const float4* rec, Walk<R>& W, const RayWeights& V,
+                                           int j, bool resume, PieceState<R>& S)
 {
     using OT = unsigned long long;
     constexpr bool PLANES = ADDR == kAddrPlanes;
@@ -177,9 +177,9 @@ __device__ __forceinline__ void walk_piece(const TraceArgs& A, Walk<R>& W, const
     const R eps_end = L * eps_rel;
     const int max_iter = W.max_iter;
     auto fetch = [&](long long i) -> PR {
-        if constexpr (MA) return load_grad_rec(A.rec, i);
-        else if constexpr (GEN) return __ldg(reinterpret_cast<const float2*>(A.rec) + i);
-        else return load_rec(A.rec, i);
+        if constexpr (MA) return load_grad_rec(rec, i);
+        else if constexpr (GEN) return __ldg(reinterpret_cast<const float2*>(rec) + i);
+        else return load_rec(rec, i);
     };
     // (the channel pair the walk integrates) of a record
     auto pair = [&](const PR& r) -> float2 {
@@ -594,14 +594,14 @@ __device__ __forceinline__ void walk_flat(const TraceArgs& A, const Walk<float>&
 // sets the walk up again, so that nothing of the caller's loop outlives the
 // call in registers but what PieceState holds.
 template <int FORM>
-__device__ __noinline__ void index_piece(const TraceArgs& A, long long rid, float bh, float bl, float Lj, float D0j,
+__device__ __noinline__ void index_piece(const TraceArgs& A, const float4* rec, long long rid, float bh, float bl, float Lj, float D0j,
                                          int j, bool resume, PieceState<float>& S)
 {
     RayWeights V;
     ray_weights<FORM>(A, rid, V);
     Walk<float> W;
     walk_setup<float>(A, rid, bh, bl, Lj, D0j, 0.0, 0.0, W);
-    walk_piece<RR_TRILINEAR, float, FORM, kAddrIndex>(A, W, V, j, resume, S);
+    walk_piece<RR_TRILINEAR, float, FORM, kAddrIndex>(A, rec, W, V, j, resume, S);
 }
 
 // Whether a multi-step kernel sets a ray's constants up once, outside its loop
@@ -614,9 +614,11 @@ template <int FORM, int ADDR>
 constexpr bool kHoist = ADDR == kAddrFlat && (FORM == kFormKahan || FORM == kFormShear);
 
 // PER: periodic bundles only. REGACC: one of several steps of a launch; acc and
-// W0 (the ray's constants) live across them.
+// W0 (the ray's constants) live across them. A0: the kernel's own arguments (A,
+// but for the step's fields in a multi-step kernel), whose address the
+// out-of-line path takes.
 template <int INTERP, class R, int FORM, int ADDR, bool PER, bool REGACC = false>
-__device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, RayAcc* acc = nullptr,
+__device__ __forceinline__ void trace_ray(const TraceArgs& A, const TraceArgs& A0, int ix, int iy, RayAcc* acc = nullptr,
                                           const Walk<R>* W0 = nullptr)
 {
     static_assert(!REGACC || (FORM != kFormPlain && sizeof(R) == 4), "register accumulators: FP32 compensated forms");
@@ -712,12 +714,12 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, int ix, int iy, Ra
                 Q.qa = S.qa; Q.ga = S.ga;
                 Q.qb = S.qb; Q.gb = S.gb;
             }
-            index_piece<FORM>(A, rid, bh, bl, Lj, D0j, j, resume, Q);
+            index_piece<FORM>(A0, A.rec, rid, bh, bl, Lj, D0j, j, resume, Q);
             S = Q;
         }
     } else {
         if constexpr (FLAT) walk_flat<FORM, FORM == kFormKahan || FORM == kFormPlain || FORM == kFormMoments>(A, W, V, j == 0, j + 1 < nsub, resume, fB, fd, S);
-        else walk_piece<INTERP, R, FORM, ADDR>(A, W, V, j, resume, S);
+        else walk_piece<INTERP, R, FORM, ADDR>(A, A.rec, W, V, j, resume, S);
     }
     }
 
@@ -796,7 +798,7 @@ __global__ void __launch_bounds__(NT_MAX, 2) trace_kernel(const __grid_constant_
     prefetch_ahead(A, t);
     int ix, iy;
     tile_ray(t, blockIdx.x, blockIdx.y, ix, iy);
-    if (ix < A.nx && iy < A.ny) trace_ray<INTERP, R, FORM, ADDR, PER>(A, ix, iy);
+    if (ix < A.nx && iy < A.ny) trace_ray<INTERP, R, FORM, ADDR, PER>(A, A, ix, iy);
 }
 
 // Consecutive steps of one bundle in one launch (the default FP32 form): each
@@ -808,7 +810,7 @@ __global__ void __launch_bounds__(NT_MAX, 2) trace_kernel(const __grid_constant_
 // accumulators) and all launches but one.
 template <int INTERP, int ADDR, int FORM, bool PER>
 __global__ void __launch_bounds__(NT_MAX, 2)
-    trace_steps_kernel(const TraceArgs A, const __grid_constant__ StepBlock S, const TileCfg t)
+    trace_steps_kernel(const __grid_constant__ TraceArgs A, const __grid_constant__ StepBlock S, const TileCfg t)
 {
     prefetch_ahead(A, t);
     int ix, iy;
@@ -831,7 +833,7 @@ __global__ void __launch_bounds__(NT_MAX, 2)
         As.fo[0] = st.fo[0]; As.fo[1] = st.fo[1]; As.fo[2] = st.fo[2];
         As.fe[0] = st.fe[0]; As.fe[1] = st.fe[1]; As.fe[2] = st.fe[2];
         As.fs0 = st.fs0; As.fs1 = st.fs1;
-        trace_ray<INTERP, float, FORM, ADDR, PER, true>(As, ix, iy, &acc, &W0);
+        trace_ray<INTERP, float, FORM, ADDR, PER, true>(As, A, ix, iy, &acc, &W0);
     }
     if (acc.loaded) {
         const long long rid = (long long)iy * A.nx + ix;
@@ -890,7 +892,7 @@ __global__ void __launch_bounds__(NT_MAX, 2) trace_batch_kernel(const BatchArgs 
             const int ntx = B.tiles_x[cone];
             int ix, iy;
             tile_ray(B.tile, local % ntx, local / ntx, ix, iy);
-            if (ix < sA.nx && iy < sA.ny) trace_ray<INTERP, R, kFormKahan, ADDR, PER>(sA, ix, iy);
+            if (ix < sA.nx && iy < sA.ny) trace_ray<INTERP, R, kFormKahan, ADDR, PER>(sA, sA, ix, iy);
             __syncthreads();
         }
     }
@@ -975,10 +977,12 @@ template <int FORM>
 static cudaError_t launch_steps_form(const TraceArgs& a, const StepBlock& b, int interp, bool flat, dim3 grid, int nt,
                               const TileCfg& t, cudaStream_t s)
 {
-    // trilinear: steps that all take the flat addressing (periodic); NGP: any
+    // trilinear: steps that all take the flat addressing (periodic), or choose
+    // it per sub-step; NGP: any
     if (interp == RR_TRILINEAR) {
-        if (!flat || !a.periodic) return cudaErrorInvalidValue;
-        trace_steps_kernel<RR_TRILINEAR, kAddrFlat, FORM, true><<<grid, nt, 0, s>>>(a, b, t);
+        if (flat && a.periodic) trace_steps_kernel<RR_TRILINEAR, kAddrFlat, FORM, true><<<grid, nt, 0, s>>>(a, b, t);
+        else if (a.periodic) trace_steps_kernel<RR_TRILINEAR, kAddrAuto, FORM, true><<<grid, nt, 0, s>>>(a, b, t);
+        else trace_steps_kernel<RR_TRILINEAR, kAddrAuto, FORM, false><<<grid, nt, 0, s>>>(a, b, t);
     } else {
         constexpr int ADDR = FORM == kFormKahan ? kAddrPlanes : kAddrIndex;
         if (a.periodic) trace_steps_kernel<RR_NGP, ADDR, FORM, true><<<grid, nt, 0, s>>>(a, b, t);
