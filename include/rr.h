@@ -136,6 +136,13 @@ const char* rr_status_string(rr_status s);
 rr_status rr_create(const rr_bundle_desc* bundle, rr_ctx** out);
 
 /*
+ * The library keeps the memory of destroyed contexts for later ones (at most
+ * 1 GiB in at most 64 blocks per process; an allocation of its own that fails
+ * frees it first). rr_release_cached gives all of it back now.
+ */
+rr_status rr_release_cached(void);
+
+/*
  * A context for the rows [y0, y1) of `bundle` only: the rays of pixels
  * (i_x, i_y) with y0 <= i_y < y1, directions from Eq. (txty) with the whole
  * bundle's N_y, ids counted from row y0 (Eq. rayid restricted to the band).

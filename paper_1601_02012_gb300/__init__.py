@@ -18,13 +18,13 @@ from ._rr import rr_amr_create, rr_amr_destroy, rr_amr_sizes, rr_amr_tidal, rr_a
 from ._rr import RR_SHEAR, rr_shear  # noqa: E402
 from ._rr import RR_METHOD_A, rr_gradient_records  # noqa: E402
 from ._rr import RR_GENERIC, rr_scalar_records, rr_set_kernels, rr_set_observer  # noqa: E402
-from ._rr import rr_upload_box  # noqa: E402
+from ._rr import rr_release_cached, rr_upload_box  # noqa: E402
 
 __all__ = [
     "Batch", "AmrMesh", "source_kappa", "rr_amr_create", "rr_amr_destroy", "rr_amr_sizes", "rr_amr_tidal",
     "rr_amr_trace_step", "RR_SHEAR", "rr_shear", "RR_METHOD_A", "rr_gradient_records", "trace_method_a",
     "gradient_buffer", "RR_GENERIC", "rr_scalar_records", "rr_set_kernels", "rr_set_observer", "scalar_buffer",
-    "trace_tiles", "rr_upload_box",
+    "trace_tiles", "rr_upload_box", "rr_release_cached",
     "Tracer", "pipeline_steps", "box_record_buffer", "trace_kappa", "trace_shear", "record_buffer", "grad_buffer", "RRError", "rr_create", "rr_destroy", "rr_reset",
     "rr_tidal_tensor", "rr_footprint_bbox", "rr_trace_step", "rr_finalize", "rr_sync_status",
     "rr_segment_count", "rr_status_string", "rr_step_count", "rr_trace_step_adjoint", "rr_tidal_tensor_adjoint",

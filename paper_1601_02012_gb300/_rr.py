@@ -77,6 +77,7 @@ def load() -> C.CDLL:
             "rr_create": ([P, C.POINTER(C.c_void_p)], C.c_int),
             "rr_create_band": ([P, I32, I32, C.POINTER(C.c_void_p)], C.c_int),
             "rr_destroy": ([P], C.c_int),
+            "rr_release_cached": ([], C.c_int),
             "rr_reset": ([P, P], C.c_int),
             "rr_tidal_tensor": ([P, P, P, P, I32, P, P], C.c_int),
             "rr_footprint_bbox": ([P, P, D, D, P], C.c_int),
@@ -213,6 +214,11 @@ def rr_create_band(bundle: rr_bundle_desc, y0: int, y1: int) -> C.c_void_p:
 
 def rr_destroy(ctx) -> None:
     _check(load().rr_destroy(ctx), "rr_destroy")
+
+
+def rr_release_cached() -> None:
+    """Free the memory kept from destroyed contexts."""
+    _check(load().rr_release_cached(), "rr_release_cached")
 
 
 def rr_reset(ctx, stream=None) -> None:

@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cmath>
 #include <new>
+#include <type_traits>
 
 #include "rr_internal.h"
 
@@ -32,24 +33,6 @@ rr_status status_from_word(uint32_t w)
     if (w & kErrRange) return RR_ERR_RANGE;
     return RR_OK;
 }
-
-void free_state(RayState& s)
-{
-    cudaFree(s.dir);
-    cudaFree(s.dirh);
-    cudaFree(s.dirl);
-    cudaFree(s.kacc);
-    cudaFree(s.bacc);
-    cudaFree(s.kmom);
-    cudaFree(s.bmom);
-    cudaFree(s.g1acc);
-    cudaFree(s.g2acc);
-    cudaFree(s.nseg);
-    cudaFree(s.err);
-    cudaFree(s.total);
-    s = RayState{};
-}
-
 
 }  // namespace
 
@@ -193,6 +176,7 @@ rr_status validate_step(rr_ctx* ctx, const rr_grid_desc* grid, const float* rec,
 }
 
 rr_status status_of_cuda(cudaError_t e) { return from_cuda(e); }
+rr_status status_of_word(uint32_t w) { return status_from_word(w); }
 
 }  // namespace rr
 
@@ -287,42 +271,40 @@ static rr_status create_context(const rr_bundle_desc* bundle, int32_t y0, int32_
         ctx->kq[3 * c + 2] = -1.0 / bundle->chi_s;
     }
     cudaGetDevice(&ctx->device);
+    // one block for the whole state, each array 256-byte aligned
     const size_t nr = (size_t)bundle->nx * (size_t)(y1 - y0);
-    cudaError_t e = cudaSuccess;
     RayState& s = ctx->st;
-    if (e == cudaSuccess) e = cudaMalloc(&s.dir, 3 * nr * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&s.dirh, nr * sizeof(float4));
-    if (e == cudaSuccess) e = cudaMalloc(&s.dirl, nr * sizeof(float4));
-    if (e == cudaSuccess) e = cudaMalloc(&s.kacc, nr * sizeof(float2));
-    if (e == cudaSuccess) e = cudaMalloc(&s.bacc, nr * sizeof(float2));
-    if (e == cudaSuccess) e = cudaMalloc(&s.nseg, nr * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMalloc(&s.err, sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMalloc(&s.total, sizeof(unsigned long long));
-    if (e == cudaSuccess) e = cudaMallocHost(&ctx->host_err, sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMallocHost(&ctx->host_total, sizeof(unsigned long long));
-    if (e == cudaSuccess) e = cudaMemset(s.kacc, 0, nr * sizeof(float2));
-    if (e == cudaSuccess) e = cudaMemset(s.bacc, 0, nr * sizeof(float2));
-    if (bundle->flags & RR_SOURCE_MOMENTS) {
-        if (e == cudaSuccess) e = cudaMalloc(&s.kmom, nr * sizeof(float2));
-        if (e == cudaSuccess) e = cudaMalloc(&s.bmom, nr * sizeof(float2));
-        if (e == cudaSuccess) e = cudaMemset(s.kmom, 0, nr * sizeof(float2));
-        if (e == cudaSuccess) e = cudaMemset(s.bmom, 0, nr * sizeof(float2));
+    const bool f64 = (bundle->flags & RR_FP64_DDA) || !(bundle->flags & RR_PERIODIC);
+    const bool mom = bundle->flags & RR_SOURCE_MOMENTS, shear = bundle->flags & RR_SHEAR;
+    size_t bytes = 0;
+    auto room = [&](bool have, size_t n) {
+        const size_t at = bytes;
+        if (have) bytes += (n + 255) / 256 * 256;
+        return have ? at : (size_t)-1;
+    };
+    const size_t dir = room(f64, 3 * nr * sizeof(double)), dirh = room(true, nr * sizeof(float4));
+    const size_t dirl = room(true, nr * sizeof(float4)), kacc = room(true, nr * sizeof(float2));
+    const size_t bacc = room(true, nr * sizeof(float2)), kmom = room(mom, nr * sizeof(float2));
+    const size_t bmom = room(mom, nr * sizeof(float2)), g1acc = room(shear, nr * sizeof(float2));
+    const size_t g2acc = room(shear, nr * sizeof(float2)), nseg = room(true, nr * sizeof(uint32_t));
+    const size_t err = room(true, sizeof(uint32_t)), words = room(true, sizeof(Words));
+    cudaError_t e = pool_take(bytes, &ctx->block);
+    if (e != cudaSuccess) {
+        delete ctx;
+        return from_cuda(e);
     }
-    if (bundle->flags & RR_SHEAR) {
-        if (e == cudaSuccess) e = cudaMalloc(&s.g1acc, nr * sizeof(float2));
-        if (e == cudaSuccess) e = cudaMalloc(&s.g2acc, nr * sizeof(float2));
-        if (e == cudaSuccess) e = cudaMemset(s.g1acc, 0, nr * sizeof(float2));
-        if (e == cudaSuccess) e = cudaMemset(s.g2acc, 0, nr * sizeof(float2));
-    }
-    if (e == cudaSuccess) e = cudaMemset(s.nseg, 0, nr * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMemset(s.err, 0, sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMemset(s.total, 0, sizeof(unsigned long long));
-    if (e == cudaSuccess) e = launch_init_directions(*bundle, s.dir, s.dirh, s.dirl, 0, y0, y1 - y0);
+    auto put = [&](auto*& p, size_t at) {
+        using T = std::remove_reference_t<decltype(p)>;
+        p = at == (size_t)-1 ? nullptr : reinterpret_cast<T>(static_cast<char*>(ctx->block.dev) + at);
+    };
+    put(s.dir, dir); put(s.dirh, dirh); put(s.dirl, dirl);
+    put(s.kacc, kacc); put(s.bacc, bacc); put(s.kmom, kmom); put(s.bmom, bmom);
+    put(s.g1acc, g1acc); put(s.g2acc, g2acc);
+    put(s.nseg, nseg); put(s.err, err); put(s.words, words);
+    e = launch_init_state(*bundle, s, 0, y0, y1 - y0);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
-        free_state(s);
-        if (ctx->host_err) cudaFreeHost(ctx->host_err);
-        if (ctx->host_total) cudaFreeHost(ctx->host_total);
+        pool_give(ctx->block, false);
         delete ctx;
         return from_cuda(e);
     }
@@ -343,10 +325,13 @@ rr_status rr_create_band(const rr_bundle_desc* bundle, int32_t y0, int32_t y1, r
 rr_status rr_destroy(rr_ctx* ctx)
 {
     if (!ctx) return RR_ERR_ARG;
-    cudaDeviceSynchronize();
-    free_state(ctx->st);
-    cudaFreeHost(ctx->host_err);
-    cudaFreeHost(ctx->host_total);
+    // (the device the state lives on, which need not be the current one)
+    int dev = ctx->device;
+    cudaGetDevice(&dev);
+    if (dev != ctx->device) cudaSetDevice(ctx->device);
+    const bool idle = cudaDeviceSynchronize() == cudaSuccess;
+    pool_give(ctx->block, idle);
+    if (dev != ctx->device) cudaSetDevice(dev);
     delete ctx;
     return RR_OK;
 }
@@ -354,16 +339,8 @@ rr_status rr_destroy(rr_ctx* ctx)
 rr_status rr_reset(rr_ctx* ctx, void* stream)
 {
     if (!ctx) return RR_ERR_ARG;
-    cudaStream_t s = (cudaStream_t)stream;
-    const size_t nr = (size_t)ctx->bundle.nx * ctx->bundle.ny;
-    cudaError_t e = cudaMemsetAsync(ctx->st.kacc, 0, nr * sizeof(float2), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->st.bacc, 0, nr * sizeof(float2), s);
-    if (e == cudaSuccess && ctx->st.kmom) e = cudaMemsetAsync(ctx->st.kmom, 0, nr * sizeof(float2), s);
-    if (e == cudaSuccess && ctx->st.bmom) e = cudaMemsetAsync(ctx->st.bmom, 0, nr * sizeof(float2), s);
-    if (e == cudaSuccess && ctx->st.g1acc) e = cudaMemsetAsync(ctx->st.g1acc, 0, nr * sizeof(float2), s);
-    if (e == cudaSuccess && ctx->st.g2acc) e = cudaMemsetAsync(ctx->st.g2acc, 0, nr * sizeof(float2), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->st.nseg, 0, nr * sizeof(uint32_t), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->st.err, 0, sizeof(uint32_t), s);
+    const cudaError_t e = launch_clear_state(ClearItem{ctx->st, (long long)ctx->bundle.nx * ctx->bundle.ny},
+                                             (cudaStream_t)stream);
     ctx->log.clear();
     ctx->last_total = 0;
     return from_cuda(e);
@@ -701,10 +678,10 @@ rr_status rr_sync_status(rr_ctx* ctx, void* stream)
 {
     if (!ctx) return RR_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = cudaMemcpyAsync(ctx->host_err, ctx->st.err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+    cudaError_t e = cudaMemcpyAsync(&ctx->block.host->err, ctx->st.err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return from_cuda(e);
-    return status_from_word(*ctx->host_err);
+    return status_from_word(ctx->block.host->err);
 }
 
 rr_status rr_finalize(rr_ctx* ctx, double* kappa, double* kappa_born, void* stream)
@@ -712,15 +689,13 @@ rr_status rr_finalize(rr_ctx* ctx, double* kappa, double* kappa_born, void* stre
     if (!ctx || !kappa) return RR_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     const int nr = ctx->bundle.nx * ctx->bundle.ny;
-    cudaError_t e = launch_finalize(nr, ctx->st.kacc, ctx->st.bacc, ctx->st.nseg, kappa, kappa_born,
-                                    ctx->st.total, s, ctx->st.kmom, ctx->st.bmom, ctx->bundle.chi_s,
+    // (the kernel hands the segment total and the error word to the host)
+    cudaError_t e = launch_finalize(nr, ctx->st, kappa, kappa_born, ctx->block.host, s, ctx->bundle.chi_s,
                                     (ctx->bundle.flags & RR_METHOD_A) != 0);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(ctx->host_total, ctx->st.total, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return from_cuda(e);
-    rr_status st = rr_sync_status(ctx, stream);
-    ctx->last_total = *ctx->host_total;
-    return st;
+    ctx->last_total = ctx->block.host->total;
+    return status_from_word(ctx->block.host->err);
 }
 
 rr_status rr_segment_count(rr_ctx* ctx, uint64_t* total, uint32_t* per_ray, void* stream)

@@ -34,6 +34,8 @@ struct rr_batch {
     TraceArgs* d_args = nullptr;
     int* d_tiles = nullptr;
     int* d_counter = nullptr;
+    ClearItem* d_items = nullptr;   // every bundle's state
+    HostWords* h_words = nullptr;   // pinned: totals and error words
     int total_tiles = 0;
 };
 
@@ -48,6 +50,8 @@ void free_batch(rr_batch* b)
     cudaFree(b->d_args);
     cudaFree(b->d_tiles);
     cudaFree(b->d_counter);
+    cudaFree(b->d_items);
+    cudaFreeHost(b->h_words);
     delete b;
 }
 
@@ -111,6 +115,16 @@ rr_status rr_batch_create(int32_t n, const rr_bundle_desc* bundles, rr_batch** o
     if (e == cudaSuccess) e = cudaMalloc(&b->d_args, sizeof(TraceArgs) * (size_t)n);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_tiles, sizeof(int) * (size_t)(2 * n + 1));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_counter, sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_items, sizeof(ClearItem) * (size_t)n);
+    if (e == cudaSuccess) e = cudaMallocHost(&b->h_words, sizeof(HostWords) * (size_t)n);
+    if (e == cudaSuccess) {
+        std::vector<ClearItem> items((size_t)n);
+        for (int i = 0; i < n; ++i) {
+            const rr_ctx* c = b->cones[(size_t)i];
+            items[(size_t)i] = ClearItem{c->st, (long long)c->bundle.nx * c->bundle.ny};
+        }
+        e = cudaMemcpy(b->d_items, items.data(), sizeof(ClearItem) * (size_t)n, cudaMemcpyHostToDevice);
+    }
     if (e != cudaSuccess) {
         free_batch(b);
         return status_of_cuda(e);
@@ -146,27 +160,19 @@ rr_status rr_batch_context(rr_batch* b, int32_t i, rr_ctx** ctx)
 rr_status rr_batch_reset(rr_batch* b, void* stream)
 {
     if (!b) return RR_ERR_ARG;
+    // rr_reset of every bundle, in one launch
     for (size_t i = 0; i < b->cones.size(); ++i) {
-        rr_status st = rr_reset(b->cones[i], stream);
-        if (st != RR_OK) return st;
+        b->cones[i]->log.clear();
+        b->cones[i]->last_total = 0;
         b->staged[i] = false;
     }
-    return RR_OK;
+    return rr_batch_clear(b, stream);
 }
 
 rr_status rr_batch_clear(rr_batch* b, void* stream)
 {
     if (!b) return RR_ERR_ARG;
-    cudaStream_t s = (cudaStream_t)stream;
-    for (rr_ctx* c : b->cones) {
-        const size_t nr = (size_t)c->bundle.nx * c->bundle.ny;
-        cudaError_t e = cudaMemsetAsync(c->st.kacc, 0, nr * sizeof(float2), s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->st.bacc, 0, nr * sizeof(float2), s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->st.nseg, 0, nr * sizeof(uint32_t), s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->st.err, 0, sizeof(uint32_t), s);
-        if (e != cudaSuccess) return status_of_cuda(e);
-    }
-    return RR_OK;
+    return status_of_cuda(launch_clear_states(b->d_items, (int)b->cones.size(), (cudaStream_t)stream));
 }
 
 rr_status rr_batch_set_step(rr_batch* b, int32_t i, const rr_grid_desc* grid, const float* rec, double chi_a,
@@ -223,8 +229,7 @@ rr_status rr_batch_finalize(rr_batch* b, double* const* kappa, double* const* ka
         rr_ctx* c = b->cones[i];
         if (!kappa[i]) return RR_ERR_ARG;
         const int nr = c->bundle.nx * c->bundle.ny;
-        cudaError_t e = launch_finalize(nr, c->st.kacc, c->st.bacc, c->st.nseg, kappa[i],
-                                        kappa_born ? kappa_born[i] : nullptr, c->st.total, s);
+        cudaError_t e = launch_finalize(nr, c->st, kappa[i], kappa_born ? kappa_born[i] : nullptr, nullptr, s);
         if (e != cudaSuccess) return status_of_cuda(e);
     }
     return RR_OK;
@@ -233,15 +238,17 @@ rr_status rr_batch_finalize(rr_batch* b, double* const* kappa, double* const* ka
 rr_status rr_batch_sync_status(rr_batch* b, uint64_t* total_segments, void* stream)
 {
     if (!b) return RR_ERR_ARG;
+    // every bundle's total and error word in one launch and one synchronisation
+    cudaStream_t s = (cudaStream_t)stream;
+    cudaError_t e = launch_collect_words(b->d_items, (int)b->cones.size(), b->h_words, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return status_of_cuda(e);
     rr_status worst = RR_OK;
     uint64_t tot = 0;
-    for (rr_ctx* c : b->cones) {
-        cudaError_t e = cudaMemcpyAsync(c->host_total, c->st.total, sizeof(unsigned long long),
-                                        cudaMemcpyDeviceToHost, (cudaStream_t)stream);
-        if (e != cudaSuccess) return status_of_cuda(e);
-        rr_status st = rr_sync_status(c, stream);
-        c->last_total = *c->host_total;
-        tot += c->last_total;
+    for (size_t i = 0; i < b->cones.size(); ++i) {
+        const rr_status st = status_of_word(b->h_words[i].err);
+        b->cones[i]->last_total = b->h_words[i].total;
+        tot += b->h_words[i].total;
         if (st != RR_OK && worst == RR_OK) worst = st;
     }
     if (total_segments) *total_segments = tot;

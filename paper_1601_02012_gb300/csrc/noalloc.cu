@@ -93,7 +93,7 @@ extern "C" rr_status rr_trace_step_noalloc(const rr_bundle_desc* bundle, const r
     cudaStream_t s = (cudaStream_t)stream;
     const size_t nr = (size_t)bundle->nx * bundle->ny;
     uint32_t* err = reinterpret_cast<uint32_t*>(base + kOffErr);
-    unsigned long long* total = reinterpret_cast<unsigned long long*>(base + kOffTotal);
+    Words* words = reinterpret_cast<Words*>(base + kOffTotal);
     double* dir = reinterpret_cast<double*>(base + kOffDir);
     float4* dirh = reinterpret_cast<float4*>(base + kOffDirh);
     float4* dirl = reinterpret_cast<float4*>(base + kOffDirl);
@@ -101,14 +101,8 @@ extern "C" rr_status rr_trace_step_noalloc(const rr_bundle_desc* bundle, const r
     float2* bacc = reinterpret_cast<float2*>(base + kOffBacc);
     uint32_t* nseg = reinterpret_cast<uint32_t*>(base + kOffNseg);
 
-    // The array keeps the previous call's contents: clear what accumulates.
-    e = cudaMemsetAsync(err, 0, sizeof(uint32_t), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(kacc, 0, nr * sizeof(float2), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(bacc, 0, nr * sizeof(float2), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(nseg, 0, nr * sizeof(uint32_t), s);
-    if (e == cudaSuccess) e = launch_init_directions(*bundle, dir, dirh, dirl, s);
-    if (e != cudaSuccess) return to_status(e);
-
+    // The array keeps the previous call's contents: what accumulates is cleared
+    // with the directions.
     RayState rs;
     rs.dir = dir;
     rs.dirh = dirh;
@@ -117,10 +111,12 @@ extern "C" rr_status rr_trace_step_noalloc(const rr_bundle_desc* bundle, const r
     rs.bacc = bacc;
     rs.nseg = nseg;
     rs.err = err;
-    rs.total = total;
+    rs.words = words;
+    e = launch_init_state(*bundle, rs, s);
+    if (e != cudaSuccess) return to_status(e);
     const TraceArgs a = make_trace_args(*bundle, rs, grid, rec, chi_a, chi_b, scale, a_step, nullptr, nullptr);
     e = launch_trace(a, bundle->interp, (bundle->flags & RR_FP64_DDA) != 0, s);
-    if (e == cudaSuccess) e = launch_finalize((int)nr, kacc, bacc, nseg, kappa, kappa_born, total, s);
+    if (e == cudaSuccess) e = launch_finalize((int)nr, rs, kappa, kappa_born, nullptr, s);
     if (e != cudaSuccess) return to_status(e);
 
     uint32_t word = 0;

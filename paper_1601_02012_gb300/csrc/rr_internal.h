@@ -19,7 +19,7 @@ enum : uint32_t { kErrStepLimit = 1u, kErrNonFinite = 2u, kErrRange = 4u };
 
 // Per-ray state, structure of arrays, indexed by ray id (Eq. rayid).
 struct RayState {
-    double* dir = nullptr;      // 3 per ray: n_hat (Eq. raypos), FP64
+    double* dir = nullptr;      // 3 per ray: n_hat (Eq. raypos), FP64 (FP64 and bounded walks only)
     float4* dirh = nullptr;     // n_hat rounded to FP32 (x, y, z, 0)
     float4* dirl = nullptr;     // n_hat - dirh rounded to FP32 (float-float low parts)
     float2* kacc = nullptr;     // kappa accumulated across steps, float-float (hi, lo); A moment (moments form)
@@ -30,8 +30,34 @@ struct RayState {
     float2* g2acc = nullptr;    // shear form only: gamma2, float-float
     uint32_t* nseg = nullptr;   // non-empty segments since reset
     uint32_t* err = nullptr;    // device error word
-    unsigned long long* total = nullptr;  // segment total written by finalize
+    struct Words* words = nullptr;   // segment total written by finalize
 };
+
+// finalize's words on the device: the total of the last call, and the running
+// sum and block count of the current one (both 0 between calls).
+struct Words {
+    unsigned long long total, sum;
+    unsigned int done;
+};
+
+// What finalize leaves for the host (pinned memory the kernel writes).
+struct HostWords {
+    unsigned long long total;
+    uint32_t err;
+};
+
+// One device allocation and one pinned HostWords, from a bounded process-wide
+// pool (pool.cu): a context's whole state.
+struct Block {
+    void* dev = nullptr;
+    size_t bytes = 0;
+    HostWords* host = nullptr;
+    int device = -1;
+};
+cudaError_t pool_take(size_t bytes, Block* out);
+// idle: the device has finished with the block (it may be kept); otherwise it is freed.
+void pool_give(const Block& b, bool idle);
+void pool_clear();
 
 struct StepRecord {
     rr_grid_desc grid;
@@ -139,9 +165,19 @@ struct BatchArgs {
 };
 
 // Launchers (one per translation unit).
-// Directions of the rows [row0, row0 + nrows) of bundle b (all rows: nrows < 0).
-cudaError_t launch_init_directions(const rr_bundle_desc& b, double* dir, float4* dirh, float4* dirl, cudaStream_t s,
-                                   int row0 = 0, int nrows = -1);
+// Directions of the rows [row0, row0 + nrows) of bundle b (all rows: nrows < 0)
+// and zeros in every accumulator, counter and word that st holds.
+cudaError_t launch_init_state(const rr_bundle_desc& b, const RayState& st, cudaStream_t s, int row0 = 0,
+                              int nrows = -1);
+// Zeros in the accumulators, counters and error words of n ray states (a device table).
+struct ClearItem {
+    RayState st;
+    long long nrays;
+};
+cudaError_t launch_clear_states(const ClearItem* items, int n, cudaStream_t s);
+cudaError_t launch_clear_state(const ClearItem& item, cudaStream_t s);
+// The totals and error words of n ray states (a device table) into pinned host memory.
+cudaError_t launch_collect_words(const ClearItem* items, int n, HostWords* out, cudaStream_t s);
 // kind 0: tidal records (2 float4 per point); kind 1: gradient records (1 float4)
 // compact (with a bbox): the records stored box-local, point (i, j, k) of the
 // box at (i ey + j) ez + k
@@ -184,10 +220,9 @@ cudaError_t launch_tidal_adjoint(const rr_grid_desc& g, const float* grad_rec, i
 // per axis (unwrapped point indices; an axis whose extent reaches n is whole).
 cudaError_t zero_grad_records(const rr_grid_desc& g, float* grad_rec, const long long* box0, const long long* box1,
                               cudaStream_t s);
-cudaError_t launch_finalize(int nrays, const float2* kacc, const float2* bacc, const uint32_t* nseg,
-                            double* out_kappa, double* out_kborn, unsigned long long* total, cudaStream_t s,
-                            const float2* kmom = nullptr, const float2* bmom = nullptr, double chi_s = 0.0,
-                            bool add_born = false);
+// (host: receives the segment total and the error word when the kernel has run)
+cudaError_t launch_finalize(int nrays, const RayState& st, double* out_kappa, double* out_kborn, HostWords* host,
+                            cudaStream_t s, double chi_s = 0.0, bool add_born = false);
 cudaError_t launch_moments(int nrays, const float2* kacc, const float2* kmom, const float2* bacc, const float2* bmom,
                            double* out, cudaStream_t s);
 cudaError_t launch_shear_out(int nrays, const float2* g1acc, const float2* g2acc, double* gamma1, double* gamma2,
@@ -229,6 +264,7 @@ StepRecord make_step_record(const rr_ctx* ctx, const rr_grid_desc* grid, double 
 rr_status validate_step(rr_ctx* ctx, const rr_grid_desc* grid, const float* rec, double chi_a, double chi_b,
                         double scale, double a_step);
 rr_status status_of_cuda(cudaError_t e);
+rr_status status_of_word(uint32_t w);
 
 // hi = (float)x, lo = (float)(x - hi)
 inline void split_ff(double x, float& hi, float& lo)
@@ -250,8 +286,7 @@ struct rr_ctx {
     int device = 0;
     std::vector<rr::StepRecord> log;
     unsigned long long last_total = 0;
-    uint32_t* host_err = nullptr;             // pinned
-    unsigned long long* host_total = nullptr; // pinned
+    rr::Block block;                          // everything st points into, and the pinned words
     bool relocated = false;                   // observer moved since the last step: no continuity check
     double kq[6] = {0, 1, 0, 0, 1, 0};        // generic form kernels (set at create and by rr_set_kernels)
 };
