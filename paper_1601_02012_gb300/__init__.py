@@ -437,40 +437,96 @@ def pipeline_steps(n, records, trace, stream, side=None, nbuf=1, timing=None):
         used[i].record(stream)
 
 
+#: Points that one record launch costs over what its points cost: a launch over
+#: one step's footprint takes about 4.5 us whatever its size, the time in which
+#: the record kernel writes half a million points (whole grids: 5 TB/s).
+_LAUNCH_POINTS = 500_000
+
+
+def _union(boxes, n):
+    """The box that holds all the (unwrapped) boxes, an axis that it covers whole as [0, n)."""
+    out = []
+    for a in range(3):
+        lo, hi = min(b[2 * a] for b in boxes), max(b[2 * a + 1] for b in boxes)
+        out += [0, n[a]] if hi - lo >= n[a] else [lo, hi]
+    return tuple(out)
+
+
+def _points(box):
+    return (box[1] - box[0]) * (box[3] - box[2]) * (box[5] - box[4])
+
+
+def _cheaper(one, boxes):
+    """Whether one launch over the box ``one`` costs less than a launch per box of ``boxes``."""
+    return _points(one) <= sum(_points(bb) for bb in boxes) + (len(boxes) - 1) * _LAUNCH_POINTS
+
+
+def _trace_pass(tr, grid, phi, steps, delta=None, footprint=True, stream=None, group=16):
+    """The steps of a pass on one potential, through ``tr``.
+
+    The potential is the same in every step, so a point's record is too: the
+    records of the box that holds several steps' footprints are computed by one
+    launch and each of these steps reads them, unless that box holds so many
+    more points than the footprints together that a launch per step costs less.
+    Periodic trilinear bundles in the FP32 walk keep such boxes alone, one per
+    ``group`` steps (box-local: no wrap in the walk); the other forms, and cones
+    that reach around the box, write into a whole grid's buffer. ``group`` steps
+    are traced per launch (16 at most); group=1: one rr_trace_step per step on
+    whole-grid records."""
+    steps = list(steps)
+    if not steps:
+        return
+    n = [int(v) for v in grid.n]
+    interp, flags = int(tr.desc.interp), int(tr.desc.flags)
+    boxed = group > 1 and footprint and not (tr.method_a or tr.generic) and interp == RR_TRILINEAR and \
+        (flags & _rr.RR_PERIODIC) and not (flags & _rr.RR_FP64_DDA)
+    if boxed:
+        boxes = [tr.footprint(grid, st.chi_a, st.chi_b, pad=1) for st in steps]
+        boxed = all(bb[2 * a + 1] - bb[2 * a] < n[a] for bb in boxes for a in range(3))
+    if boxed:
+        for i in range(0, len(steps), group):
+            bbs = boxes[i:i + group]
+            one = _union(bbs, n)
+            if all(one[2 * a + 1] - one[2 * a] < n[a] for a in range(3)) and _points(one) < 2 ** 31 and _cheaper(one, bbs):
+                rec = box_record_buffer(one, device=phi.device)
+                tr.tidal_box(grid, phi, rec, one, delta=delta, stream=stream)
+                bbs, recs = [one] * len(bbs), [rec] * len(bbs)
+            else:
+                recs = [box_record_buffer(bb, device=phi.device) for bb in bbs]
+                for bb, rec in zip(bbs, recs):
+                    tr.tidal_box(grid, phi, rec, bb, delta=delta, stream=stream)
+            tr.steps(grid, recs, steps[i:i + group], boxes=bbs, stream=stream)
+        return
+    rec = tr.record_buffer(grid, device=phi.device)
+    boxes = [tr.footprint(grid, st.chi_a, st.chi_b) for st in steps] if footprint else [None]
+    if footprint and len(boxes) > 1:
+        one = _union(boxes, n)
+        if _cheaper(one, boxes):
+            boxes = [one]
+    for bb in boxes:
+        tr.tidal(grid, phi, rec, delta=delta, bbox=bb, stream=stream)
+    if group > 1:
+        for i in range(0, len(steps), group):
+            tr.steps(grid, [rec] * len(steps[i:i + group]), steps[i:i + group], stream=stream)
+    else:
+        for st in steps:
+            tr.step(grid, rec, st.chi_a, st.chi_b, st.scale, st.a, stream=stream)
+
+
 def trace_kappa(phi, grid, bundle, steps, delta=None, fp64_dda=False, footprint=True, stream=None, group=16):
     """Trace a bundle through a sequence of steps on one potential.
 
     phi: device float32 tensor n0 x n1 x n2 (Phi/c^2 at cell centres).
     steps: objects with chi_a, chi_b, scale, a (the step's field is scale * Phi).
-    For each step the records are recomputed (restricted to the step's
-    footprint when ``footprint``) and the bundle is advanced; returns the FP64
-    (kappa, kappa_born) maps and the number of cell segments. For a periodic
-    trilinear bundle in the FP32 walk whose steps' footprints (widened by a
-    point) are smaller than the grid, each step's records are computed over
-    its footprint box only (box-local) and ``group`` steps are traced per
-    launch (rr_trace_steps; the same maps bit for bit); group=1: one
-    rr_trace_step per step on whole-grid records.
+    The records are computed over the steps' footprints (over the whole grid
+    without ``footprint``) and the bundle is advanced, ``group`` steps per
+    launch (the same maps bit for bit for every group; group=1: one
+    rr_trace_step per step on whole-grid records); returns the FP64 (kappa,
+    kappa_born) maps and the number of cell segments.
     """
     tr = Tracer(bundle, fp64_dda=fp64_dda)
     try:
-        boxes = None
-        if group > 1 and footprint and not fp64_dda and int(bundle.interp) == RR_TRILINEAR and \
-                (int(tr.desc.flags) & _rr.RR_PERIODIC):
-            boxes = [tr.footprint(grid, st.chi_a, st.chi_b, pad=1) for st in steps]
-            if any(bb[2 * a + 1] - bb[2 * a] >= int(grid.n[a]) for bb in boxes for a in range(3)):
-                boxes = None
-        if boxes is not None:
-            recs = [box_record_buffer(bb, device=phi.device) for bb in boxes]
-            for i in range(0, len(steps), group):
-                for k in range(i, min(i + group, len(steps))):
-                    tr.tidal_box(grid, phi, recs[k], boxes[k], delta=delta, stream=stream)
-                tr.steps(grid, recs[i:i + group], steps[i:i + group], boxes=boxes[i:i + group], stream=stream)
-        else:
-            rec = record_buffer(grid, device=phi.device)
-            for st in steps:
-                bbox = tr.footprint(grid, st.chi_a, st.chi_b) if footprint else None
-                tr.tidal(grid, phi, rec, delta=delta, bbox=bbox, stream=stream)
-                tr.step(grid, rec, st.chi_a, st.chi_b, st.scale, st.a, stream=stream)
+        _trace_pass(tr, grid, phi, steps, delta, footprint, stream, group)
         k, kb = tr.finalize(stream=stream)
         return k, kb, tr.segments()
     finally:
@@ -484,11 +540,7 @@ def trace_method_a(phi, grid, bundle, steps, delta=None, footprint=True, stream=
     kappa_born is the density term alone."""
     tr = Tracer(bundle, method_a=True)
     try:
-        rec = tr.record_buffer(grid, device=phi.device)
-        for st in steps:
-            bbox = tr.footprint(grid, st.chi_a, st.chi_b) if footprint else None
-            tr.tidal(grid, phi, rec, delta=delta, bbox=bbox, stream=stream)
-            tr.step(grid, rec, st.chi_a, st.chi_b, st.scale, st.a, stream=stream)
+        _trace_pass(tr, grid, phi, steps, delta, footprint, stream)
         k, kb = tr.finalize(stream=stream)
         return k, kb, tr.segments()
     finally:
@@ -508,12 +560,8 @@ def trace_tiles(tiles, bundle, steps, footprint=True, stream=None):
     tr = Tracer(b)
     try:
         for phi, grid, obs in tiles:
-            rec = record_buffer(grid, device=phi.device)
             tr.set_observer(obs)
-            for st in steps:
-                bbox = tr.footprint(grid, st.chi_a, st.chi_b) if footprint else None
-                tr.tidal(grid, phi, rec, bbox=bbox, stream=stream)
-                tr.step(grid, rec, st.chi_a, st.chi_b, st.scale, st.a, stream=stream)
+            _trace_pass(tr, grid, phi, steps, None, footprint, stream)
         k, kb = tr.finalize(stream=stream)
         return k, kb, tr.segments()
     finally:
@@ -526,11 +574,7 @@ def trace_shear(phi, grid, bundle, steps, delta=None, footprint=True, stream=Non
     each [ny, nx], and the number of cell segments."""
     tr = Tracer(bundle, shear=True)
     try:
-        rec = record_buffer(grid, device=phi.device)
-        for st in steps:
-            bbox = tr.footprint(grid, st.chi_a, st.chi_b) if footprint else None
-            tr.tidal(grid, phi, rec, delta=delta, bbox=bbox, stream=stream)
-            tr.step(grid, rec, st.chi_a, st.chi_b, st.scale, st.a, stream=stream)
+        _trace_pass(tr, grid, phi, steps, delta, footprint, stream)
         k, kb = tr.finalize(stream=stream)
         g1, g2 = tr.shear(stream=stream)
         return k, kb, g1, g2, tr.segments()
@@ -544,7 +588,7 @@ def _make_autograd():
     class TraceKappa(torch.autograd.Function):
         """(kappa, kappa_born) = trace(phi) as a differentiable torch op.
 
-        forward: rr_tidal_tensor + rr_trace_step per step + rr_finalize;
+        forward: the records, rr_trace_steps and rr_finalize;
         backward: rr_trace_backward (the hand-written adjoint), giving dL/dPhi
         for the FP32 potential. The maps are FP64, shaped [ny, nx].
         """
@@ -552,11 +596,7 @@ def _make_autograd():
         @staticmethod
         def forward(ctx, phi, grid, bundle, steps, footprint=True):
             tr = Tracer(bundle)
-            rec = record_buffer(grid, device=phi.device)
-            for st in steps:
-                bbox = tr.footprint(grid, st.chi_a, st.chi_b) if footprint else None
-                tr.tidal(grid, phi.detach().contiguous(), rec, bbox=bbox)
-                tr.step(grid, rec, st.chi_a, st.chi_b, st.scale, st.a)
+            _trace_pass(tr, grid, phi.detach().contiguous(), steps, footprint=footprint)
             k, kb = tr.finalize()
             ctx.tracer = tr
             ctx.grid = grid

@@ -77,18 +77,14 @@ def trace_kappa_sharded(phi, grid, bundle, steps, rank: int, world: int, group=N
     passes the same potential and steps, traces its band and returns the
     whole (kappa, kappa_born) maps and the whole bundle's segment count."""
     import torch
-    from . import Tracer, record_buffer
+    from . import Tracer, _trace_pass
     y0, y1 = band_rows(int(bundle.ny), rank, world)
     nx = int(bundle.nx)
     segs = 0
     if y1 > y0:
         tr = Tracer(bundle, rows=(y0, y1))
         try:
-            rec = record_buffer(grid, device=phi.device)
-            for st in steps:
-                bbox = tr.footprint(grid, st.chi_a, st.chi_b) if footprint else None
-                tr.tidal(grid, phi, rec, bbox=bbox, stream=stream)
-                tr.step(grid, rec, st.chi_a, st.chi_b, st.scale, st.a, stream=stream)
+            _trace_pass(tr, grid, phi, steps, footprint=footprint, stream=stream)
             k, kb = tr.finalize(stream=stream)
             segs = tr.segments()
         finally:
@@ -115,16 +111,12 @@ def _make_autograd():
 
         @staticmethod
         def forward(ctx, phi, grid, bundle, steps, rank, world, group=None, footprint=True):
-            from . import Tracer, record_buffer
+            from . import Tracer, _trace_pass
             y0, y1 = band_rows(int(bundle.ny), rank, world)
             tr = None
             if y1 > y0:
                 tr = Tracer(bundle, rows=(y0, y1))
-                rec = record_buffer(grid, device=phi.device)
-                for st in steps:
-                    bbox = tr.footprint(grid, st.chi_a, st.chi_b) if footprint else None
-                    tr.tidal(grid, phi.detach().contiguous(), rec, bbox=bbox)
-                    tr.step(grid, rec, st.chi_a, st.chi_b, st.scale, st.a)
+                _trace_pass(tr, grid, phi.detach().contiguous(), steps, footprint=footprint)
                 k, kb = tr.finalize()
             else:
                 k = torch.empty((0, int(bundle.nx)), dtype=torch.float64, device=phi.device)
