@@ -64,9 +64,13 @@ __device__ __forceinline__ void trace_ray_amr(const TraceArgs& A, const AmrDevic
     constexpr bool GEN = FORM == kFormGeneric;
     // AHEAD: advance to the next cell before integrating the current one and
     // load its coarse link then, so that the load overlaps the segment's
-    // arithmetic (faster for the shear and Method A walks, whose segments
-    // carry more arithmetic; slower for the default and generic ones)
-    constexpr bool AHEAD = SH || MA;
+    // arithmetic (four steps of 1024^2 rays over 128^3 and four levels, default
+    // form: 1292 -> 1229 us; slower for the generic one)
+    constexpr bool AHEAD = !GEN;
+    // WIDE: a corner's record in one 32-byte load (with AHEAD 1229 -> 1160 us:
+    // nothing spills; 3 % slower without it). The records of Method A and of the
+    // generic form need only be 16-byte aligned.
+    constexpr bool WIDE = FORM == kFormKahan;
     const long long rid = (long long)iy * A.nx + ix;
     const int NF = A.n0;   // finest cells per side
     RayRange rg;
@@ -206,11 +210,7 @@ __device__ __forceinline__ void trace_ray_amr(const TraceArgs& A, const AmrDevic
                     const float4* r = A.rec + 16 * (long long)leaf;
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {
-                        // (two 16-byte loads: one 32-byte load per corner measured 3 % slower here)
-                        const int rc = c ^ flip;
-                        Rec x;
-                        x.a = __ldg(r + 2 * rc);
-                        x.b = __ldg(r + 2 * rc + 1);
+                        const Rec x = WIDE ? load_rec32(r, c ^ flip) : load_rec(r, c ^ flip);
                         q2[c] = MA ? radial_pair(nd, x.a) : make_float2(project(W.w, x), x.b.z);
                         if constexpr (MA) q2[c].y = x.b.z;
                         if constexpr (GEN) q2[c] = make_float2(x.a.x, x.a.y);
