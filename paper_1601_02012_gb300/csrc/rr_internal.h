@@ -146,6 +146,7 @@ struct AdjArgs {
     double* grad;
     double kscale;              // the step's scale
     double bscale;              // scale * 1.5 Omega_m (H0/c)^2 / a_step
+    int first = 0;              // first sub-step of the launch
 };
 
 // Ray-tile shape: a warp covers wx x (32/wx) pixels, a block bwx x bwy warps.
