@@ -112,14 +112,15 @@ constexpr float kSliver = 4.76837158203125e-07f;
 //  kAddrAuto:   kAddrFlat for the sub-steps whose own cells and vertex planes
 //               lie inside the grid without a wrap (counted exactly as the walk
 //               will cross them, so a ray that ends on the box face z = 0 still
-//               qualifies), kAddrIndex out of line for the others. Whole-grid
-//               records of steps the host cannot clear: steps that reach the
-//               observer on the box face, bounded boxes, batches. Grids of
-//               fewer than 2^31 points. (One step of 1024^2 rays through 256
-//               cells down to z = 0: 3.13 ms by vertex planes, 2.55 ms; a batch
-//               of 16 cones 12.30 ms by vertex indices, 9.87 ms. With both
-//               loops inlined the rare one's registers spill into the common
-//               one: 10.5 ms; with one loop that branches per crossing 12.4 ms.)
+//               qualifies), up to the first that does not; the ray's rest out
+//               of line, its outside sub-steps by kAddrIndex. Whole-grid records
+//               of steps the host cannot clear: steps that reach the observer
+//               on the box face, bounded boxes, batches. Grids of fewer than
+//               2^31 points. (One step of 1024^2 rays through 256 cells down to
+//               z = 0: 3.13 ms by vertex planes, 2.35 ms; a batch of 16 cones
+//               12.30 ms by vertex indices, 9.20 ms. With both loops in one
+//               function, or a call inside the sub-steps' loop, the rare path's
+//               registers spill into the common one: 2.45 to 2.68 ms.)
 //  kAddrFlat:   no wrap: a 32-bit point index B of the mirrored cell's entry
 //               corner and a constant signed stride d_a per axis (the next
 //               vertex plane along the motion), so the 8 corners are B plus
@@ -486,20 +487,21 @@ __device__ __forceinline__ void add_segment(const TraceArgs& A, const Walk<float
 // loop on the last segment and on the cap alike. Bound by issue slots (FMA pipes
 // 58 % and ALU 47 % busy at 75 % issue); production pass, trace kernels 22.62 ->
 // 21.52 ms without the last segment in the loop, 20.83 ms with one test.
-// (B: point index of the entry corner, fd: index step per axis along the
-// motion; more: another sub-step follows)
-template <int FORM, bool SELECT>
-__device__ __forceinline__ void walk_flat(const TraceArgs& A, const Walk<float>& W, const RayWeights& V, bool first,
-                                          bool more, bool resume, int B, const int fd[3], PieceState<float>& S)
+// (B, D0, fd, SEAM: flat_start's; more: another sub-step follows; WIDE: a record in one 32-byte load)
+template <int FORM, bool SELECT, bool SEAM, bool WIDE = true>
+__device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec, const Walk<float>& W, const RayWeights& V, bool first,
+                                          bool more, bool resume, int B, const int D0[3], const int fd[3],
+                                          PieceState<float>& S)
 {
     constexpr bool SH = FORM == kFormShear;
     constexpr bool MA = FORM == kFormMethodA;
     constexpr bool GEN = FORM == kFormGeneric;
     using PR = typename std::conditional<MA, float4, typename std::conditional<GEN, float2, Rec>::type>::type;
     auto fetch = [&](int i) -> PR {
-        if constexpr (MA) return load_grad_rec(A.rec, (unsigned)i);
-        else if constexpr (GEN) return __ldg(reinterpret_cast<const float2*>(A.rec) + (unsigned)i);
-        else return load_rec32(A.rec, (unsigned)i);
+        if constexpr (MA) return load_grad_rec(rec, (unsigned)i);
+        else if constexpr (GEN) return __ldg(reinterpret_cast<const float2*>(rec) + (unsigned)i);
+        else if constexpr (WIDE) return load_rec32(rec, (unsigned)i);
+        else return load_rec(rec, (unsigned)i);
     };
     auto pair = [&](const PR& r) -> float2 {
         if constexpr (MA) return radial_pair(V.nd, r);
@@ -509,13 +511,14 @@ __device__ __forceinline__ void walk_flat(const TraceArgs& A, const Walk<float>&
     float2 q[8], g[SH ? 8 : 1];
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
-        const PR r = fetch(B + ((m & 1) ? fd[0] : 0) + ((m & 2) ? fd[1] : 0) + ((m & 4) ? fd[2] : 0));
+        const PR r = fetch(B + ((m & 1) ? D0[0] : 0) + ((m & 2) ? D0[1] : 0) + ((m & 4) ? D0[2] : 0));
         q[m] = pair(r);
         if constexpr (SH) g[m] = make_float2(project(V.w1, r), project(V.w2, r));
     }
     float sig = 0.f;                          // path from the sub-step start to the segment entry
     float T[3] = {W.T0[0], W.T0[1], W.T0[2]};   // path to the next face crossing per axis
     float kf[3] = {0.f, 0.f, 0.f};            // crossings so far
+    int D[3] = {D0[0], D0[1], D0[2]};         // entry to exit side of the cell (fd but for SEAM)
     const float lim = W.L - W.L * kSliver;
     int left = W.max_iter + 1;
     // (a resumed first segment is not a new one; it is integrated unless the
@@ -541,16 +544,23 @@ __device__ __forceinline__ void walk_flat(const TraceArgs& A, const Walk<float>&
         --left;
         const bool e0 = !e2 && !p1, e1 = !e2 && p1;
         // the new exit-side corners, loaded ahead of this segment's arithmetic:
-        // B + 2 d_e plus 0, d_A, d_B, d_A + d_B over the other two axes A < B
+        // the plane beyond the exit side along e, plus 0, d_A, d_B, d_A + d_B over
+        // the other two axes A < B
         const int fde = e2 ? fd[2] : (p1 ? fd[1] : fd[0]);
-        const int P = B + 2 * fde;
-        const int dA = e0 ? fd[1] : fd[0];
-        const int dB = e2 ? fd[1] : fd[2];
+        const int de = SEAM ? (e2 ? D[2] : (p1 ? D[1] : D[0])) : fde;
+        const int P = B + de + fde;
+        const int dA = e0 ? D[1] : D[0];
+        const int dB = e2 ? D[1] : D[2];
         const PR r[4] = {fetch(P), fetch(P + dA), fetch(P + dB), fetch(P + dA + dB)};
         add_segment<FORM, SELECT>(A, W, q, g, T, sig, tend, S);
         // cross the exit face
         sig = tend;
-        B += fde;
+        B += de;
+        if constexpr (SEAM) {
+            if (e0) D[0] = fd[0];
+            if (e1) D[1] = fd[1];
+            if (e2) D[2] = fd[2];
+        }
         if (e0) { kf[0] += 1.f; T[0] = fmaf(kf[0], W.td[0], W.T0[0]); }
         if (e1) { kf[1] += 1.f; T[1] = fmaf(kf[1], W.td[1], W.T0[1]); }
         if (e2) { kf[2] += 1.f; T[2] = fmaf(kf[2], W.td[2], W.T0[2]); }
@@ -590,18 +600,85 @@ __device__ __forceinline__ void walk_flat(const TraceArgs& A, const Walk<float>&
     }
 }
 
-// A sub-step by wrapped vertex indices, out of line: kAddrAuto's rare path. It
-// sets the walk up again, so that nothing of the caller's loop outlives the
-// call in registers but what PieceState holds.
-template <int FORM>
-__device__ __noinline__ void index_piece(const TraceArgs& A, const float4* rec, long long rid, float bh, float bl, float Lj, float D0j,
-                                         int j, bool resume, PieceState<float>& S)
+// The flat walk's start: the point index B of the sub-step's entry corner, the
+// index step D per axis to the first cell's exit side and fd from plane to plane
+// along the motion; whether every vertex plane the sub-step can read lies inside
+// the records' box. SEAM (the whole grid's records): crossings are counted as
+// the walk will make them, not two more than the path allows, and the entry side
+// of the first cell may be the periodic image of plane 0 (a ray that comes in
+// through the far face): D is then not fd.
+template <bool SEAM>
+__device__ __forceinline__ bool flat_start(const TraceArgs& A, const Walk<float>& W, int& B, int D[3], int fd[3])
 {
+    const int nn[3] = {A.n0, A.n1, A.n2};
+    bool inside = true;
+    B = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        // box-local vertex and cell coordinates (the records' box starts at fo,
+        // periodically)
+        const int sa = a == 0 ? A.fs0 : (a == 1 ? A.fs1 : 1);
+        int vl = W.vlo[a] - A.fo[a];
+        if (vl < 0) vl += nn[a];
+        int cl = W.c[a] - A.fo[a];
+        if (cl < 0) cl += nn[a];
+        B += vl * sa;
+        fd[a] = W.sgn[a] * sa;
+        D[a] = SEAM ? (W.vhi[a] - W.vlo[a]) * sa : fd[a];
+        // crossings this sub-step can make on axis a; cells c .. c + sgn K,
+        // vertex planes one further
+        int K = 0;
+        if (W.T0[a] < W.L) {
+            const float x = (W.L - W.T0[a]) * W.v[a];
+            if (x < 4194304.f) K = f2i_exact(x) + 2;
+            else inside = false;
+            if constexpr (SEAM) {
+                // the walk crosses face k (k = 0, 1, ...) on this axis while
+                // T_k = T0 + k td < L - eps_end, and T_k never decreases with k:
+                // drop the margin that the walk's own test rules out
+                const float lim = W.L - W.L * kSliver;
+#pragma unroll
+                for (int r = 0; r < 3; ++r)
+                    if (K > 0 && !(fmaf((float)(K - 1), W.td[a], W.T0[a]) < lim)) --K;
+            }
+        }
+        const int lo = W.sgn[a] > 0 ? cl : cl - K, hi = W.sgn[a] > 0 ? cl + K + 1 : (SEAM ? cl : cl + 1);
+        if (lo < 0 || hi > A.fe[a] - 1) inside = false;
+    }
+    return inside;
+}
+
+// A sub-step that resumes inside the previous one's last cell does not start a
+// new cell segment.
+template <class R>
+__device__ __forceinline__ bool resumes(const Walk<R>& W, const PieceState<R>& S, int j)
+{
+    return j > 0 && W.c[0] == S.pc0 && W.c[1] == S.pc1 && W.c[2] == S.pc2;
+}
+
+// The sub-steps j .. nsub - 1 of a ray from the first that does not lie inside
+// the grid, out of line (kAddrAuto): those inside by flat offsets, the others by
+// wrapped vertex indices. It sets the walk up from the ray's interval alone and
+// the caller has left its loop, so that the common path keeps no register for it.
+template <int FORM>
+__device__ __noinline__ void finish_ray(const TraceArgs& A, const float4* rec, long long rid, float ch, float cl,
+                                        float Lf, float D0f, int j, int nsub, float dsub, PieceState<float>& state)
+{
+    const RayRange rg{ch, cl, Lf, D0f, 0.0, 0.0};
+    PieceState<float> S = state;
     RayWeights V;
     ray_weights<FORM>(A, rid, V);
-    Walk<float> W;
-    walk_setup<float>(A, rid, bh, bl, Lj, D0j, 0.0, 0.0, W);
-    walk_piece<RR_TRILINEAR, float, FORM, kAddrIndex>(A, rec, W, V, j, resume, S);
+    for (; j < nsub && !S.overflow; ++j) {
+        float bh, bl, Lj, D0j;
+        sub_step(rg, j, nsub, dsub, bh, bl, Lj, D0j);
+        Walk<float> W;
+        walk_setup<float>(A, rid, bh, bl, Lj, D0j, 0.0, 0.0, W);
+        int B, D[3], fd[3];
+        const bool inside = flat_start<true>(A, W, B, D, fd), resume = resumes(W, S, j);
+        if (inside) walk_flat<FORM, false, true, false>(A, rec, W, V, j == 0, j + 1 < nsub, resume, B, D, fd, S);
+        else walk_piece<RR_TRILINEAR, float, FORM, kAddrIndex>(A, rec, W, V, j, resume, S);
+    }
+    state = S;
 }
 
 // Whether a multi-step kernel sets a ray's constants up once, outside its loop
@@ -615,8 +692,8 @@ constexpr bool kHoist = ADDR == kAddrFlat && (FORM == kFormKahan || FORM == kFor
 
 // PER: periodic bundles only. REGACC: one of several steps of a launch; acc and
 // W0 (the ray's constants) live across them. A0: the kernel's own arguments (A,
-// but for the step's fields in a multi-step kernel), whose address the
-// out-of-line path takes.
+// but for the step's fields in a multi-step kernel), whose address finish_ray
+// takes.
 template <int INTERP, class R, int FORM, int ADDR, bool PER, bool REGACC = false>
 __device__ __forceinline__ void trace_ray(const TraceArgs& A, const TraceArgs& A0, int ix, int iy, RayAcc* acc = nullptr,
                                           const Walk<R>* W0 = nullptr)
@@ -629,7 +706,6 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, const TraceArgs& A
     constexpr bool SH = !F64 && FORM == kFormShear;
     constexpr bool MA = !F64 && FORM == kFormMethodA;
     const long long rid = (long long)iy * A.nx + ix;
-    const int nn[3] = {A.n0, A.n1, A.n2};
     RayRange rg;
     if (!ray_range<PER>(A, rid, rg)) return;
     if (!REGACC || !acc->loaded) {
@@ -651,76 +727,30 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, const TraceArgs& A
     Walk<R> W;
     if constexpr (HOIST) W = *W0;
     PieceState<R> S;
+    int rest = -1;   // AUTO: the first sub-step that does not lie inside
     for (int j = 0; j < nsub && !S.overflow; ++j) {
     float bh, bl, Lj, D0j;
     sub_step(rg, j, nsub, dsub, bh, bl, Lj, D0j);
     walk_setup<R, false, !HOIST>(A, rid, bh, bl, Lj, D0j, rg.hi, rg.lo, W);
-    // FLAT: entry corner B, strides d
-    int fB = 0, fd[3] = {0, 0, 0};
-    bool inside = true;
     if constexpr (FLAT) {
-        const int* c = W.c;
-        const int* sgn = W.sgn;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            // box-local vertex and cell coordinates (the records' box starts
-            // at fo, periodically)
-            const int sa = a == 0 ? A.fs0 : (a == 1 ? A.fs1 : 1);
-            int vl = W.vlo[a] - A.fo[a];
-            if (vl < 0) vl += nn[a];
-            int cl = c[a] - A.fo[a];
-            if (cl < 0) cl += nn[a];
-            fB += vl * sa;
-            fd[a] = sgn[a] * sa;
-            // crossings this sub-step can make on axis a (2 more than the path
-            // allows, for rounding); cells c .. c + sgn K, vertex planes one further
-            int K = 0;
-            if (W.T0[a] < W.L) {
-                const float x = (W.L - W.T0[a]) * W.v[a];
-                if (x < 4194304.f) K = f2i_exact(x) + 2;
-                else inside = false;
-                if constexpr (AUTO) {
-                    // the walk crosses face k (k = 0, 1, ...) on this axis while
-                    // T_k = T0 + k td < L - eps_end, and T_k never decreases with
-                    // k: drop the margin that the walk's own test rules out
-                    const float lim = W.L - W.L * kSliver;
-#pragma unroll
-                    for (int r = 0; r < 3; ++r)
-                        if (K > 0 && !(fmaf((float)(K - 1), W.td[a], W.T0[a]) < lim)) --K;
-                }
-            }
-            const int lo = sgn[a] > 0 ? cl : cl - K, hi = sgn[a] > 0 ? cl + K + 1 : cl + 1;
-            if (lo < 0 || hi > A.fe[a] - 1) inside = false;
-        }
-        if (!AUTO && !inside) {
-            atomicOr(A.err, kErrRange);
+        int B, D[3], fd[3];
+        if (!flat_start<AUTO>(A, W, B, D, fd)) {
+            if constexpr (AUTO) rest = j;
+            else atomicOr(A.err, kErrRange);
             break;
         }
+        constexpr bool SELECT = !AUTO && (FORM == kFormKahan || FORM == kFormPlain || FORM == kFormMoments);
+        walk_flat<FORM, SELECT, AUTO>(A, A.rec, W, V, j == 0, j + 1 < nsub, resumes(W, S, j), B, D, fd, S);
+    } else {
+        walk_piece<INTERP, R, FORM, ADDR>(A, A.rec, W, V, j, resumes(W, S, j), S);
     }
-    // a sub-step that resumes inside the previous one's last cell does not
-    // start a new cell segment
-    const bool resume = j > 0 && W.c[0] == S.pc0 && W.c[1] == S.pc1 && W.c[2] == S.pc2;
+    }
     if constexpr (AUTO) {
-        if (inside) {
-            walk_flat<FORM, false>(A, W, V, j == 0, j + 1 < nsub, resume, fB, fd, S);
-        } else {
-            // (only what the form carries: each further word costs the common
-            // path registers around the call)
-            PieceState<R> Q;
-            Q.s2 = S.s2;
-            Q.cnt = S.cnt;
-            if constexpr (SH || FORM == kFormMoments) Q.s2m = S.s2m;
-            if constexpr (MA) {
-                Q.qa = S.qa; Q.ga = S.ga;
-                Q.qb = S.qb; Q.gb = S.gb;
-            }
-            index_piece<FORM>(A0, A.rec, rid, bh, bl, Lj, D0j, j, resume, Q);
+        if (rest >= 0) {
+            PieceState<R> Q = S;
+            finish_ray<FORM>(A0, A.rec, rid, rg.ch, rg.cl, rg.Lf, rg.D0f, rest, nsub, dsub, Q);
             S = Q;
         }
-    } else {
-        if constexpr (FLAT) walk_flat<FORM, FORM == kFormKahan || FORM == kFormPlain || FORM == kFormMoments>(A, W, V, j == 0, j + 1 < nsub, resume, fB, fd, S);
-        else walk_piece<INTERP, R, FORM, ADDR>(A, A.rec, W, V, j, resume, S);
-    }
     }
 
     if constexpr (MA) {
