@@ -620,15 +620,15 @@ rr_status rr_trace_steps(rr_ctx* ctx, const rr_grid_desc* grid, int32_t nsteps, 
     cudaStream_t s = (cudaStream_t)stream;
     cudaError_t e = cudaSuccess;
     // blocks of up to kMaxStepBlock steps go to one launch each: steps that all
-    // take the flat addressing, or all choose it per sub-step (trilinear), or
-    // any (NGP); a step on a grid of 2^31 points is launched on its own
+    // take the flat addressing, or all choose it per sub-step (trilinear),
+    // as NGP steps do; a step on a grid of 2^31 points is launched on its own
     const bool small = a0.fe[0] > 0;
     int32_t i = 0;
     while (i < nsteps && e == cudaSuccess) {
         const bool tri = b.interp == RR_TRILINEAR;
         auto flat_at = [&](int32_t k) { return boxes || flat_ok(whole, b.obs, *grid, chi_a[k], chi_b[k]); };
         const bool flat = tri && flat_at(i);
-        if (tri && !flat && !small) {
+        if (!flat && !small) {
             const TraceArgs a = make_trace_args(ctx, grid, rec[i], chi_a[i], chi_b[i], scale[i], a_step[i]);
             e = launch_trace(a, b.interp, false, s, TileCfg{}, form, false);
             ++i;

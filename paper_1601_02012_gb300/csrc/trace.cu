@@ -434,65 +434,77 @@ __device__ __forceinline__ void walk_piece(const TraceArgs& A, const float4* rec
     S.pc0 = c[0]; S.pc1 = c[1]; S.pc2 = c[2];
 }
 
-// The contribution of one segment of the FP32 trilinear walk (path sig .. tend
-// of the sub-step, corner pairs q and, for the shear, g) to the step's sums;
+// The contribution of one segment of the FP32 walk (path sig .. tend of the
+// sub-step, corner pairs q and, for the shear, g; NGP: the cell's own pair) to
+// the step's sums;
 // slivers are skipped. SELECT: by selecting the old sums afterwards instead of
 // branching around the arithmetic (three control instructions a segment):
 // default form 21.52 -> 21.23 ms per production pass; the forms with more sums
 // or fewer registers to spare keep the branch.
-template <int FORM, bool SELECT>
-__device__ __forceinline__ void add_segment(const TraceArgs& A, const Walk<float>& W, const float2 q[8],
+template <int INTERP, int FORM, bool SELECT>
+__device__ __forceinline__ void add_segment(const TraceArgs& A, const Walk<float>& W, const float2* q,
                                             const float2* g, const float T[3], float sig, float tend,
                                             PieceState<float>& S)
 {
+    constexpr bool TRI = INTERP == RR_TRILINEAR;
     const float t = tend - sig;
     // mirrored entry point of this segment
     float u[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) u[a] = __saturatef(fmaf(sig - T[a], W.v[a], W.cu[a]));
+    for (int a = 0; a < 3; ++a) u[a] = TRI ? __saturatef(fmaf(sig - T[a], W.v[a], W.cu[a])) : 0.f;
     const bool live = t > tend * kSliver;
     if (!SELECT && !live) return;
     const PieceState<float> S0 = S;
     const float chis = (float)A.chi_s, ichis = A.inv_chi_s_f;
     float2 e[4];
-    line_cubic2(q, bc2(u[0]), bc2(u[1]), bc2(u[2]), bc2(W.v[0]), bc2(W.v[1]), bc2(W.v[2]), e);
+    if constexpr (TRI)
+        line_cubic2(q, bc2(u[0]), bc2(u[1]), bc2(u[2]), bc2(W.v[0]), bc2(W.v[1]), bc2(W.v[2]), e);
     const float chiA = W.chiA0 - sig;
     if constexpr (FORM == kFormMoments) {
-        S.s2.add(dot_kernel(e, t, chiA, -1.f, 0.f));
-        S.s2m.add(dot_kernel(e, t, chiA * chiA, -2.f * chiA, 1.f));
+        S.s2.add(TRI ? dot_kernel(e, t, chiA, -1.f, 0.f) : segment_ngp(q[0], t, chiA, -1.f, 0.f));
+        S.s2m.add(TRI ? dot_kernel(e, t, chiA * chiA, -2.f * chiA, 1.f)
+                      : segment_ngp(q[0], t, chiA * chiA, -2.f * chiA, 1.f));
     } else if constexpr (FORM == kFormGeneric) {
         // each channel's kernel about the entry point: K(chi_A - s) = K(chi_A) -
         // K'(chi_A) s + k2 s^2
         const float2 G0 = make_float2(fmaf(chiA, fmaf(chiA, A.kq[2], A.kq[1]), A.kq[0]),
                                       fmaf(chiA, fmaf(chiA, A.kq[5], A.kq[4]), A.kq[3]));
         const float2 G1 = make_float2(-fmaf(2.f * A.kq[2], chiA, A.kq[1]), -fmaf(2.f * A.kq[5], chiA, A.kq[4]));
-        S.s2.add(dot_kernel_pair(e, t, G0, G1, make_float2(A.kq[2], A.kq[5])));
+        const float2 G2 = make_float2(A.kq[2], A.kq[5]), tt = bc2(t);
+        if constexpr (TRI) S.s2.add(dot_kernel_pair(e, t, G0, G1, G2));
+        else
+            S.s2.add(__fmul2_rn(q[0], __fmul2_rn(tt, __ffma2_rn(tt, __ffma2_rn(tt, __fmul2_rn(G2, bc2(1.f / 3.f)),
+                                                                              __fmul2_rn(G1, bc2(0.5f))), G0))));
     } else {
         float G0, G1, G2;
         kernel_coeffs(t, sig, W.chiA0, W.D0, chis, ichis, G0, G1, G2);
-        const float2 x = FORM == kFormMethodA ? dot_kernel_a(e, t, G0, G1, G2) : dot_kernel(e, t, G0, G1, G2);
+        float2 x;
+        if constexpr (TRI) x = FORM == kFormMethodA ? dot_kernel_a(e, t, G0, G1, G2) : dot_kernel(e, t, G0, G1, G2);
+        else x = FORM == kFormMethodA ? segment_ngp_a(q[0], t, G0, G1, G2) : segment_ngp(q[0], t, G0, G1, G2);
         if constexpr (FORM == kFormPlain) S.s2.s = __fadd2_rn(S.s2.s, x);
         else S.s2.add(x);
         if constexpr (FORM == kFormShear)
-            S.s2m.add(segment_trilinear(g, u[0], u[1], u[2], W.v[0], W.v[1], W.v[2], t, G0, G1, G2));
+            S.s2m.add(TRI ? segment_trilinear(g, u[0], u[1], u[2], W.v[0], W.v[1], W.v[2], t, G0, G1, G2)
+                          : segment_ngp(g[0], t, G0, G1, G2));
     }
     ++S.cnt;
     if (SELECT && !live) S = S0;
 }
 
-// walk_piece with flat addressing (FP32 trilinear): the same segments with the
-// same arithmetic. The loop holds crossings only; the segment that ends the
+// walk_piece with flat addressing (FP32): the same segments with the same
+// arithmetic. The loop holds crossings only; the segment that ends the
 // sub-step follows it, once for the whole warp, without the loads, the
 // projections and the corner shift that a crossing needs, and one test ends the
 // loop on the last segment and on the cap alike. Bound by issue slots (FMA pipes
 // 58 % and ALU 47 % busy at 75 % issue); production pass, trace kernels 22.62 ->
 // 21.52 ms without the last segment in the loop, 20.83 ms with one test.
 // (B, D0, fd, SEAM: flat_start's; more: another sub-step follows; WIDE: a record in one 32-byte load)
-template <int FORM, bool SELECT, bool SEAM, bool WIDE = true>
+template <int INTERP, int FORM, bool SELECT, bool SEAM, bool WIDE = true>
 __device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec, const Walk<float>& W, const RayWeights& V, bool first,
                                           bool more, bool resume, int B, const int D0[3], const int fd[3],
                                           PieceState<float>& S)
 {
+    constexpr bool TRI = INTERP == RR_TRILINEAR;
     constexpr bool SH = FORM == kFormShear;
     constexpr bool MA = FORM == kFormMethodA;
     constexpr bool GEN = FORM == kFormGeneric;
@@ -508,9 +520,10 @@ __device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec,
         else if constexpr (GEN) return r;
         else return make_float2(project(W.w, r), r.b.z);
     };
-    float2 q[8], g[SH ? 8 : 1];
+    constexpr int NQ = TRI ? 8 : 1;   // corners, or the cell (B: its index)
+    float2 q[NQ], g[SH ? NQ : 1];
 #pragma unroll
-    for (int m = 0; m < 8; ++m) {
+    for (int m = 0; m < NQ; ++m) {
         const PR r = fetch(B + ((m & 1) ? D0[0] : 0) + ((m & 2) ? D0[1] : 0) + ((m & 4) ? D0[2] : 0));
         q[m] = pair(r);
         if constexpr (SH) g[m] = make_float2(project(V.w1, r), project(V.w2, r));
@@ -530,7 +543,8 @@ __device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec,
             float u[3];
 #pragma unroll
             for (int a = 0; a < 3; ++a) u[a] = __saturatef(fmaf(sig - T[a], W.v[a], W.cu[a]));
-            S.qa = trilinear_x(q, u[0], u[1], u[2]);
+            if constexpr (TRI) S.qa = trilinear_x(q, u[0], u[1], u[2]);
+            else S.qa = q[0].x;
             S.ga = W.D0 * W.chiA0 * A.inv_chi_s_f;
         }
     }
@@ -551,8 +565,16 @@ __device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec,
         const int P = B + de + fde;
         const int dA = e0 ? D[1] : D[0];
         const int dB = e2 ? D[1] : D[2];
-        const PR r[4] = {fetch(P), fetch(P + dA), fetch(P + dB), fetch(P + dA + dB)};
-        add_segment<FORM, SELECT>(A, W, q, g, T, sig, tend, S);
+        PR r[TRI ? 4 : 1];
+        if constexpr (TRI) {
+            r[0] = fetch(P);
+            r[1] = fetch(P + dA);
+            r[2] = fetch(P + dB);
+            r[3] = fetch(P + dA + dB);
+        } else {
+            r[0] = fetch(B + de);   // the next cell
+        }
+        add_segment<INTERP, FORM, SELECT>(A, W, q, g, T, sig, tend, S);
         // cross the exit face
         sig = tend;
         B += de;
@@ -564,14 +586,19 @@ __device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec,
         if (e0) { kf[0] += 1.f; T[0] = fmaf(kf[0], W.td[0], W.T0[0]); }
         if (e1) { kf[1] += 1.f; T[1] = fmaf(kf[1], W.td[1], W.T0[1]); }
         if (e2) { kf[2] += 1.f; T[2] = fmaf(kf[2], W.td[2], W.T0[2]); }
-        float2 p[4];
+        if constexpr (TRI) {
+            float2 p[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) p[i] = pair(r[i]);
-        shift_corners(q, p, e0, e1);
-        if constexpr (SH) {
+            for (int i = 0; i < 4; ++i) p[i] = pair(r[i]);
+            shift_corners(q, p, e0, e1);
+            if constexpr (SH) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) p[i] = make_float2(project(V.w1, r[i]), project(V.w2, r[i]));
-            shift_corners(g, p, e0, e1);
+                for (int i = 0; i < 4; ++i) p[i] = make_float2(project(V.w1, r[i]), project(V.w2, r[i]));
+                shift_corners(g, p, e0, e1);
+            }
+        } else {
+            q[0] = pair(r[0]);
+            if constexpr (SH) g[0] = make_float2(project(V.w1, r[0]), project(V.w2, r[0]));
         }
     }
     // (no crossing left: the cap ended the walk, or it ended on its last allowed one)
@@ -579,7 +606,7 @@ __device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec,
         S.overflow = true;
         return;
     }
-    add_segment<FORM, SELECT>(A, W, q, g, T, sig, W.L, S);
+    add_segment<INTERP, FORM, SELECT>(A, W, q, g, T, sig, W.L, S);
     if constexpr (MA) {
         // the surface term at the end of the interval (the last sub-step's stays)
         const float t = W.L - sig;
@@ -587,7 +614,8 @@ __device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec,
 #pragma unroll
         for (int a = 0; a < 3; ++a)
             u[a] = __saturatef(fmaf(t, W.v[a], __saturatef(fmaf(sig - T[a], W.v[a], W.cu[a]))));
-        S.qb = trilinear_x(q, u[0], u[1], u[2]);
+        if constexpr (TRI) S.qb = trilinear_x(q, u[0], u[1], u[2]);
+        else S.qb = q[0].x;
         float G0, G1, G2;
         kernel_coeffs(t, sig, W.chiA0, W.D0, (float)A.chi_s, A.inv_chi_s_f, G0, G1, G2);
         S.gb = fmaf(t, fmaf(t, G2, G1), G0);
@@ -606,8 +634,9 @@ __device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec,
 // the records' box. SEAM (the whole grid's records): crossings are counted as
 // the walk will make them, not two more than the path allows, and the entry side
 // of the first cell may be the periodic image of plane 0 (a ray that comes in
-// through the far face): D is then not fd.
-template <bool SEAM>
+// through the far face): D is then not fd. NGP: cells for vertices (B the cell's
+// index, D = fd).
+template <int INTERP, bool SEAM>
 __device__ __forceinline__ bool flat_start(const TraceArgs& A, const Walk<float>& W, int& B, int D[3], int fd[3])
 {
     const int nn[3] = {A.n0, A.n1, A.n2};
@@ -618,13 +647,13 @@ __device__ __forceinline__ bool flat_start(const TraceArgs& A, const Walk<float>
         // box-local vertex and cell coordinates (the records' box starts at fo,
         // periodically)
         const int sa = a == 0 ? A.fs0 : (a == 1 ? A.fs1 : 1);
-        int vl = W.vlo[a] - A.fo[a];
+        int vl = (INTERP == RR_TRILINEAR ? W.vlo[a] : W.c[a]) - A.fo[a];
         if (vl < 0) vl += nn[a];
         int cl = W.c[a] - A.fo[a];
         if (cl < 0) cl += nn[a];
         B += vl * sa;
         fd[a] = W.sgn[a] * sa;
-        D[a] = SEAM ? (W.vhi[a] - W.vlo[a]) * sa : fd[a];
+        D[a] = SEAM && INTERP == RR_TRILINEAR ? (W.vhi[a] - W.vlo[a]) * sa : fd[a];
         // crossings this sub-step can make on axis a; cells c .. c + sgn K,
         // vertex planes one further
         int K = 0;
@@ -642,7 +671,8 @@ __device__ __forceinline__ bool flat_start(const TraceArgs& A, const Walk<float>
                     if (K > 0 && !(fmaf((float)(K - 1), W.td[a], W.T0[a]) < lim)) --K;
             }
         }
-        const int lo = W.sgn[a] > 0 ? cl : cl - K, hi = W.sgn[a] > 0 ? cl + K + 1 : (SEAM ? cl : cl + 1);
+        constexpr int up = INTERP == RR_TRILINEAR ? 1 : 0;
+        const int lo = W.sgn[a] > 0 ? cl : cl - K, hi = W.sgn[a] > 0 ? cl + K + up : (SEAM ? cl : cl + 1);
         if (lo < 0 || hi > A.fe[a] - 1) inside = false;
     }
     return inside;
@@ -660,7 +690,7 @@ __device__ __forceinline__ bool resumes(const Walk<R>& W, const PieceState<R>& S
 // the grid, out of line (kAddrAuto): those inside by flat offsets, the others by
 // wrapped vertex indices. It sets the walk up from the ray's interval alone and
 // the caller has left its loop, so that the common path keeps no register for it.
-template <int FORM>
+template <int INTERP, int FORM>
 __device__ __noinline__ void finish_ray(const TraceArgs& A, const float4* rec, long long rid, float ch, float cl,
                                         float Lf, float D0f, int j, int nsub, float dsub, PieceState<float>& state)
 {
@@ -674,9 +704,9 @@ __device__ __noinline__ void finish_ray(const TraceArgs& A, const float4* rec, l
         Walk<float> W;
         walk_setup<float>(A, rid, bh, bl, Lj, D0j, 0.0, 0.0, W);
         int B, D[3], fd[3];
-        const bool inside = flat_start<true>(A, W, B, D, fd), resume = resumes(W, S, j);
-        if (inside) walk_flat<FORM, false, true, false>(A, rec, W, V, j == 0, j + 1 < nsub, resume, B, D, fd, S);
-        else walk_piece<RR_TRILINEAR, float, FORM, kAddrIndex>(A, rec, W, V, j, resume, S);
+        const bool inside = flat_start<INTERP, true>(A, W, B, D, fd), resume = resumes(W, S, j);
+        if (inside) walk_flat<INTERP, FORM, false, INTERP == RR_TRILINEAR, false>(A, rec, W, V, j == 0, j + 1 < nsub, resume, B, D, fd, S);
+        else walk_piece<INTERP, float, FORM, kAddrIndex>(A, rec, W, V, j, resume, S);
     }
     state = S;
 }
@@ -701,7 +731,7 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, const TraceArgs& A
     static_assert(!REGACC || (FORM != kFormPlain && sizeof(R) == 4), "register accumulators: FP32 compensated forms");
     constexpr bool AUTO = ADDR == kAddrAuto;
     constexpr bool FLAT = ADDR == kAddrFlat || AUTO;
-    static_assert(!FLAT || (INTERP == RR_TRILINEAR && sizeof(R) == 4), "flat addressing: FP32 trilinear walk");
+    static_assert(!FLAT || sizeof(R) == 4, "flat addressing: FP32 walk");
     constexpr bool F64 = sizeof(R) == 8;
     constexpr bool SH = !F64 && FORM == kFormShear;
     constexpr bool MA = !F64 && FORM == kFormMethodA;
@@ -734,13 +764,13 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, const TraceArgs& A
     walk_setup<R, false, !HOIST>(A, rid, bh, bl, Lj, D0j, rg.hi, rg.lo, W);
     if constexpr (FLAT) {
         int B, D[3], fd[3];
-        if (!flat_start<AUTO>(A, W, B, D, fd)) {
+        if (!flat_start<INTERP, AUTO>(A, W, B, D, fd)) {
             if constexpr (AUTO) rest = j;
             else atomicOr(A.err, kErrRange);
             break;
         }
         constexpr bool SELECT = !AUTO && (FORM == kFormKahan || FORM == kFormPlain || FORM == kFormMoments);
-        walk_flat<FORM, SELECT, AUTO>(A, A.rec, W, V, j == 0, j + 1 < nsub, resumes(W, S, j), B, D, fd, S);
+        walk_flat<INTERP, FORM, SELECT, AUTO && INTERP == RR_TRILINEAR>(A, A.rec, W, V, j == 0, j + 1 < nsub, resumes(W, S, j), B, D, fd, S);
     } else {
         walk_piece<INTERP, R, FORM, ADDR>(A, A.rec, W, V, j, resumes(W, S, j), S);
     }
@@ -748,7 +778,7 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, const TraceArgs& A
     if constexpr (AUTO) {
         if (rest >= 0) {
             PieceState<R> Q = S;
-            finish_ray<FORM>(A0, A.rec, rid, rg.ch, rg.cl, rg.Lf, rg.D0f, rest, nsub, dsub, Q);
+            finish_ray<INTERP, FORM>(A0, A.rec, rid, rg.ch, rg.cl, rg.Lf, rg.D0f, rest, nsub, dsub, Q);
             S = Q;
         }
     }
@@ -822,8 +852,15 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, const TraceArgs& A
 }
 
 
+// Blocks of NT_MAX threads per SM: the NGP walk's default sums need few
+// registers outside their rare path (256^3, 1024^2 rays, 20 steps: 1199 us with 2
+// blocks, 1072 with 3, 1012 with 4, at 64 registers); the trilinear ones spill
+// into their loop with more than 2.
+template <int INTERP, class R, int FORM>
+constexpr int kBlocks = INTERP == RR_NGP && sizeof(R) == 4 && (FORM == kFormKahan || FORM == kFormPlain) ? 4 : 2;
+
 template <int INTERP, class R, int FORM, int ADDR, bool PER>
-__global__ void __launch_bounds__(NT_MAX, 2) trace_kernel(const __grid_constant__ TraceArgs A, const TileCfg t)
+__global__ void __launch_bounds__(NT_MAX, kBlocks<INTERP, R, FORM>) trace_kernel(const __grid_constant__ TraceArgs A, const TileCfg t)
 {
     prefetch_ahead(A, t);
     int ix, iy;
@@ -839,7 +876,7 @@ __global__ void __launch_bounds__(NT_MAX, 2) trace_kernel(const __grid_constant_
 // is the per-launch and per-step traffic of the ray state (directions,
 // accumulators) and all launches but one.
 template <int INTERP, int ADDR, int FORM, bool PER>
-__global__ void __launch_bounds__(NT_MAX, 2)
+__global__ void __launch_bounds__(NT_MAX, kBlocks<INTERP, float, FORM>)
     trace_steps_kernel(const __grid_constant__ TraceArgs A, const __grid_constant__ StepBlock S, const TileCfg t)
 {
     prefetch_ahead(A, t);
@@ -886,7 +923,7 @@ __global__ void __launch_bounds__(NT_MAX, 2)
 // waiting), finds the bundle by binary search in the tile offsets, stages that
 // bundle's arguments in shared memory and traces the tile.
 template <int INTERP, class R, int ADDR, bool PER>
-__global__ void __launch_bounds__(NT_MAX, 2) trace_batch_kernel(const BatchArgs B)
+__global__ void __launch_bounds__(NT_MAX, kBlocks<INTERP, R, kFormKahan>) trace_batch_kernel(const BatchArgs B)
 {
     __shared__ TraceArgs sA;
     __shared__ int s_item, s_cone;
@@ -955,11 +992,12 @@ cudaError_t launch_addr(const TraceArgs& a, const dim3& grid, int nt, cudaStream
 template <int INTERP, class R, int FORM>
 cudaError_t launch_one(const TraceArgs& a, const dim3& grid, int nt, cudaStream_t s, const TileCfg& t)
 {
-    if constexpr (INTERP == RR_TRILINEAR && sizeof(R) == 4) {
+    if constexpr (sizeof(R) == 4) {
         // fewer than 2^31 points
         if (a.fe[0] > 0) return launch_addr<INTERP, R, FORM, kAddrAuto>(a, grid, nt, s, t);
     }
-    return launch_addr<INTERP, R, FORM, FORM == kFormKahan ? kAddrPlanes : kAddrIndex>(a, grid, nt, s, t);
+    return launch_addr<INTERP, R, FORM, FORM == kFormKahan && INTERP == RR_TRILINEAR ? kAddrPlanes : kAddrIndex>(
+        a, grid, nt, s, t);
 }
 
 template <int FORM>
@@ -1007,16 +1045,16 @@ template <int FORM>
 static cudaError_t launch_steps_form(const TraceArgs& a, const StepBlock& b, int interp, bool flat, dim3 grid, int nt,
                               const TileCfg& t, cudaStream_t s)
 {
-    // trilinear: steps that all take the flat addressing (periodic), or choose
-    // it per sub-step; NGP: any
+    // (grids of fewer than 2^31 points) trilinear: steps that all take the flat
+    // addressing (periodic), or choose it per sub-step, as NGP steps do
     if (interp == RR_TRILINEAR) {
         if (flat && a.periodic) trace_steps_kernel<RR_TRILINEAR, kAddrFlat, FORM, true><<<grid, nt, 0, s>>>(a, b, t);
         else if (a.periodic) trace_steps_kernel<RR_TRILINEAR, kAddrAuto, FORM, true><<<grid, nt, 0, s>>>(a, b, t);
         else trace_steps_kernel<RR_TRILINEAR, kAddrAuto, FORM, false><<<grid, nt, 0, s>>>(a, b, t);
     } else {
-        constexpr int ADDR = FORM == kFormKahan ? kAddrPlanes : kAddrIndex;
-        if (a.periodic) trace_steps_kernel<RR_NGP, ADDR, FORM, true><<<grid, nt, 0, s>>>(a, b, t);
-        else trace_steps_kernel<RR_NGP, ADDR, FORM, false><<<grid, nt, 0, s>>>(a, b, t);
+        if (a.fe[0] <= 0) return cudaErrorInvalidValue;
+        if (a.periodic) trace_steps_kernel<RR_NGP, kAddrAuto, FORM, true><<<grid, nt, 0, s>>>(a, b, t);
+        else trace_steps_kernel<RR_NGP, kAddrAuto, FORM, false><<<grid, nt, 0, s>>>(a, b, t);
     }
     return cudaGetLastError();
 }
@@ -1056,8 +1094,8 @@ BatchKernel batch_kernel_of(int interp, bool fp64_dda, bool small)
         return small ? trace_batch_kernel<RR_TRILINEAR, float, kAddrAuto, PER>
                      : trace_batch_kernel<RR_TRILINEAR, float, kAddrIndex, PER>;
     }
-    return fp64_dda ? trace_batch_kernel<RR_NGP, double, kAddrIndex, PER>
-                    : trace_batch_kernel<RR_NGP, float, kAddrIndex, PER>;
+    if (fp64_dda) return trace_batch_kernel<RR_NGP, double, kAddrIndex, PER>;
+    return small ? trace_batch_kernel<RR_NGP, float, kAddrAuto, PER> : trace_batch_kernel<RR_NGP, float, kAddrIndex, PER>;
 }
 
 BatchKernel batch_kernel(int interp, bool fp64_dda, bool small, bool periodic)

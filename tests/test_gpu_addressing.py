@@ -56,9 +56,11 @@ def _close(got, want):
 
 @pytest.mark.parametrize("name", sorted(CASES))
 @pytest.mark.parametrize("form", ["default", "shear", "method_a"])
-def test_against_oracle(rrp, oracle_lib, name, form):
+@pytest.mark.parametrize("interp", [1, 0])
+def test_against_oracle(rrp, oracle_lib, name, form, interp):
     import torch
     g, b, steps = _setup(name)
+    b.interp = interp
     phi = synth.random_field(g.n, 77, np.float32)
     H, d = oracle_lib.fields(g, phi.astype(np.float64))
     ph = torch.from_numpy(phi).cuda()
