@@ -55,6 +55,28 @@ __device__ __forceinline__ void shift_corners(float2 q[8], const float2 p[4], bo
     for (int i = 0; i < 8; ++i) q[i] = n[i];
 }
 
+// a shared-memory read that the compiler neither hoists nor merges
+__device__ __forceinline__ float4 lds_again(unsigned a)
+{
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+    return v;
+}
+
+// (gamma1, gamma2) of N records. The twelve weights are read again for each
+// crossing (three 16-byte reads) instead of holding registers through the
+// segment's arithmetic, where they spilled (228 -> 116 bytes; 256^3, 1024^2 rays,
+// 20 steps: 4.36 -> 4.21 ms).
+template <int N>
+__device__ __forceinline__ void shear_pairs(unsigned sw, const Rec* r, float2* g)
+{
+    const float4 a = lds_again(sw), b = lds_again(sw + 16 * NT_MAX), c = lds_again(sw + 32 * NT_MAX);
+    const float w1[6] = {a.x, a.y, a.z, a.w, b.x, b.y}, w2[6] = {b.z, b.w, c.x, c.y, c.z, c.w};
+#pragma unroll
+    for (int i = 0; i < N; ++i) g[i] = make_float2(project(w1, r[i]), project(w2, r[i]));
+}
+
 // What the sub-steps of one ray's step accumulate and hand on.
 template <class R>
 struct PieceState {
@@ -71,14 +93,22 @@ struct PieceState {
 
 // The form's own per-ray constants.
 struct RayWeights {
-    float w1[6], w2[6];   // shear form: the Q weights of gamma1, gamma2
+    unsigned sw;          // shear form: the Q weights of gamma1, gamma2 in shared memory
     float4 nd;            // Method A: the direction, for n . grad Phi
 };
 
 template <int FORM>
 __device__ __forceinline__ void ray_weights(const TraceArgs& A, long long rid, RayWeights& V)
 {
-    if constexpr (FORM == kFormShear) shear_weights(A.dirh[rid], V.w1, V.w2);
+    if constexpr (FORM == kFormShear) {
+        __shared__ float4 sw[3 * NT_MAX];
+        float w1[6], w2[6];
+        shear_weights(A.dirh[rid], w1, w2);
+        sw[threadIdx.x] = make_float4(w1[0], w1[1], w1[2], w1[3]);
+        sw[NT_MAX + threadIdx.x] = make_float4(w1[4], w1[5], w2[0], w2[1]);
+        sw[2 * NT_MAX + threadIdx.x] = make_float4(w2[2], w2[3], w2[4], w2[5]);
+        V.sw = (unsigned)__cvta_generic_to_shared(sw + threadIdx.x);
+    }
     if constexpr (FORM == kFormMethodA) V.nd = A.dirh[rid];
 }
 
@@ -210,12 +240,12 @@ __device__ __forceinline__ void walk_piece(const TraceArgs& A, const float4* rec
             }
             const PR r = fetch(o);
             q2[m] = pair(r);
-            if constexpr (SH) g2[m] = make_float2(project(V.w1, r), project(V.w2, r));
+            if constexpr (SH) shear_pairs<1>(V.sw, &r, &g2[m]);
         }
     } else {
         const PR r = fetch(c[0] * sx + c[1] * sy + c[2]);
         q2[0] = pair(r);
-        if constexpr (SH) g2[0] = make_float2(project(V.w1, r), project(V.w2, r));
+        if constexpr (SH) shear_pairs<1>(V.sw, &r, &g2[0]);
     }
 
     // (a resumed first segment is not a new one; it is integrated below unless
@@ -419,12 +449,12 @@ __device__ __forceinline__ void walk_piece(const TraceArgs& A, const float4* rec
             shift_corners(q2, p2, e == 0, e == 1);
             if constexpr (SH) {
 #pragma unroll
-                for (int r = 0; r < 4; ++r) p2[r] = make_float2(project(V.w1, nr[r]), project(V.w2, nr[r]));
+                for (int r = 0; r < 4; ++r) shear_pairs<1>(V.sw, &nr[r], &p2[r]);
                 shift_corners(g2, p2, e == 0, e == 1);
             }
         } else {
             q2[0] = pair(nr[0]);
-            if constexpr (SH) g2[0] = make_float2(project(V.w1, nr[0]), project(V.w2, nr[0]));
+            if constexpr (SH) shear_pairs<1>(V.sw, &nr[0], &g2[0]);
         }
         if (++iter > max_iter) {
             S.overflow = true;
@@ -497,7 +527,9 @@ __device__ __forceinline__ void add_segment(const TraceArgs& A, const Walk<float
 // projections and the corner shift that a crossing needs, and one test ends the
 // loop on the last segment and on the cap alike. Bound by issue slots (FMA pipes
 // 58 % and ALU 47 % busy at 75 % issue); production pass, trace kernels 22.62 ->
-// 21.52 ms without the last segment in the loop, 20.83 ms with one test.
+// 21.52 ms without the last segment in the loop, 20.83 ms with one test, 20.33 ms
+// with the ray's constants hoisted (kHoist), 19.72 ms with the new corners
+// projected before the crossing's bookkeeping.
 // (B, D0, fd, SEAM: flat_start's; more: another sub-step follows; WIDE: a record in one 32-byte load)
 template <int INTERP, int FORM, bool SELECT, bool SEAM, bool WIDE = true>
 __device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec, const Walk<float>& W, const RayWeights& V, bool first,
@@ -526,7 +558,7 @@ __device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec,
     for (int m = 0; m < NQ; ++m) {
         const PR r = fetch(B + ((m & 1) ? D0[0] : 0) + ((m & 2) ? D0[1] : 0) + ((m & 4) ? D0[2] : 0));
         q[m] = pair(r);
-        if constexpr (SH) g[m] = make_float2(project(V.w1, r), project(V.w2, r));
+        if constexpr (SH) shear_pairs<1>(V.sw, &r, &g[m]);
     }
     float sig = 0.f;                          // path from the sub-step start to the segment entry
     float T[3] = {W.T0[0], W.T0[1], W.T0[2]};   // path to the next face crossing per axis
@@ -551,9 +583,9 @@ __device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec,
     while (true) {
         // exit plane: the nearest face crossing (lowest axis on ties)
         const bool p1 = T[1] < T[0];
-        const float t01 = p1 ? T[1] : T[0];
+        const float t01 = fminf(T[1], T[0]);
         const bool e2 = T[2] < t01;
-        const float tend = e2 ? T[2] : t01;
+        const float tend = fminf(T[2], t01);
         if (!(tend < lim) | (left == 0)) break;
         --left;
         const bool e0 = !e2 && !p1, e1 = !e2 && p1;
@@ -575,6 +607,19 @@ __device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec,
             r[0] = fetch(B + de);   // the next cell
         }
         add_segment<INTERP, FORM, SELECT>(A, W, q, g, T, sig, tend, S);
+        if constexpr (TRI) {
+            float2 p[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) p[i] = pair(r[i]);
+            shift_corners(q, p, e0, e1);
+            if constexpr (SH) {
+                shear_pairs<4>(V.sw, r, p);
+                shift_corners(g, p, e0, e1);
+            }
+        } else {
+            q[0] = pair(r[0]);
+            if constexpr (SH) shear_pairs<1>(V.sw, &r[0], &g[0]);
+        }
         // cross the exit face
         sig = tend;
         B += de;
@@ -586,20 +631,6 @@ __device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec,
         if (e0) { kf[0] += 1.f; T[0] = fmaf(kf[0], W.td[0], W.T0[0]); }
         if (e1) { kf[1] += 1.f; T[1] = fmaf(kf[1], W.td[1], W.T0[1]); }
         if (e2) { kf[2] += 1.f; T[2] = fmaf(kf[2], W.td[2], W.T0[2]); }
-        if constexpr (TRI) {
-            float2 p[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) p[i] = pair(r[i]);
-            shift_corners(q, p, e0, e1);
-            if constexpr (SH) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) p[i] = make_float2(project(V.w1, r[i]), project(V.w2, r[i]));
-                shift_corners(g, p, e0, e1);
-            }
-        } else {
-            q[0] = pair(r[0]);
-            if constexpr (SH) g[0] = make_float2(project(V.w1, r[0]), project(V.w2, r[0]));
-        }
     }
     // (no crossing left: the cap ended the walk, or it ended on its last allowed one)
     if (left == 0 && fminf(fminf(T[0], T[1]), T[2]) < lim) {
@@ -721,10 +752,10 @@ template <int FORM, int ADDR>
 constexpr bool kHoist = ADDR == kAddrFlat && (FORM == kFormKahan || FORM == kFormShear);
 
 // PER: periodic bundles only. REGACC: one of several steps of a launch; acc and
-// W0 (the ray's constants) live across them. A0: the kernel's own arguments (A,
+// W0 (the ray's constants) live across them. BATCH: in the persistent kernel. A0: the kernel's own arguments (A,
 // but for the step's fields in a multi-step kernel), whose address finish_ray
 // takes.
-template <int INTERP, class R, int FORM, int ADDR, bool PER, bool REGACC = false>
+template <int INTERP, class R, int FORM, int ADDR, bool PER, bool REGACC = false, bool BATCH = false>
 __device__ __forceinline__ void trace_ray(const TraceArgs& A, const TraceArgs& A0, int ix, int iy, RayAcc* acc = nullptr,
                                           const Walk<R>* W0 = nullptr)
 {
@@ -769,7 +800,10 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, const TraceArgs& A
             else atomicOr(A.err, kErrRange);
             break;
         }
-        constexpr bool SELECT = !AUTO && (FORM == kFormKahan || FORM == kFormPlain || FORM == kFormMoments);
+        // (see add_segment; kernels that hold more, and the NGP walk at 64
+        // registers, branch)
+        constexpr bool SELECT = INTERP == RR_TRILINEAR && !BATCH && !(AUTO && REGACC) &&
+                                (FORM == kFormKahan || FORM == kFormPlain || FORM == kFormMoments);
         walk_flat<INTERP, FORM, SELECT, AUTO && INTERP == RR_TRILINEAR>(A, A.rec, W, V, j == 0, j + 1 < nsub, resumes(W, S, j), B, D, fd, S);
     } else {
         walk_piece<INTERP, R, FORM, ADDR>(A, A.rec, W, V, j, resumes(W, S, j), S);
@@ -959,7 +993,7 @@ __global__ void __launch_bounds__(NT_MAX, kBlocks<INTERP, R, kFormKahan>) trace_
             const int ntx = B.tiles_x[cone];
             int ix, iy;
             tile_ray(B.tile, local % ntx, local / ntx, ix, iy);
-            if (ix < sA.nx && iy < sA.ny) trace_ray<INTERP, R, kFormKahan, ADDR, PER>(sA, sA, ix, iy);
+            if (ix < sA.nx && iy < sA.ny) trace_ray<INTERP, R, kFormKahan, ADDR, PER, false, true>(sA, sA, ix, iy);
             __syncthreads();
         }
     }
