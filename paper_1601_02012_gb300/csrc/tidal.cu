@@ -6,15 +6,15 @@
 // along x through a chunk of planes. Per plane it keeps three planes of the
 // potential (with a one-cell halo) in a shared ring, and every thread
 // evaluates the six central-difference second derivatives at its two centres
-// (whose stencils share their middle rows: 28 shared-memory reads instead of
-// 2 x 19). For records at vertices, vertex (y, z) of the plane is the upper
+// (whose stencils share their middle rows, and take the values they share with
+// the previous planes' from registers: 12 shared-memory reads). For records at vertices, vertex (y, z) of the plane is the upper
 // corner of centres (y-1..y, z-1..z): the z pair is summed with a warp
 // shuffle, the y pair in registers (the vertex between a thread's two rows)
 // or through shared memory (the vertex between two warps), and the record is
 // the mean of that 2 x 2 sum and the previous plane's (kept in registers) --
 // the 8 cells around the vertex. The first centre row and column of the block
-// are the halo of its 15 x 31 vertices. The next potential plane is loaded
-// into registers while the current one is processed. HBM traffic per point:
+// are the halo of its 15 x 31 vertices. The next potential planes are on their
+// way while the current one is processed. HBM traffic per point:
 // the potential read about 1.2 times (halo re-reads hit L2) and the 32-byte
 // record written once: 36 algorithmic bytes per point. The gradient records
 // (KIND 1) take the same march with the three central first differences and
@@ -116,7 +116,7 @@ __device__ __forceinline__ void store_rec(float4* r, float c0, float c1, float c
 constexpr int RP = TZ + 8;                          // 40 floats per row
 constexpr int PYR = TY + 2;                         // 18 rows
 constexpr int SLOT = ((PYR * RP * 4 + 127) / 128) * 128 / 4;   // floats per ring slot
-constexpr int NSLOT = 5;                            // planes c - 1 .. c + 1 in use, c + 2, c + 3 arriving
+constexpr int NSLOT = 6;                            // planes c, c + 1 in use, c + 2 .. c + 4 arriving (5: 908 us, see tidal_kernel)
 constexpr unsigned kWaitTries = 1u << 22;           // bound of every wait on a copy
 
 __device__ __forceinline__ unsigned smem_u32(const void* p)
@@ -159,19 +159,23 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned pari
 // Hxz, Hyz, delta} in 2 float4; KIND 1: gradient records, 4 channels
 // {d_x Phi, d_y Phi, d_z Phi, delta} in 1 float4. Each thread owns the two
 // centres (2 w, z) and (2 w + 1, z) of its warp w, lane z: the two stencils
-// share their middle rows, so 28 shared-memory reads serve two centres (19 for
-// one alone), and the vertex between the two rows sums its y pair in
+// share their middle rows, and the vertex between the two rows sums its y pair in
 // registers.
 // TMA: the potential planes arrive in the ring by tensor copies (one thread
-// issues them two planes ahead, each completing on the slot's mbarrier), for
+// issues them three planes ahead, each completing on the slot's mbarrier), for
 // blocks whose tile needs no periodic wrap in y and z; the other blocks (at
 // the seam) and grids whose rows are not a multiple of 16 bytes load them
 // through registers, a plane ahead. A copy that does not complete within
 // kWaitTries polls makes the block write NaN records (the trace then reports
 // a non-finite sum) after waiting, bounded again, for its copies in flight.
-// (3 resident CTAs per SM: 80 registers, no spills. With the planes staged
-// through registers, 4 CTAs at 64 registers had been 9 % faster; with the
-// tensor copies, 3 CTAs measure 5 % faster than 4, whose cap spills)
+// Bound by the shared-memory pipe and its latency, then by HBM: the eight values
+// that a plane's stencils share with the next plane's are carried in registers,
+// so a thread reads 12 values per plane and two centres (28 without), the ring's
+// slots are counted instead of divided for, and copies run three planes ahead.
+// Whole 512^3 grid, vertex records: 984 -> 923 (carried) -> 908 (slots) -> 896 us
+// (a sixth slot) = 5.39 TB/s at 36 bytes a point, 81 % of the copy bandwidth; 3
+// resident CTAs per SM (80 registers, no spills): 2 measure 1063 us, 64 planes
+// per CTA 923, 20 planes 909, streaming stores 905.
 template <int MODE, int KIND, bool TMA, bool CMP = false>
 __global__ void __launch_bounds__(NT, 3) tidal_kernel(const TidalArgs a, const __grid_constant__ CUtensorMap map)
 {
@@ -233,7 +237,7 @@ __global__ void __launch_bounds__(NT, 3) tidal_kernel(const TidalArgs a, const _
         if (threadIdx.x == 0) {
             for (int k = 0; k < NSLOT; ++k) mbar_init(&mbar[k], 1);
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            for (int p = p0; p <= p0 + 3 && p <= c_last + 1; ++p) issue(p);
+            for (int p = p0; p <= p0 + 4 && p <= c_last + 1; ++p) issue(p);
         }
         __syncthreads();
         ok = arrived(p0) && arrived(p0 + 1);
@@ -271,18 +275,30 @@ __global__ void __launch_bounds__(NT, 3) tidal_kernel(const TidalArgs a, const _
     for (int k = 0; k < 2; ++k)
 #pragma unroll
         for (int q = 0; q < NC; ++q) prev[k][q] = 0.f;
+    // carried along x: the eight values of a plane that the next plane's stencils
+    // read as their neighbours below (b) and two planes of them (c: the current one)
+    const int om = o - RP, o1 = o + RP, op = o + 2 * RP;
+    auto eight = [&](const float* P, float v[8]) {
+        v[0] = P[om]; v[1] = P[o]; v[2] = P[o1]; v[3] = P[op];
+        v[4] = P[o - 1]; v[5] = P[o + 1]; v[6] = P[o1 - 1]; v[7] = P[o1 + 1];
+    };
+    float vb[8], va[8], vc[8];
+    eight(ring, vb);
+    eight(ring + SLOT, va);
+    int s1 = 1;   // slot of plane c
+    unsigned par = 0;   // phase of the slot of plane c + 1
     for (int c = c_first; c <= c_last; ++c) {
-        const float* P0 = ring + slot(c - 1) * SLOT;
-        const float* P1 = ring + slot(c) * SLOT;
-        const float* P2 = ring + slot(c + 1) * SLOT;
+        const float* P1 = ring + s1 * SLOT;
+        const int s2 = s1 + 1 == NSLOT ? 0 : s1 + 1;   // of plane c + 1
+        if (s2 == 0) par ^= 1u;
         float nxt2[LP];
         if (tma) {
             // plane c + 3 into the slot of plane c - 2, read before the last barrier
-            if (threadIdx.x == 0 && c + 3 <= c_last + 1) {
+            if (threadIdx.x == 0 && c + 4 <= c_last + 1) {
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                issue(c + 3);
+                issue(c + 4);
             }
-            ok = arrived(c + 1) && ok;
+            ok = mbar_wait(&mbar[s2], par) && ok;
         } else {
             // plane c + 2 goes into the slot of plane c - 3 (read before the last
             // barrier); plane c + 3 is fetched into registers, a whole plane of
@@ -293,15 +309,16 @@ __global__ void __launch_bounds__(NT, 3) tidal_kernel(const TidalArgs a, const _
 
         // the two stencils: rows r0 - 1 .. r0 + 2 of P1 at z - 1 .. z + 1, rows
         // r0 - 1 .. r0 + 2 of P0 and P2 at z, rows r0, r0 + 1 of P0 and P2 at z +- 1
-        const int om = o - RP, o1 = o + RP, op = o + 2 * RP;
-        const float a_m0 = P1[om - 1], a_m1 = P1[om], a_m2 = P1[om + 1];
-        const float a_00 = P1[o - 1], a_01 = P1[o], a_02 = P1[o + 1];
-        const float a_10 = P1[o1 - 1], a_11 = P1[o1], a_12 = P1[o1 + 1];
-        const float a_p0 = P1[op - 1], a_p1 = P1[op], a_p2 = P1[op + 1];
-        const float b_m = P0[om], b_0 = P0[o], b_1 = P0[o1], b_p = P0[op];
-        const float b_0m = P0[o - 1], b_0p = P0[o + 1], b_1m = P0[o1 - 1], b_1p = P0[o1 + 1];
-        const float c_m = P2[om], c_0 = P2[o], c_1 = P2[o1], c_p = P2[op];
-        const float c_0m = P2[o - 1], c_0p = P2[o + 1], c_1m = P2[o1 - 1], c_1p = P2[o1 + 1];
+        eight(ring + s2 * SLOT, vc);
+        s1 = s2;
+        const float a_m0 = P1[om - 1], a_m1 = va[0], a_m2 = P1[om + 1];
+        const float a_00 = va[4], a_01 = va[1], a_02 = va[5];
+        const float a_10 = va[6], a_11 = va[2], a_12 = va[7];
+        const float a_p0 = P1[op - 1], a_p1 = va[3], a_p2 = P1[op + 1];
+        const float b_m = vb[0], b_0 = vb[1], b_1 = vb[2], b_p = vb[3];
+        const float b_0m = vb[4], b_0p = vb[5], b_1m = vb[6], b_1p = vb[7];
+        const float c_m = vc[0], c_0 = vc[1], c_1 = vc[2], c_p = vc[3];
+        const float c_0m = vc[4], c_0p = vc[5], c_1m = vc[6], c_1p = vc[7];
         float dl[2] = {0.f, 0.f};
         if (a.delta) {
             const size_t base = (size_t)wrapi(c, a.n0) * a.n1 * a.n2;
@@ -375,6 +392,11 @@ __global__ void __launch_bounds__(NT, 3) tidal_kernel(const TidalArgs a, const _
                     a.rec[pt] = make_float4(h[k][0], h[k][1], h[k][2], h[k][3]);
                 }
             }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            vb[i] = va[i];
+            va[i] = vc[i];
         }
         if (!tma) {
 #pragma unroll
