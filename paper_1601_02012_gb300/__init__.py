@@ -472,10 +472,15 @@ def _trace_pass(tr, grid, phi, steps, delta=None, footprint=True, stream=None, g
     ``group`` steps (box-local: no wrap in the walk); the other forms, and cones
     that reach around the box, write into a whole grid's buffer. ``group`` steps
     are traced per launch (16 at most); group=1: one rr_trace_step per step on
-    whole-grid records."""
+    whole-grid records.
+
+    Returns the record buffers, which the caller holds until ``stream`` has
+    passed the steps: torch would hand freed ones to work on the current stream,
+    which need not be ``stream``."""
     steps = list(steps)
+    held = []
     if not steps:
-        return
+        return held
     n = [int(v) for v in grid.n]
     interp, flags = int(tr.desc.interp), int(tr.desc.flags)
     boxed = group > 1 and footprint and not (tr.method_a or tr.generic) and interp == RR_TRILINEAR and \
@@ -495,9 +500,11 @@ def _trace_pass(tr, grid, phi, steps, delta=None, footprint=True, stream=None, g
                 recs = [box_record_buffer(bb, device=phi.device) for bb in bbs]
                 for bb, rec in zip(bbs, recs):
                     tr.tidal_box(grid, phi, rec, bb, delta=delta, stream=stream)
+            held += recs
             tr.steps(grid, recs, steps[i:i + group], boxes=bbs, stream=stream)
-        return
+        return held
     rec = tr.record_buffer(grid, device=phi.device)
+    held.append(rec)
     boxes = [tr.footprint(grid, st.chi_a, st.chi_b) for st in steps] if footprint else [None]
     if footprint and len(boxes) > 1:
         one = _union(boxes, n)
@@ -511,6 +518,7 @@ def _trace_pass(tr, grid, phi, steps, delta=None, footprint=True, stream=None, g
     else:
         for st in steps:
             tr.step(grid, rec, st.chi_a, st.chi_b, st.scale, st.a, stream=stream)
+    return held
 
 
 def trace_kappa(phi, grid, bundle, steps, delta=None, fp64_dda=False, footprint=True, stream=None, group=16):
@@ -526,8 +534,9 @@ def trace_kappa(phi, grid, bundle, steps, delta=None, fp64_dda=False, footprint=
     """
     tr = Tracer(bundle, fp64_dda=fp64_dda)
     try:
-        _trace_pass(tr, grid, phi, steps, delta, footprint, stream, group)
-        k, kb = tr.finalize(stream=stream)
+        held = _trace_pass(tr, grid, phi, steps, delta, footprint, stream, group)
+        k, kb = tr.finalize(stream=stream)   # waits for the stream
+        del held
         return k, kb, tr.segments()
     finally:
         tr.close()
@@ -540,8 +549,9 @@ def trace_method_a(phi, grid, bundle, steps, delta=None, footprint=True, stream=
     kappa_born is the density term alone."""
     tr = Tracer(bundle, method_a=True)
     try:
-        _trace_pass(tr, grid, phi, steps, delta, footprint, stream)
-        k, kb = tr.finalize(stream=stream)
+        held = _trace_pass(tr, grid, phi, steps, delta, footprint, stream)
+        k, kb = tr.finalize(stream=stream)   # waits for the stream
+        del held
         return k, kb, tr.segments()
     finally:
         tr.close()
@@ -559,10 +569,12 @@ def trace_tiles(tiles, bundle, steps, footprint=True, stream=None):
     b.periodic = False
     tr = Tracer(b)
     try:
+        held = []
         for phi, grid, obs in tiles:
             tr.set_observer(obs)
-            _trace_pass(tr, grid, phi, steps, None, footprint, stream)
-        k, kb = tr.finalize(stream=stream)
+            held = _trace_pass(tr, grid, phi, steps, None, footprint, stream)
+        k, kb = tr.finalize(stream=stream)   # waits for the stream
+        del held
         return k, kb, tr.segments()
     finally:
         tr.close()
@@ -574,8 +586,9 @@ def trace_shear(phi, grid, bundle, steps, delta=None, footprint=True, stream=Non
     each [ny, nx], and the number of cell segments."""
     tr = Tracer(bundle, shear=True)
     try:
-        _trace_pass(tr, grid, phi, steps, delta, footprint, stream)
-        k, kb = tr.finalize(stream=stream)
+        held = _trace_pass(tr, grid, phi, steps, delta, footprint, stream)
+        k, kb = tr.finalize(stream=stream)   # waits for the stream
+        del held
         g1, g2 = tr.shear(stream=stream)
         return k, kb, g1, g2, tr.segments()
     finally:
@@ -596,8 +609,10 @@ def _make_autograd():
         @staticmethod
         def forward(ctx, phi, grid, bundle, steps, footprint=True):
             tr = Tracer(bundle)
-            _trace_pass(tr, grid, phi.detach().contiguous(), steps, footprint=footprint)
-            k, kb = tr.finalize()
+            flat = phi.detach().contiguous()
+            held = _trace_pass(tr, grid, flat, steps, footprint=footprint)
+            k, kb = tr.finalize()   # waits for the stream
+            del held
             ctx.tracer = tr
             ctx.grid = grid
             return k, kb

@@ -84,7 +84,7 @@ def trace_kappa_sharded(phi, grid, bundle, steps, rank: int, world: int, group=N
     if y1 > y0:
         tr = Tracer(bundle, rows=(y0, y1))
         try:
-            _trace_pass(tr, grid, phi, steps, footprint=footprint, stream=stream)
+            held = _trace_pass(tr, grid, phi, steps, footprint=footprint, stream=stream)
             k, kb = tr.finalize(stream=stream)
             segs = tr.segments()
         finally:
@@ -116,7 +116,8 @@ def _make_autograd():
             tr = None
             if y1 > y0:
                 tr = Tracer(bundle, rows=(y0, y1))
-                _trace_pass(tr, grid, phi.detach().contiguous(), steps, footprint=footprint)
+                flat = phi.detach().contiguous()
+                held = _trace_pass(tr, grid, flat, steps, footprint=footprint)
                 k, kb = tr.finalize()
             else:
                 k = torch.empty((0, int(bundle.nx)), dtype=torch.float64, device=phi.device)
