@@ -59,6 +59,23 @@ __device__ __forceinline__ void load_factors(const float G[7], float* __restrict
     __syncwarp();
 }
 
+// The contributions of a ray whose derivative is infinite or NaN, one by one:
+// in the product they would reach every point the warp flushes (0 x NaN).
+__device__ __noinline__ void add_alone(double* __restrict__ grad, float4 n, float gk, float gb, int nr, uint32_t P0,
+                                       uint32_t Da, uint32_t Db, float F0, float F1, float F2, float F3)
+{
+    const float w[6] = {n.y * n.y + n.z * n.z, n.x * n.x + n.z * n.z, n.x * n.x + n.y * n.y,
+                        -2.f * n.x * n.y,      -2.f * n.x * n.z,      -2.f * n.y * n.z};
+    for (int r = 0; r < nr; ++r) {
+        const float f = r == 0 ? F0 : (r == 1 ? F1 : (r == 2 ? F2 : F3));
+        if (f == 0.f) continue;
+        double* p = grad + 8 * (size_t)(P0 + ((r & 1) ? Da : 0) + ((r & 2) ? Db : 0));
+        for (int c = 0; c < 6; ++c)
+            if (gk != 0.f) atomicAdd(p + c, (double)(gk * f * w[c]));
+        if (gb != 0.f) atomicAdd(p + 6, (double)(gb * f));
+    }
+}
+
 // Adds F[r] G_c to channel c of the gradient records of the points P0 + {0, Da,
 // Db, Da + Db} (r = 0 .. 3: the corners of the face a crossing leaves; NR = 1:
 // P0 alone, the cell of the NGP form), for every lane with `part` set; all
@@ -77,7 +94,7 @@ __device__ __forceinline__ void load_factors(const float G[7], float* __restrict
 // times the shared-memory data.
 template <int NR>
 __device__ __forceinline__ void flush_points(double* __restrict__ grad, uint32_t P0, uint32_t Da, uint32_t Db,
-                                             const float F[NR], bool part, const float4 row[8], float* __restrict__ sm)
+                                             const float* F, bool part, const float4 row[8], float* __restrict__ sm)
 {
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -121,7 +138,7 @@ __device__ __forceinline__ void flush_points(double* __restrict__ grad, uint32_t
 // warp. Bound by issue slots and the shared-memory round trip of the flush (60 %
 // issue, FP64 and L2 atomics below 21 %); 80, 96 and 128 registers (6, 5, 4
 // blocks per SM) are within 2 %. One step of 256 cells, 1024^2 rays: backward
-// 5.39 -> 3.57 ms; two steps of 32 cells, 96^2 rays: 287 -> 55 us.
+// 5.39 -> 3.63 ms; two steps of 32 cells, 96^2 rays: 287 -> 58 us.
 template <int INTERP, class R, bool PER>
 __global__ void __launch_bounds__(32 * kAdjWarps, (INTERP == RR_TRILINEAR && sizeof(R) == 4) ? 4 : 1)
     trace_adjoint_kernel(const TraceArgs A, const AdjArgs B, const TileCfg tc)
@@ -149,6 +166,8 @@ __global__ void __launch_bounds__(32 * kAdjWarps, (INTERP == RR_TRILINEAR && siz
     }
     if (j >= nsub) alive = false;
     if (!__any_sync(FULL, alive)) return;
+    const bool odd = alive && !(isfinite(gk) && isfinite(gb));   // adds on its own (add_alone)
+    const bool any_odd = __any_sync(FULL, odd);
     const int nn[3] = {A.n0, A.n1, A.n2};
     const R chis = (R)A.chi_s;
     const R ichis = F64 ? (R)(1.0 / A.chi_s) : (R)A.inv_chi_s_f;
@@ -171,12 +190,23 @@ __global__ void __launch_bounds__(32 * kAdjWarps, (INTERP == RR_TRILINEAR && siz
     }
     float4 row[8];
     {
-        const float G[7] = {alive ? gk * W.w[0] : 0.f, alive ? gk * W.w[1] : 0.f, alive ? gk * W.w[2] : 0.f,
-                            alive ? gk * W.w[3] : 0.f, alive ? gk * W.w[4] : 0.f, alive ? gk * W.w[5] : 0.f,
-                            alive ? gb : 0.f};
+        const bool sum = alive && !odd;
+        const float G[7] = {sum ? gk * W.w[0] : 0.f, sum ? gk * W.w[1] : 0.f, sum ? gk * W.w[2] : 0.f,
+                            sum ? gk * W.w[3] : 0.f, sum ? gk * W.w[4] : 0.f, sum ? gk * W.w[5] : 0.f,
+                            sum ? gb : 0.f};
         load_factors(G, sm, row);
     }
     const bool work = alive;
+    // a face (or cell) of this ray into the records, with the warp
+    auto flush = [&](uint32_t P, uint32_t Da, uint32_t Db, const float* F, bool part) {
+        constexpr int NR = TRI ? 4 : 1;
+        flush_points<NR>(B.grad, P, Da, Db, F, part && !odd, row, sm);
+        if (any_odd && odd && part)
+            add_alone(B.grad, A.dirh[rid], B.dkappa ? (float)(B.dkappa[rid] * B.kscale) : 0.f,
+                      B.dkborn ? (float)(B.dkborn[rid] * B.bscale) : 0.f, NR, P, Da, Db, F[0], F[TRI ? 1 : 0],
+                      F[TRI ? 2 : 0], F[TRI ? 3 : 0]);
+        __syncwarp();
+    };
     const R L = W.L, chiA0 = W.chiA0, D0 = W.D0;
     const R eps_end = L * eps_rel;
     float S[TRI ? 8 : 1] = {0.f};
@@ -230,7 +260,7 @@ __global__ void __launch_bounds__(32 * kAdjWarps, (INTERP == RR_TRILINEAR && siz
             // axis a; r = 0..3 runs over the face's corners, the first of
             // the two other axes (a < b) as bit 0
             const float F[4] = {S[0], e0 ? S[2] : S[1], e2 ? S[2] : S[4], e0 ? S[6] : (e1 ? S[5] : S[3])};
-            flush_points<4>(B.grad, P0, e0 ? D[1] : D[0], e2 ? D[1] : D[2], F, cross, row, sm);
+            flush(P0, e0 ? D[1] : D[0], e2 ? D[1] : D[2], F, cross);
             // the exit face's sums become the entry face's
             if (cross) {
                 const float s1 = S[1], s2 = S[2], s3 = S[3], s4 = S[4], s5 = S[5], s6 = S[6], s7 = S[7];
@@ -244,7 +274,7 @@ __global__ void __launch_bounds__(32 * kAdjWarps, (INTERP == RR_TRILINEAR && siz
                 S[7] = 0.f;
             }
         } else {
-            flush_points<1>(B.grad, P0, 0, 0, S, cross, row, sm);
+            flush(P0, 0, 0, S, cross);
             if (cross) S[0] = 0.f;
         }
         alive = cross;
@@ -277,10 +307,10 @@ __global__ void __launch_bounds__(32 * kAdjWarps, (INTERP == RR_TRILINEAR && siz
     // flush everything still pending
     if constexpr (TRI) {
         const float lo[4] = {S[0], S[1], S[2], S[3]}, hi[4] = {S[4], S[5], S[6], S[7]};
-        flush_points<4>(B.grad, P0, D[0], D[1], lo, work, row, sm);
-        flush_points<4>(B.grad, P0 + D[2], D[0], D[1], hi, work, row, sm);
+        flush(P0, D[0], D[1], lo, work);
+        flush(P0 + D[2], D[0], D[1], hi, work);
     } else {
-        flush_points<1>(B.grad, P0, 0, 0, S, work, row, sm);
+        flush(P0, 0, 0, S, work);
     }
     if (overflow) atomicOr(A.err, kErrStepLimit);
 }

@@ -53,3 +53,40 @@ def test_gradient(rrp, oracle_lib, nx, ny, fov, interp, periodic, fp64):
     rms = np.sqrt(np.mean(want[support] ** 2))
     assert np.linalg.norm(got - want) <= 1e-5 * np.linalg.norm(want)
     assert np.abs(got - want).max() <= 1e-4 * rms
+
+
+@pytest.mark.parametrize("interp", [1, 0])
+def test_nan_stays_with_its_ray(rrp, interp):
+    """A NaN and an infinite derivative reach only the points their own rays touch."""
+    import torch
+    g = synth.Grid((24, 24, 40), 36.0)
+    b = synth.Bundle(16, 8, synth.deg(30), synth.deg(20), (18.0, 17.0, 1.0), 50.0, interp=interp)
+    st = synth.Step(50.0, 4.0, 1.0, 1.0)
+    phi = torch.from_numpy(synth.random_field(g.n, 4, np.float32)).cuda()
+    where = rrp.RR_AT_VERTICES if interp else rrp.RR_AT_CENTRES
+
+    def records(y):
+        tr = rrp.Tracer(b)
+        rec = rrp.record_buffer(g)
+        rrp.rr_tidal_tensor(rrp.grid_desc(g), phi, None, rec, where)
+        tr.step(g, rec, st.chi_a, st.chi_b, st.scale, st.a)
+        tr.finalize()
+        out = torch.zeros((g.ncells, 16), dtype=torch.float32, device="cuda")
+        rrp.rr_trace_step_adjoint(tr.ctx, 0, torch.from_numpy(y).cuda(), None, out)
+        torch.cuda.synchronize()
+        tr.close()
+        return out.view(torch.float64).cpu().numpy()
+
+    y = np.random.default_rng(1).standard_normal((8, 16))
+    clean = records(y)
+    bad = [(1, 3, np.nan), (5, 12, np.inf)]
+    own = np.zeros(g.ncells, bool)
+    for r, c, v in bad:
+        one = np.zeros_like(y)
+        one[r, c] = 1.0
+        own |= (records(one) != 0).any(1)
+        y[r, c] = v
+    got = records(y)
+    assert not np.isfinite(got[own][:, 0]).all()
+    rms = np.sqrt(np.mean(clean ** 2))
+    assert np.isfinite(got[~own]).all() and np.abs(got[~own] - clean[~own]).max() <= 1e-5 * rms
