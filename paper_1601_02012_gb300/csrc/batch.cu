@@ -28,6 +28,7 @@ struct rr_batch {
     int blocks_per_sm = 0;       // 0: as many as fit (occupancy)
     int sms = 1;
     std::vector<bool> staged;
+    std::vector<bool> heavy;     // staged steps that cross the seam often
     // host staging (pinned) and its device copy
     TraceArgs* h_args = nullptr;
     int* h_tiles = nullptr;      // tile_start[n+1] then tiles_x[n]
@@ -99,6 +100,7 @@ rr_status rr_batch_create(int32_t n, const rr_bundle_desc* bundles, rr_batch** o
     for (int i = 0; i < n; ++i) b->periodic = b->periodic && (bundles[i].flags & RR_PERIODIC);
     b->cones.assign((size_t)n, nullptr);
     b->staged.assign((size_t)n, false);
+    b->heavy.assign((size_t)n, false);
     for (int i = 0; i < n; ++i) {
         rr_status st = rr_create(&bundles[i], &b->cones[(size_t)i]);
         if (st != RR_OK) {
@@ -183,6 +185,7 @@ rr_status rr_batch_set_step(rr_batch* b, int32_t i, const rr_grid_desc* grid, co
     rr_status st = validate_step(c, grid, rec, chi_a, chi_b, scale, a_step);
     if (st != RR_OK) return st;
     b->h_args[i] = make_trace_args(c, grid, rec, chi_a, chi_b, scale, a_step);
+    b->heavy[(size_t)i] = seam_heavy(c->bundle, c->bundle.obs, *grid, chi_a, chi_b);
     c->log.push_back(make_step_record(c, grid, chi_a, chi_b, scale, a_step));
     b->staged[(size_t)i] = true;
     return RR_OK;
@@ -217,7 +220,12 @@ rr_status rr_batch_trace(rr_batch* b, void* stream)
     a.chunk = b->chunk;
     a.tile = b->tile;
     bool small = true;
-    for (int i = 0; i < n; ++i) small = small && b->h_args[i].fe[0] > 0;
+    int heavy = 0;
+    for (int i = 0; i < n; ++i) {
+        small = small && b->h_args[i].fe[0] > 0;
+        heavy += b->heavy[(size_t)i];
+    }
+    if (2 * heavy > n) small = false;   // (wrapped indices for all)
     return status_of_cuda(launch_trace_batch(a, b->interp, b->fp64, grid_blocks(b), s, small, b->periodic));
 }
 

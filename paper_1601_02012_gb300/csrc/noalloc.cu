@@ -115,7 +115,8 @@ extern "C" rr_status rr_trace_step_noalloc(const rr_bundle_desc* bundle, const r
     e = launch_init_state(*bundle, rs, s);
     if (e != cudaSuccess) return to_status(e);
     const TraceArgs a = make_trace_args(*bundle, rs, grid, rec, chi_a, chi_b, scale, a_step, nullptr, nullptr);
-    e = launch_trace(a, bundle->interp, (bundle->flags & RR_FP64_DDA) != 0, s);
+    e = launch_trace(a, bundle->interp, (bundle->flags & RR_FP64_DDA) != 0, s, TileCfg{}, kFormKahan, false,
+                     seam_heavy(*bundle, bundle->obs, *grid, chi_a, chi_b));
     if (e == cudaSuccess) e = launch_finalize((int)nr, rs, kappa, kappa_born, nullptr, s);
     if (e != cudaSuccess) return to_status(e);
 

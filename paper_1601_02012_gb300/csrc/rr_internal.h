@@ -192,8 +192,10 @@ enum { kAddrIndex = 0, kAddrPlanes = 1, kAddrFlat = 2, kAddrAuto = 3 };
 // flat: the caller has checked that no ray of the step comes within a cell of
 // the periodic seam and that the grid has fewer than 2^31 points (used by the
 // default FP32 trilinear periodic form only; ignored otherwise).
+// wrapped: wrapped indices throughout instead of a choice per sub-step
+// (trilinear; seam_heavy).
 cudaError_t launch_trace(const TraceArgs& a, int interp, bool fp64_dda, cudaStream_t s, const TileCfg& t,
-                         int form = kFormKahan, bool flat = false);
+                         int form = kFormKahan, bool flat = false, bool wrapped = false);
 // small: every bundle's grid has fewer than 2^31 points; periodic: every bundle is
 cudaError_t launch_trace_batch(const BatchArgs& b, int interp, bool fp64_dda, int blocks, cudaStream_t s, bool small,
                                bool periodic);
@@ -255,6 +257,7 @@ void footprint_box(const rr_bundle_desc& b, const double obs[3], const rr_grid_d
 // below and 3 above on every axis (no vertex plane the walk reads lies
 // across the seam).
 bool flat_ok(const rr_bundle_desc& b, const double obs[3], const rr_grid_desc& g, double chi_a, double chi_b);
+bool seam_heavy(const rr_bundle_desc& b, const double obs[3], const rr_grid_desc& g, double chi_a, double chi_b);
 // Argument checks of a bundle and a grid description (RR_OK or RR_ERR_ARG).
 rr_status check_bundle(const rr_bundle_desc* b);
 rr_status check_grid(const rr_grid_desc* g);

@@ -134,11 +134,8 @@ constexpr float kSliver = 4.76837158203125e-07f;
 //  kAddrIndex:  vertex indices per axis, with periodic wrap (any grid).
 //  kAddrPlanes: the 64-bit record offsets of the mirrored cell's two vertex
 //               planes per axis (entry and exit side), with wrap, so that a
-//               record's offset is two additions (6.5 % faster than indices
-//               on the production workload). The persistent batch kernel,
-//               which also holds its staged arguments, and the forms with
-//               more per-segment state (moments, shear, Method A, generic)
-//               measured 1.5-4 % slower with them and keep indices.
+//               record's offset is two additions: the FP64 walk's. (In FP32,
+//               one step through 8 periods of 24^3: 1014 us, by indices 960.)
 //  kAddrAuto:   kAddrFlat for the sub-steps whose own cells and vertex planes
 //               lie inside the grid without a wrap (counted exactly as the walk
 //               will cross them, so a ray that ends on the box face z = 0 still
@@ -1024,27 +1021,30 @@ cudaError_t launch_addr(const TraceArgs& a, const dim3& grid, int nt, cudaStream
 }
 
 template <int INTERP, class R, int FORM>
-cudaError_t launch_one(const TraceArgs& a, const dim3& grid, int nt, cudaStream_t s, const TileCfg& t)
+cudaError_t launch_one(const TraceArgs& a, const dim3& grid, int nt, cudaStream_t s, const TileCfg& t,
+                       bool wrapped = false)
 {
     if constexpr (sizeof(R) == 4) {
         // fewer than 2^31 points
-        if (a.fe[0] > 0) return launch_addr<INTERP, R, FORM, kAddrAuto>(a, grid, nt, s, t);
+        if (a.fe[0] > 0 && !(wrapped && INTERP == RR_TRILINEAR))
+            return launch_addr<INTERP, R, FORM, kAddrAuto>(a, grid, nt, s, t);
     }
-    return launch_addr<INTERP, R, FORM, FORM == kFormKahan && INTERP == RR_TRILINEAR ? kAddrPlanes : kAddrIndex>(
+    return launch_addr<INTERP, R, FORM, FORM == kFormKahan && INTERP == RR_TRILINEAR && sizeof(R) == 8 ? kAddrPlanes : kAddrIndex>(
         a, grid, nt, s, t);
 }
 
 template <int FORM>
-cudaError_t launch_form(const TraceArgs& a, int interp, const dim3& grid, int nt, cudaStream_t s, const TileCfg& t)
+cudaError_t launch_form(const TraceArgs& a, int interp, const dim3& grid, int nt, cudaStream_t s, const TileCfg& t,
+                        bool wrapped)
 {
-    return interp == RR_TRILINEAR ? launch_one<RR_TRILINEAR, float, FORM>(a, grid, nt, s, t)
+    return interp == RR_TRILINEAR ? launch_one<RR_TRILINEAR, float, FORM>(a, grid, nt, s, t, wrapped)
                                   : launch_one<RR_NGP, float, FORM>(a, grid, nt, s, t);
 }
 
 }  // namespace
 
 cudaError_t launch_trace(const TraceArgs& a, int interp, bool fp64_dda, cudaStream_t s, const TileCfg& t,
-                         int form, bool flat)
+                         int form, bool flat, bool wrapped)
 {
     if (!tile_ok(t)) return cudaErrorInvalidValue;
     const dim3 grid = tile_grid(t, a.nx, a.ny);
@@ -1064,14 +1064,14 @@ cudaError_t launch_trace(const TraceArgs& a, int interp, bool fp64_dda, cudaStre
         return interp == RR_TRILINEAR ? launch_one<RR_TRILINEAR, double, kFormKahan>(a, grid, nt, s, t)
                                       : launch_one<RR_NGP, double, kFormKahan>(a, grid, nt, s, t);
     switch (form) {
-    case kFormPlain: return launch_form<kFormPlain>(a, interp, grid, nt, s, t);
-    case kFormMoments: return launch_form<kFormMoments>(a, interp, grid, nt, s, t);
-    case kFormGeneric: return launch_form<kFormGeneric>(a, interp, grid, nt, s, t);
-    case kFormMethodA: return launch_form<kFormMethodA>(a, interp, grid, nt, s, t);
+    case kFormPlain: return launch_form<kFormPlain>(a, interp, grid, nt, s, t, wrapped);
+    case kFormMoments: return launch_form<kFormMoments>(a, interp, grid, nt, s, t, wrapped);
+    case kFormGeneric: return launch_form<kFormGeneric>(a, interp, grid, nt, s, t, wrapped);
+    case kFormMethodA: return launch_form<kFormMethodA>(a, interp, grid, nt, s, t, wrapped);
     // (the shear form's 128-register cap of two resident blocks spills a few
     // bytes; 168 registers without spills measured 2 % slower)
-    case kFormShear: return launch_form<kFormShear>(a, interp, grid, nt, s, t);
-    default: return launch_form<kFormKahan>(a, interp, grid, nt, s, t);
+    case kFormShear: return launch_form<kFormShear>(a, interp, grid, nt, s, t, wrapped);
+    default: return launch_form<kFormKahan>(a, interp, grid, nt, s, t, wrapped);
     }
 }
 
@@ -1079,15 +1079,15 @@ template <int FORM>
 static cudaError_t launch_steps_form(const TraceArgs& a, const StepBlock& b, int interp, bool flat, dim3 grid, int nt,
                               const TileCfg& t, cudaStream_t s)
 {
-    // (grids of fewer than 2^31 points) trilinear: steps that all take the flat
+    // trilinear (grids of fewer than 2^31 points): steps that all take the flat
     // addressing (periodic), or choose it per sub-step, as NGP steps do
     if (interp == RR_TRILINEAR) {
         if (flat && a.periodic) trace_steps_kernel<RR_TRILINEAR, kAddrFlat, FORM, true><<<grid, nt, 0, s>>>(a, b, t);
         else if (a.periodic) trace_steps_kernel<RR_TRILINEAR, kAddrAuto, FORM, true><<<grid, nt, 0, s>>>(a, b, t);
         else trace_steps_kernel<RR_TRILINEAR, kAddrAuto, FORM, false><<<grid, nt, 0, s>>>(a, b, t);
     } else {
-        if (a.fe[0] <= 0) return cudaErrorInvalidValue;
-        if (a.periodic) trace_steps_kernel<RR_NGP, kAddrAuto, FORM, true><<<grid, nt, 0, s>>>(a, b, t);
+        if (a.fe[0] <= 0) trace_steps_kernel<RR_NGP, kAddrIndex, FORM, false><<<grid, nt, 0, s>>>(a, b, t);
+        else if (a.periodic) trace_steps_kernel<RR_NGP, kAddrAuto, FORM, true><<<grid, nt, 0, s>>>(a, b, t);
         else trace_steps_kernel<RR_NGP, kAddrAuto, FORM, false><<<grid, nt, 0, s>>>(a, b, t);
     }
     return cudaGetLastError();
