@@ -100,6 +100,7 @@ TraceArgs make_trace_args(const rr_bundle_desc& b, const RayState& st, const rr_
     a.Lf = (float)(chi_a - chi_b);
     a.D0f = (float)(b.chi_s - chi_a);
     a.inv_chi_s_f = (float)(1.0 / b.chi_s);
+    a.chi_sf = (float)b.chi_s;
     a.sub_len = (float)(32.0 * a.h);
     // (as a ray divides its own clipped path)
     a.nsub = (int)std::max(1.f, std::min(ceilf(a.Lf / a.sub_len), 1e9f));

@@ -42,13 +42,14 @@ namespace {
 // slower on the production pass).
 __device__ __forceinline__ void shift_corners(float2 q[8], const float2 p[4], bool e0, bool e1)
 {
+    const bool e2 = !e0 && !e1;
     float2 n[8];
-    n[0] = e0 ? q[1] : (e1 ? q[2] : q[4]);
-    n[1] = e0 ? p[0] : (e1 ? q[3] : q[5]);
-    n[2] = e0 ? q[3] : (e1 ? p[0] : q[6]);
-    n[3] = (e0 || e1) ? p[1] : q[7];
-    n[4] = e0 ? q[5] : (e1 ? q[6] : p[0]);
-    n[5] = e0 ? p[2] : (e1 ? q[7] : p[1]);
+    n[0] = e2 ? q[4] : (e1 ? q[2] : q[1]);
+    n[1] = e2 ? q[5] : (e1 ? q[3] : p[0]);
+    n[2] = e2 ? q[6] : (e1 ? p[0] : q[3]);
+    n[3] = e2 ? q[7] : p[1];
+    n[4] = e2 ? p[0] : (e1 ? q[6] : q[5]);
+    n[5] = e2 ? p[1] : (e1 ? q[7] : p[2]);
     n[6] = e0 ? q[7] : p[2];
     n[7] = p[3];
 #pragma unroll
@@ -466,8 +467,8 @@ __device__ __forceinline__ void walk_piece(const TraceArgs& A, const float4* rec
 // the step's sums;
 // slivers are skipped. SELECT: by selecting the old sums afterwards instead of
 // branching around the arithmetic (three control instructions a segment):
-// default form 21.52 -> 21.23 ms per production pass; the forms with more sums
-// or fewer registers to spare keep the branch.
+// default form 21.52 -> 21.23 ms per production pass; the shear form, with twice
+// the sums, and the kernels without registers to spare keep the branch.
 template <int INTERP, int FORM, bool SELECT>
 __device__ __forceinline__ void add_segment(const TraceArgs& A, const Walk<float>& W, const float2* q,
                                             const float2* g, const float T[3], float sig, float tend,
@@ -482,7 +483,7 @@ __device__ __forceinline__ void add_segment(const TraceArgs& A, const Walk<float
     const bool live = t > tend * kSliver;
     if (!SELECT && !live) return;
     const PieceState<float> S0 = S;
-    const float chis = (float)A.chi_s, ichis = A.inv_chi_s_f;
+    const float chis = A.chi_sf, ichis = A.inv_chi_s_f;
     float2 e[4];
     if constexpr (TRI)
         line_cubic2(q, bc2(u[0]), bc2(u[1]), bc2(u[2]), bc2(W.v[0]), bc2(W.v[1]), bc2(W.v[2]), e);
@@ -526,7 +527,9 @@ __device__ __forceinline__ void add_segment(const TraceArgs& A, const Walk<float
 // 58 % and ALU 47 % busy at 75 % issue); production pass, trace kernels 22.62 ->
 // 21.52 ms without the last segment in the loop, 20.83 ms with one test, 20.33 ms
 // with the ray's constants hoisted (kHoist), 19.72 ms with the new corners
-// projected before the crossing's bookkeeping.
+// projected before the crossing's bookkeeping, 19.40 ms with the crossings of all
+// axes evaluated anew and the shift's selects ordered by the z face, the
+// commonest (one step of 256 cells 2.24 -> 2.13 ms, batch 8.91 -> 8.36 ms).
 // (B, D0, fd, SEAM: flat_start's; more: another sub-step follows; WIDE: a record in one 32-byte load)
 template <int INTERP, int FORM, bool SELECT, bool SEAM, bool WIDE = true>
 __device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec, const Walk<float>& W, const RayWeights& V, bool first,
@@ -625,9 +628,14 @@ __device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec,
             if (e1) D[1] = fd[1];
             if (e2) D[2] = fd[2];
         }
-        if (e0) { kf[0] += 1.f; T[0] = fmaf(kf[0], W.td[0], W.T0[0]); }
-        if (e1) { kf[1] += 1.f; T[1] = fmaf(kf[1], W.td[1], W.T0[1]); }
-        if (e2) { kf[2] += 1.f; T[2] = fmaf(kf[2], W.td[2], W.T0[2]); }
+        // (every axis' next crossing evaluated again, the same but for axis e: no
+        // predicates, no chain through the exit axis)
+        kf[0] += e0 ? 1.f : 0.f;
+        kf[1] += e1 ? 1.f : 0.f;
+        kf[2] += e2 ? 1.f : 0.f;
+        T[0] = fmaf(kf[0], W.td[0], W.T0[0]);
+        T[1] = fmaf(kf[1], W.td[1], W.T0[1]);
+        T[2] = fmaf(kf[2], W.td[2], W.T0[2]);
     }
     // (no crossing left: the cap ended the walk, or it ended on its last allowed one)
     if (left == 0 && fminf(fminf(T[0], T[1]), T[2]) < lim) {
@@ -645,7 +653,7 @@ __device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec,
         if constexpr (TRI) S.qb = trilinear_x(q, u[0], u[1], u[2]);
         else S.qb = q[0].x;
         float G0, G1, G2;
-        kernel_coeffs(t, sig, W.chiA0, W.D0, (float)A.chi_s, A.inv_chi_s_f, G0, G1, G2);
+        kernel_coeffs(t, sig, W.chiA0, W.D0, A.chi_sf, A.inv_chi_s_f, G0, G1, G2);
         S.gb = fmaf(t, fmaf(t, G2, G1), G0);
     }
     if (more) {
@@ -741,12 +749,11 @@ __device__ __noinline__ void finish_ray(const TraceArgs& A, const float4* rec, l
 
 // Whether a multi-step kernel sets a ray's constants up once, outside its loop
 // over the steps, and takes the sub-steps' division from the host. Production
-// pass, trace kernels: default form 20.83 -> 20.33 ms, shear (256^3, 1024^2 rays,
-// 20 steps) 4.46 -> 4.37 ms; the moments, Method A and the index walks spill or
-// gain nothing (3.00 -> 3.08, 2.57 -> 2.63, NGP 1.73 -> 1.78 ms) and keep both
-// inside.
-template <int FORM, int ADDR>
-constexpr bool kHoist = ADDR == kAddrFlat && (FORM == kFormKahan || FORM == kFormShear);
+// pass, trace kernels: default form 20.83 -> 20.33 ms; 256^3, 1024^2 rays, 20
+// steps: shear 4.46 -> 4.37, moments 2.90 -> 2.82, Method A (with selects for
+// slivers) 2.52 -> 2.41 ms; the kernels that choose their addressing spill.
+template <int ADDR>
+constexpr bool kHoist = ADDR == kAddrFlat;
 
 // PER: periodic bundles only. REGACC: one of several steps of a launch; acc and
 // W0 (the ray's constants) live across them. BATCH: in the persistent kernel. A0: the kernel's own arguments (A,
@@ -776,7 +783,7 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, const TraceArgs& A
         }
     }
     // FP32: sub-steps of at most sub_len, so that the path variable stays small
-    constexpr bool HOIST = REGACC && kHoist<FORM, ADDR>;
+    constexpr bool HOIST = REGACC && kHoist<ADDR>;
     const int nsub = F64 ? 1 : (HOIST ? A.nsub : max(1, (int)ceilf(rg.Lf / A.sub_len)));
     const float dsub = HOIST ? A.dsub : rg.Lf / (float)nsub;
 
@@ -800,7 +807,7 @@ __device__ __forceinline__ void trace_ray(const TraceArgs& A, const TraceArgs& A
         // (see add_segment; kernels that hold more, and the NGP walk at 64
         // registers, branch)
         constexpr bool SELECT = INTERP == RR_TRILINEAR && !BATCH && !(AUTO && REGACC) &&
-                                (FORM == kFormKahan || FORM == kFormPlain || FORM == kFormMoments);
+                                FORM != kFormShear;
         walk_flat<INTERP, FORM, SELECT, AUTO && INTERP == RR_TRILINEAR>(A, A.rec, W, V, j == 0, j + 1 < nsub, resumes(W, S, j), B, D, fd, S);
     } else {
         walk_piece<INTERP, R, FORM, ADDR>(A, A.rec, W, V, j, resumes(W, S, j), S);
@@ -917,7 +924,7 @@ __global__ void __launch_bounds__(NT_MAX, kBlocks<INTERP, float, FORM>)
     RayAcc acc;
     acc.loaded = false;
     Walk<float> W0;
-    if constexpr (kHoist<FORM, ADDR>) ray_consts<float>(A, (long long)iy * A.nx + ix, W0);
+    if constexpr (kHoist<ADDR>) ray_consts<float>(A, (long long)iy * A.nx + ix, W0);
     for (int g = 0; g < S.n; ++g) {
         const StepArgs& st = S.s[g];
         TraceArgs As = A;

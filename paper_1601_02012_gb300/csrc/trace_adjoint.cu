@@ -295,9 +295,12 @@ __global__ void __launch_bounds__(32 * kAdjWarps, (INTERP == RR_TRILINEAR && siz
                         D[a] = (uint32_t)(nvhi - W.vhi[a]) * st[a];
                         W.vhi[a] = nvhi;
                     }
-                    kf[a] += (R)1;
-                    T[a] = fma(kf[a], W.td[a], W.T0[a]);
                 }
+            kf[0] += e0 ? (R)1 : (R)0;
+            kf[1] += e1 ? (R)1 : (R)0;
+            kf[2] += e2 ? (R)1 : (R)0;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) T[a] = fma(kf[a], W.td[a], W.T0[a]);
             if (--left < 0) {
                 overflow = true;
                 alive = false;
