@@ -148,6 +148,7 @@ struct AdjArgs {
     double kscale;              // the step's scale
     double bscale;              // scale * 1.5 Omega_m (H0/c)^2 / a_step
     int first = 0;              // first sub-step of the launch
+    int tiles_x = 0;            // ray tiles along x
 };
 
 // Ray-tile shape: a warp covers wx x (32/wx) pixels, a block bwx x bwy warps.

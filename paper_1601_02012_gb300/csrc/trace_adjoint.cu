@@ -125,7 +125,7 @@ __device__ __forceinline__ void flush_points(double* __restrict__ grad, uint32_t
     }
 }
 
-// Adjoint of one sub-step (B.first + blockIdx.z) of one step: replays the walk and, for
+// Adjoint of one sub-step (B.first + blockIdx.x % pieces) of one step: replays the walk and, for
 // every point the ray's segments read (the 8 vertices of each cell, or its
 // centre), accumulates dI/dq of the segment integrals (the transpose of the
 // forward map) while the point stays in the ray's current cell; a point is
@@ -135,10 +135,14 @@ __device__ __forceinline__ void flush_points(double* __restrict__ grad, uint32_t
 // the records take sums), so each is a thread of its own: a small bundle fills
 // the GPU by shorter ones. The lanes of a warp stay together to the warp's last
 // crossing, those that are done adding nothing: every flush is one of a whole
-// warp. Bound by issue slots and the shared-memory round trip of the flush (60 %
-// issue, FP64 and L2 atomics below 21 %); 80, 96 and 128 registers (6, 5, 4
-// blocks per SM) are within 2 %. One step of 256 cells, 1024^2 rays: backward
-// 5.39 -> 3.63 ms; two steps of 32 cells, 96^2 rays: 287 -> 58 us.
+// warp. Consecutive blocks are the sub-steps of one ray tile: the first sub-steps
+// of all rays add to the few points around the observer, and run together
+// (sub-step slowest) they queued for those points' L2 lines, for a time that
+// depended on where the records lay in memory (3.25 to 3.63 ms; now 3.00 ms).
+// Bound by issue slots and the shared-memory round trip of the flush (FP64 and L2
+// atomics below 21 %); 4 blocks per SM, 5 are 4 % slower. One step of 256 cells,
+// 1024^2 rays: backward 5.39 -> 3.00 ms; two steps of 32 cells, 96^2 rays: 287 ->
+// 58 us.
 template <int INTERP, class R, bool PER>
 __global__ void __launch_bounds__(32 * kAdjWarps, (INTERP == RR_TRILINEAR && sizeof(R) == 4) ? 4 : 1)
     trace_adjoint_kernel(const TraceArgs A, const AdjArgs B, const TileCfg tc)
@@ -149,7 +153,8 @@ __global__ void __launch_bounds__(32 * kAdjWarps, (INTERP == RR_TRILINEAR && siz
     __shared__ __align__(16) float stage[kAdjWarps * 8 * kRow];
     float* sm = stage + (threadIdx.x >> 5) * 8 * kRow;
     int ix, iy;
-    tile_ray(tc, blockIdx.x, blockIdx.y, ix, iy);
+    const int pieces = gridDim.x / B.tiles_x;
+    tile_ray(tc, blockIdx.x / pieces, blockIdx.y, ix, iy);
     const bool ray = ix < A.nx && iy < A.ny;
     const long long rid = ray ? (long long)iy * A.nx + ix : 0;
     const float gk = ray && B.dkappa ? (float)(B.dkappa[rid] * B.kscale) : 0.f;
@@ -157,7 +162,7 @@ __global__ void __launch_bounds__(32 * kAdjWarps, (INTERP == RR_TRILINEAR && siz
     bool alive = ray && (gk != 0.f || gb != 0.f);
     RayRange rg;
     if (alive && !ray_range<PER>(A, rid, rg)) alive = false;
-    const int j = B.first + blockIdx.z;
+    const int j = B.first + blockIdx.x % pieces;
     int nsub = 1;
     float dsub = 0.f;
     if (!F64 && alive) {
@@ -295,12 +300,9 @@ __global__ void __launch_bounds__(32 * kAdjWarps, (INTERP == RR_TRILINEAR && siz
                         D[a] = (uint32_t)(nvhi - W.vhi[a]) * st[a];
                         W.vhi[a] = nvhi;
                     }
+                    kf[a] += (R)1;
+                    T[a] = fma(kf[a], W.td[a], W.T0[a]);
                 }
-            kf[0] += e0 ? (R)1 : (R)0;
-            kf[1] += e1 ? (R)1 : (R)0;
-            kf[2] += e2 ? (R)1 : (R)0;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) T[a] = fma(kf[a], W.td[a], W.T0[a]);
             if (--left < 0) {
                 overflow = true;
                 alive = false;
@@ -356,8 +358,12 @@ cudaError_t launch_trace_adjoint(const TraceArgs& args, const AdjArgs& b, int in
     else k = fp64_dda ? adj_kernel<RR_NGP, double>(a) : adj_kernel<RR_NGP, float>(a);
     const int pieces = fp64_dda ? 1 : a.nsub;
     AdjArgs g = b;
-    for (g.first = 0; g.first < pieces; g.first += 65535) {
-        grid.z = (unsigned)(pieces - g.first < 65535 ? pieces - g.first : 65535);
+    g.tiles_x = (int)grid.x;
+    const int most = 0x7fffffff / g.tiles_x;   // sub-steps in a launch (grid.x < 2^31)
+    for (int done = 0, n; done < pieces; done += n) {
+        n = pieces - done < most ? pieces - done : most;
+        g.first = done;
+        grid.x = (unsigned)(g.tiles_x * n);
         k<<<grid, nt, 0, s>>>(a, g, t);
     }
     return cudaGetLastError();
