@@ -461,6 +461,21 @@ def _cheaper(one, boxes):
     return _points(one) <= sum(_points(bb) for bb in boxes) + (len(boxes) - 1) * _LAUNCH_POINTS
 
 
+def _on(stream):
+    """A context in which torch allocates for ``stream`` (a torch stream, a raw
+    handle, or None: the current one): memory freed by Python while work on
+    ``stream`` still uses it then goes to later work on that stream alone."""
+    import contextlib
+
+    import torch
+    if stream is None:
+        return contextlib.nullcontext()
+    if not isinstance(stream, torch.cuda.Stream):
+        raw = stream if isinstance(stream, int) else int(stream.cuda_stream)
+        stream = torch.cuda.ExternalStream(raw) if raw else torch.cuda.default_stream()
+    return torch.cuda.stream(stream)
+
+
 def _trace_pass(tr, grid, phi, steps, delta=None, footprint=True, stream=None, group=16):
     """The steps of a pass on one potential, through ``tr``.
 
@@ -474,13 +489,11 @@ def _trace_pass(tr, grid, phi, steps, delta=None, footprint=True, stream=None, g
     are traced per launch (16 at most); group=1: one rr_trace_step per step on
     whole-grid records.
 
-    Returns the record buffers, which the caller holds until ``stream`` has
-    passed the steps: torch would hand freed ones to work on the current stream,
-    which need not be ``stream``."""
+    The record buffers are ``stream``'s (_on): they are dropped here with the
+    steps still queued."""
     steps = list(steps)
-    held = []
     if not steps:
-        return held
+        return
     n = [int(v) for v in grid.n]
     interp, flags = int(tr.desc.interp), int(tr.desc.flags)
     boxed = group > 1 and footprint and not (tr.method_a or tr.generic) and interp == RR_TRILINEAR and \
@@ -493,18 +506,20 @@ def _trace_pass(tr, grid, phi, steps, delta=None, footprint=True, stream=None, g
             bbs = boxes[i:i + group]
             one = _union(bbs, n)
             if all(one[2 * a + 1] - one[2 * a] < n[a] for a in range(3)) and _points(one) < 2 ** 31 and _cheaper(one, bbs):
-                rec = box_record_buffer(one, device=phi.device)
+                with _on(stream):
+                    rec = box_record_buffer(one, device=phi.device)
                 tr.tidal_box(grid, phi, rec, one, delta=delta, stream=stream)
                 bbs, recs = [one] * len(bbs), [rec] * len(bbs)
             else:
-                recs = [box_record_buffer(bb, device=phi.device) for bb in bbs]
+                with _on(stream):
+                    recs = [box_record_buffer(bb, device=phi.device) for bb in bbs]
                 for bb, rec in zip(bbs, recs):
                     tr.tidal_box(grid, phi, rec, bb, delta=delta, stream=stream)
-            held += recs
             tr.steps(grid, recs, steps[i:i + group], boxes=bbs, stream=stream)
-        return held
-    rec = tr.record_buffer(grid, device=phi.device)
-    held.append(rec)
+            rec = recs = None   # (the next group may take the memory)
+        return
+    with _on(stream):
+        rec = tr.record_buffer(grid, device=phi.device)
     boxes = [tr.footprint(grid, st.chi_a, st.chi_b) for st in steps] if footprint else [None]
     if footprint and len(boxes) > 1:
         one = _union(boxes, n)
@@ -518,7 +533,6 @@ def _trace_pass(tr, grid, phi, steps, delta=None, footprint=True, stream=None, g
     else:
         for st in steps:
             tr.step(grid, rec, st.chi_a, st.chi_b, st.scale, st.a, stream=stream)
-    return held
 
 
 def trace_kappa(phi, grid, bundle, steps, delta=None, fp64_dda=False, footprint=True, stream=None, group=16):
@@ -534,9 +548,8 @@ def trace_kappa(phi, grid, bundle, steps, delta=None, fp64_dda=False, footprint=
     """
     tr = Tracer(bundle, fp64_dda=fp64_dda)
     try:
-        held = _trace_pass(tr, grid, phi, steps, delta, footprint, stream, group)
-        k, kb = tr.finalize(stream=stream)   # waits for the stream
-        del held
+        _trace_pass(tr, grid, phi, steps, delta, footprint, stream, group)
+        k, kb = tr.finalize(stream=stream)
         return k, kb, tr.segments()
     finally:
         tr.close()
@@ -549,9 +562,8 @@ def trace_method_a(phi, grid, bundle, steps, delta=None, footprint=True, stream=
     kappa_born is the density term alone."""
     tr = Tracer(bundle, method_a=True)
     try:
-        held = _trace_pass(tr, grid, phi, steps, delta, footprint, stream)
-        k, kb = tr.finalize(stream=stream)   # waits for the stream
-        del held
+        _trace_pass(tr, grid, phi, steps, delta, footprint, stream)
+        k, kb = tr.finalize(stream=stream)
         return k, kb, tr.segments()
     finally:
         tr.close()
@@ -569,12 +581,10 @@ def trace_tiles(tiles, bundle, steps, footprint=True, stream=None):
     b.periodic = False
     tr = Tracer(b)
     try:
-        held = []
         for phi, grid, obs in tiles:
             tr.set_observer(obs)
-            held = _trace_pass(tr, grid, phi, steps, None, footprint, stream)
-        k, kb = tr.finalize(stream=stream)   # waits for the stream
-        del held
+            _trace_pass(tr, grid, phi, steps, None, footprint, stream)
+        k, kb = tr.finalize(stream=stream)
         return k, kb, tr.segments()
     finally:
         tr.close()
@@ -586,9 +596,8 @@ def trace_shear(phi, grid, bundle, steps, delta=None, footprint=True, stream=Non
     each [ny, nx], and the number of cell segments."""
     tr = Tracer(bundle, shear=True)
     try:
-        held = _trace_pass(tr, grid, phi, steps, delta, footprint, stream)
-        k, kb = tr.finalize(stream=stream)   # waits for the stream
-        del held
+        _trace_pass(tr, grid, phi, steps, delta, footprint, stream)
+        k, kb = tr.finalize(stream=stream)
         g1, g2 = tr.shear(stream=stream)
         return k, kb, g1, g2, tr.segments()
     finally:
@@ -610,9 +619,8 @@ def _make_autograd():
         def forward(ctx, phi, grid, bundle, steps, footprint=True):
             tr = Tracer(bundle)
             flat = phi.detach().contiguous()
-            held = _trace_pass(tr, grid, flat, steps, footprint=footprint)
-            k, kb = tr.finalize()   # waits for the stream
-            del held
+            _trace_pass(tr, grid, flat, steps, footprint=footprint)
+            k, kb = tr.finalize()
             ctx.tracer = tr
             ctx.grid = grid
             return k, kb

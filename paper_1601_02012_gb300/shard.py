@@ -84,7 +84,7 @@ def trace_kappa_sharded(phi, grid, bundle, steps, rank: int, world: int, group=N
     if y1 > y0:
         tr = Tracer(bundle, rows=(y0, y1))
         try:
-            held = _trace_pass(tr, grid, phi, steps, footprint=footprint, stream=stream)
+            _trace_pass(tr, grid, phi, steps, footprint=footprint, stream=stream)
             k, kb = tr.finalize(stream=stream)
             segs = tr.segments()
         finally:
@@ -117,7 +117,7 @@ def _make_autograd():
             if y1 > y0:
                 tr = Tracer(bundle, rows=(y0, y1))
                 flat = phi.detach().contiguous()
-                held = _trace_pass(tr, grid, flat, steps, footprint=footprint)
+                _trace_pass(tr, grid, flat, steps, footprint=footprint)
                 k, kb = tr.finalize()
             else:
                 k = torch.empty((0, int(bundle.nx)), dtype=torch.float64, device=phi.device)
