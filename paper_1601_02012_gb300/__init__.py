@@ -484,8 +484,9 @@ def _trace_pass(tr, grid, phi, steps, delta=None, footprint=True, stream=None, g
     launch and each of these steps reads them, unless that box holds so many
     more points than the footprints together that a launch per step costs less.
     Periodic trilinear bundles in the FP32 walk keep such boxes alone, one per
-    ``group`` steps (box-local: no wrap in the walk); the other forms, and cones
-    that reach around the box, write into a whole grid's buffer. ``group`` steps
+    ``group`` steps (box-local: no wrap in the walk); the other forms, cones
+    that reach around the box and boxes of 2^31 points write into a whole grid's
+    buffer. ``group`` steps
     are traced per launch (16 at most); group=1: one rr_trace_step per step on
     whole-grid records.
 
@@ -500,7 +501,8 @@ def _trace_pass(tr, grid, phi, steps, delta=None, footprint=True, stream=None, g
         (flags & _rr.RR_PERIODIC) and not (flags & _rr.RR_FP64_DDA)
     if boxed:
         boxes = [tr.footprint(grid, st.chi_a, st.chi_b, pad=1) for st in steps]
-        boxed = all(bb[2 * a + 1] - bb[2 * a] < n[a] for bb in boxes for a in range(3))
+        boxed = all(bb[2 * a + 1] - bb[2 * a] < n[a] for bb in boxes for a in range(3)) and \
+            all(_points(bb) < 2 ** 31 for bb in boxes)
     if boxed:
         for i in range(0, len(steps), group):
             bbs = boxes[i:i + group]

@@ -113,3 +113,13 @@ def test_records_belong_to_the_stream(rrp, monkeypatch, call):
     else:
         getattr(rrp, "trace_" + call)(phi, g, b, steps, stream=s)
     assert watch.streams and all(x is s for x in watch.streams)
+
+
+@pytest.mark.parametrize("call", ["kappa", "shear"])
+def test_boxes_past_32_bits(rrp, call):
+    """Steps whose own boxes hold 2^31 points or more, which box-local records
+    do not take, run on whole-grid records."""
+    import torch
+    g = synth.Grid((2048, 2048, 2048), 2048.0)
+    b = synth.Bundle(8, 8, synth.deg(50), synth.deg(50), (1024.0, 1024.0, 2.0), 2000.0)
+    getattr(rrp, "trace_" + call)(torch.empty(g.n, device="meta"), g, b, _steps(b, 2))
