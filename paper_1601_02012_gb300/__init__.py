@@ -483,12 +483,12 @@ def _trace_pass(tr, grid, phi, steps, delta=None, footprint=True, stream=None, g
     records of the box that holds several steps' footprints are computed by one
     launch and each of these steps reads them, unless that box holds so many
     more points than the footprints together that a launch per step costs less.
+    No more records than a whole grid's are held at a time.
     Periodic trilinear bundles in the FP32 walk keep such boxes alone, one per
     ``group`` steps (box-local: no wrap in the walk); the other forms, cones
     that reach around the box and boxes of 2^31 points write into a whole grid's
-    buffer. ``group`` steps
-    are traced per launch (16 at most); group=1: one rr_trace_step per step on
-    whole-grid records.
+    buffer. ``group`` steps are traced per launch (16 at most); group=1: one
+    rr_trace_step per step on whole-grid records.
 
     The record buffers are ``stream``'s (_on): they are dropped here with the
     steps still queued."""
@@ -504,7 +504,8 @@ def _trace_pass(tr, grid, phi, steps, delta=None, footprint=True, stream=None, g
         boxed = all(bb[2 * a + 1] - bb[2 * a] < n[a] for bb in boxes for a in range(3)) and \
             all(_points(bb) < 2 ** 31 for bb in boxes)
     if boxed:
-        for i in range(0, len(steps), group):
+        i = 0
+        while i < len(steps):
             bbs = boxes[i:i + group]
             one = _union(bbs, n)
             if all(one[2 * a + 1] - one[2 * a] < n[a] for a in range(3)) and _points(one) < 2 ** 31 and _cheaper(one, bbs):
@@ -513,11 +514,15 @@ def _trace_pass(tr, grid, phi, steps, delta=None, footprint=True, stream=None, g
                 tr.tidal_box(grid, phi, rec, one, delta=delta, stream=stream)
                 bbs, recs = [one] * len(bbs), [rec] * len(bbs)
             else:
+                # (as many steps as hold no more records than the whole grid)
+                while len(bbs) > 1 and sum(_points(bb) for bb in bbs) > n[0] * n[1] * n[2]:
+                    bbs.pop()
                 with _on(stream):
                     recs = [box_record_buffer(bb, device=phi.device) for bb in bbs]
                 for bb, rec in zip(bbs, recs):
                     tr.tidal_box(grid, phi, rec, bb, delta=delta, stream=stream)
-            tr.steps(grid, recs, steps[i:i + group], boxes=bbs, stream=stream)
+            tr.steps(grid, recs, steps[i:i + len(bbs)], boxes=bbs, stream=stream)
+            i += len(bbs)
             rec = recs = None   # (the next group may take the memory)
         return
     with _on(stream):

@@ -60,3 +60,30 @@ def test_tiles_beside_other_work(rrp, monkeypatch, raw):
     assert len(recorded) == 3 and got[2] == want[2]
     for x, y in zip(got[:2], want[:2]):
         assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("form", ["kappa", "shear", "grad"])
+def test_deep_pass_equals_steps(rrp, form):
+    """Forty steps through ten periods, launched in groups that hold no more
+    than a whole grid's records, against the steps one by one: bit for bit."""
+    import torch
+    g = synth.Grid((48, 48, 48), 62.4)
+    b = synth.Bundle(29, 18, synth.deg(3), synth.deg(2), (31.0, 30.0, 1.0), 9.9 * g.n[2] * g.h)
+    cuts = np.linspace(b.chi_s, 0.0, 41)
+    steps = [synth.Step(float(x), float(y), 1.0 + 0.01 * i, 0.8) for i, (x, y) in enumerate(zip(cuts[:-1], cuts[1:]))]
+    phi = torch.from_numpy(synth.random_field(g.n, 8, np.float32)).cuda()
+    tr = rrp.Tracer(b, shear=form == "shear")
+    rec = tr.record_buffer(g)
+    tr.tidal(g, phi, rec)
+    for st in steps:
+        tr.step(g, rec, st.chi_a, st.chi_b, st.scale, st.a)
+    want = list(tr.finalize()) + (list(tr.shear()) if form == "shear" else [])
+    tr.close()
+    if form == "grad":
+        phi.requires_grad_(True)
+        got = list(rrp.TraceKappa.apply(phi, g, b, steps))
+    else:
+        got = list((rrp.trace_shear if form == "shear" else rrp.trace_kappa)(phi, g, b, steps))[:-1]
+    assert len(got) == len(want)
+    for x, y in zip(got, want):
+        assert torch.equal(x.detach(), y)

@@ -123,3 +123,21 @@ def test_boxes_past_32_bits(rrp, call):
     g = synth.Grid((2048, 2048, 2048), 2048.0)
     b = synth.Bundle(8, 8, synth.deg(50), synth.deg(50), (1024.0, 1024.0, 2.0), 2000.0)
     getattr(rrp, "trace_" + call)(torch.empty(g.n, device="meta"), g, b, _steps(b, 2))
+
+
+@pytest.mark.parametrize("call", ["kappa", "shear", "method_a", "tiles"])
+@pytest.mark.parametrize("n,depth,steps,fov", [(512, 10.0, 40, 5.0), (512, 18.0, 72, 3.0), (64, 1.0, 16, 40.0),
+                                               (512, 0.97, 40, 10.0)])
+def test_no_more_than_a_whole_grid(rrp, monkeypatch, call, n, depth, steps, fov):
+    """A pass never holds more records than a whole grid has, also where the
+    cone passes through many periods and each step has a box of its own."""
+    import torch
+    g = synth.Grid((n, n, n), float(n))
+    b = synth.Bundle(64, 64, synth.deg(fov), synth.deg(fov), (0.5 * n, 0.5 * n, 1.0), depth * n)
+    phi = torch.empty(g.n, device="meta")
+    watch = Buffers(monkeypatch)
+    if call == "tiles":
+        rrp.trace_tiles([(phi, g, b.obs)] * 2, b, _steps(b, steps))
+    else:
+        getattr(rrp, "trace_" + call)(phi, g, b, _steps(b, steps))
+    assert 0 < watch.peak <= g.ncells and watch.live == 0
