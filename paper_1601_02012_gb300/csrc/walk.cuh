@@ -535,9 +535,16 @@ __device__ __forceinline__ void ray_consts(const TraceArgs& A, long long rid, Wa
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         W.sgn[a] = nh[a] > 0.f ? -1 : 1;   // motion along a is -n_a
-        if constexpr (F64) W.v[a] = (R)(fabs(A.dir[3 * rid + a]) * A.inv_h);
-        else W.v[a] = fabsf(nh[a]) * A.inv_hf;
-        W.td[a] = W.v[a] > (R)0 ? (R)1 / W.v[a] : (R)0;
+        R va;
+        if constexpr (F64) va = (R)(fabs(A.dir[3 * rid + a]) * A.inv_h);
+        else va = fabsf(nh[a]) * A.inv_hf;
+        // (a rate of 2^-112 cells per unit length or less is none: the FP32 walks
+        // form multiples of td (up to a leaf of 2^8 cells), which may not overflow:
+        // 0 x inf is NaN)
+        const R ta = (R)1 / va;
+        const bool moves = F64 ? va > (R)0 : ta < (R)0x1p112;
+        W.v[a] = moves ? va : (R)0;
+        W.td[a] = moves ? ta : (R)0;
     }
     // (sums of products rounded as written: every kernel gets the same weights)
     W.w[0] = __fadd_rn(__fmul_rn(nh[1], nh[1]), __fmul_rn(nh[2], nh[2]));
