@@ -61,8 +61,9 @@ __device__ __forceinline__ void load_factors(const float G[7], float* __restrict
 
 // The contributions of a ray whose derivative is infinite or NaN, one by one:
 // in the product they would reach every point the warp flushes (0 x NaN).
-__device__ __noinline__ void add_alone(double* __restrict__ grad, float4 n, float gk, float gb, int nr, uint32_t P0,
-                                       uint32_t Da, uint32_t Db, float F0, float F1, float F2, float F3)
+template <class PT>
+__device__ __noinline__ void add_alone(double* __restrict__ grad, float4 n, float gk, float gb, int nr, PT P0, PT Da,
+                                       PT Db, float F0, float F1, float F2, float F3)
 {
     const float w[6] = {n.y * n.y + n.z * n.z, n.x * n.x + n.z * n.z, n.x * n.x + n.y * n.y,
                         -2.f * n.x * n.y,      -2.f * n.x * n.z,      -2.f * n.y * n.z};
@@ -92,9 +93,9 @@ __device__ __noinline__ void add_alone(double* __restrict__ grad, float4 n, floa
 // crossings, two most others (a warp that straddles a cell plane). Storing every
 // lane's 28 products and summing columns, as an earlier form did, moved five
 // times the shared-memory data.
-template <int NR>
-__device__ __forceinline__ void flush_points(double* __restrict__ grad, uint32_t P0, uint32_t Da, uint32_t Db,
-                                             const float* F, bool part, const float4 row[8], float* __restrict__ sm)
+template <int NR, class PT>
+__device__ __forceinline__ void flush_points(double* __restrict__ grad, PT P0, PT Da, PT Db, const float* F, bool part,
+                                             const float4 row[8], float* __restrict__ sm)
 {
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -102,8 +103,8 @@ __device__ __forceinline__ void flush_points(double* __restrict__ grad, uint32_t
     unsigned todo = __ballot_sync(FULL, part);
     while (todo) {
         const int lead = __ffs(todo) - 1;
-        const uint32_t k0 = __shfl_sync(FULL, P0, lead);
-        const uint32_t ka = NR == 4 ? __shfl_sync(FULL, Da, lead) : 0, kb = NR == 4 ? __shfl_sync(FULL, Db, lead) : 0;
+        const PT k0 = __shfl_sync(FULL, P0, lead);
+        const PT ka = NR == 4 ? __shfl_sync(FULL, Da, lead) : 0, kb = NR == 4 ? __shfl_sync(FULL, Db, lead) : 0;
         const bool in = (todo >> lane & 1) && P0 == k0 && (NR == 1 || (Da == ka && Db == kb));
         todo &= ~__ballot_sync(FULL, in);
         __syncwarp();
@@ -119,7 +120,7 @@ __device__ __forceinline__ void flush_points(double* __restrict__ grad, uint32_t
                 y = __ffma2_rn(make_float2(f.z, f.w), make_float2(row[i].z, row[i].w), y);
             }
             const float v = (x.x + y.x) + (x.y + y.y);
-            const uint32_t key = k0 + ((mr & 1) ? ka : 0) + ((mr & 2) ? kb : 0);
+            const PT key = k0 + ((mr & 1) ? ka : 0) + ((mr & 2) ? kb : 0);
             if (mc < 7 && v != 0.f) atomicAdd(grad + 8 * (size_t)key + mc, (double)v);
         }
     }
@@ -143,7 +144,7 @@ __device__ __forceinline__ void flush_points(double* __restrict__ grad, uint32_t
 // atomics below 21 %); 4 blocks per SM, 5 are 4 % slower. One step of 256 cells,
 // 1024^2 rays: backward 5.39 -> 3.00 ms; two steps of 32 cells, 96^2 rays: 287 ->
 // 58 us.
-template <int INTERP, class R, bool PER>
+template <int INTERP, class R, bool PER, class PT>
 __global__ void __launch_bounds__(32 * kAdjWarps, (INTERP == RR_TRILINEAR && sizeof(R) == 4) ? 4 : 1)
     trace_adjoint_kernel(const TraceArgs A, const AdjArgs B, const TileCfg tc)
 {
@@ -177,20 +178,21 @@ __global__ void __launch_bounds__(32 * kAdjWarps, (INTERP == RR_TRILINEAR && siz
     const R chis = (R)A.chi_s;
     const R ichis = F64 ? (R)(1.0 / A.chi_s) : (R)A.inv_chi_s_f;
     const R eps_rel = F64 ? (R)1.4551915228366852e-11 : (R)4.76837158203125e-07;
-    const uint32_t st[3] = {(uint32_t)A.n1 * (uint32_t)A.n2, (uint32_t)A.n2, 1u};
+    const PT st[3] = {(PT)A.n1 * (PT)A.n2, (PT)A.n2, 1};
     Walk<R> W;
     // point index of the cell's entry corner (vertex vlo on every axis) and the
     // index step from vlo to vhi per axis (periodic wrap included), modulo 2^32
-    // (2^32 points of 64 bytes do not fit the device); NGP: the cell's index
-    uint32_t P0 = 0, D[3] = {0, 0, 0};
+    // for grids of at most 2^32 points and modulo 2^64 for larger ones (PT); NGP:
+    // the cell's index
+    PT P0 = 0, D[3] = {0, 0, 0};
     if (alive) {
         float bh, bl, Lj, D0j;
         sub_step(rg, j, nsub, dsub, bh, bl, Lj, D0j);
         walk_setup<R>(A, rid, bh, bl, Lj, D0j, rg.hi, rg.lo, W);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            P0 += (uint32_t)(TRI ? W.vlo[a] : W.c[a]) * st[a];
-            D[a] = (uint32_t)(W.vhi[a] - W.vlo[a]) * st[a];
+            P0 += (PT)(TRI ? W.vlo[a] : W.c[a]) * st[a];
+            D[a] = (PT)(W.vhi[a] - W.vlo[a]) * st[a];
         }
     }
     float4 row[8];
@@ -203,11 +205,11 @@ __global__ void __launch_bounds__(32 * kAdjWarps, (INTERP == RR_TRILINEAR && siz
     }
     const bool work = alive;
     // a face (or cell) of this ray into the records, with the warp
-    auto flush = [&](uint32_t P, uint32_t Da, uint32_t Db, const float* F, bool part) {
+    auto flush = [&](PT P, PT Da, PT Db, const float* F, bool part) {
         constexpr int NR = TRI ? 4 : 1;
-        flush_points<NR>(B.grad, P, Da, Db, F, part && !odd, row, sm);
+        flush_points<NR, PT>(B.grad, P, Da, Db, F, part && !odd, row, sm);
         if (any_odd && odd && part)
-            add_alone(B.grad, A.dirh[rid], B.dkappa ? (float)(B.dkappa[rid] * B.kscale) : 0.f,
+            add_alone<PT>(B.grad, A.dirh[rid], B.dkappa ? (float)(B.dkappa[rid] * B.kscale) : 0.f,
                       B.dkborn ? (float)(B.dkborn[rid] * B.bscale) : 0.f, NR, P, Da, Db, F[0], F[TRI ? 1 : 0],
                       F[TRI ? 2 : 0], F[TRI ? 3 : 0]);
         __syncwarp();
@@ -291,13 +293,13 @@ __global__ void __launch_bounds__(32 * kAdjWarps, (INTERP == RR_TRILINEAR && siz
                         const int ncell = W.c[a] + W.sgn[a], nc = wrap_once(ncell, nn[a]);
                         // the ray leaves the box (no wrap): what is pending is flushed below
                         if (!PER && !A.periodic && (ncell < 0 || ncell >= nn[a])) alive = false;
-                        if constexpr (!TRI) P0 += (uint32_t)(nc - W.c[a]) * st[a];
+                        if constexpr (!TRI) P0 += (PT)(nc - W.c[a]) * st[a];
                         W.c[a] = nc;
                     }
                     if constexpr (TRI) {
                         const int nvhi = wrap_once(W.vhi[a] + W.sgn[a], nn[a]);
                         P0 += D[a];
-                        D[a] = (uint32_t)(nvhi - W.vhi[a]) * st[a];
+                        D[a] = (PT)(nvhi - W.vhi[a]) * st[a];
                         W.vhi[a] = nvhi;
                     }
                     kf[a] += (R)1;
@@ -325,7 +327,9 @@ using AdjKernel = void (*)(const TraceArgs, const AdjArgs, const TileCfg);
 template <int INTERP, class R>
 AdjKernel adj_kernel(const TraceArgs& a)
 {
-    return a.periodic ? trace_adjoint_kernel<INTERP, R, true> : trace_adjoint_kernel<INTERP, R, false>;
+    // (64-bit point indices: one kernel for periodic and bounded grids)
+    if ((long long)a.n0 * a.n1 * a.n2 > (1LL << 32)) return trace_adjoint_kernel<INTERP, R, false, unsigned long long>;
+    return a.periodic ? trace_adjoint_kernel<INTERP, R, true, uint32_t> : trace_adjoint_kernel<INTERP, R, false, uint32_t>;
 }
 
 }  // namespace
