@@ -346,7 +346,10 @@ cudaError_t launch_trace_adjoint(const TraceArgs& args, const AdjArgs& b, int in
         // every SM sub-partition 8 warps; shorter ones, of 4 cells at least, for
         // smaller bundles, which a few serial walks leave mostly idle
         const long long warps = (long long)grid.x * grid.y * kAdjWarps;
-        const long long want = 152LL * 4 * 8;
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const long long want = (sms > 0 ? sms : 1) * 4LL * 8;
         const float longest = a.sub_len, shortest = longest * (4.f / 32.f);
         float len = longest;
         if (warps * a.nsub < want) {
