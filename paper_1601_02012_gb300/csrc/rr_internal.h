@@ -186,7 +186,6 @@ cudaError_t launch_collect_words(const ClearItem* items, int n, HostWords* out, 
 // box at (i ey + j) ez + k
 cudaError_t launch_tidal(const rr_grid_desc& g, const float* phi, const float* delta, float* rec, int where,
                          const int32_t* bbox, cudaStream_t s, int kind = 0, bool compact = false);
-cudaError_t launch_trace(const TraceArgs& a, int interp, bool fp64_dda, cudaStream_t s);
 // Forms of the FP32 walk's sums.
 enum { kFormKahan = 0, kFormPlain = 1, kFormMoments = 2, kFormShear = 3, kFormMethodA = 4, kFormGeneric = 5 };
 // Record addressing of the trilinear walk (see trace.cu).

@@ -1117,11 +1117,6 @@ cudaError_t launch_trace_steps(const TraceArgs& a, const StepBlock& b, int inter
     }
 }
 
-cudaError_t launch_trace(const TraceArgs& a, int interp, bool fp64_dda, cudaStream_t s)
-{
-    return launch_trace(a, interp, fp64_dda, s, TileCfg{});
-}
-
 namespace {
 
 using BatchKernel = void (*)(const BatchArgs);
