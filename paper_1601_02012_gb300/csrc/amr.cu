@@ -647,7 +647,7 @@ template <class T>
 cudaError_t upload(T** dst, const std::vector<T>& src)
 {
     const size_t bytes = src.size() * sizeof(T);
-    cudaError_t e = cudaMalloc((void**)dst, bytes > 0 ? bytes : 16);
+    cudaError_t e = device_alloc((void**)dst, bytes > 0 ? bytes : 16);
     if (e == cudaSuccess && bytes) e = cudaMemcpy(*dst, src.data(), bytes, cudaMemcpyHostToDevice);
     return e;
 }
@@ -759,9 +759,9 @@ rr_status rr_amr_create(const rr_amr_desc* desc, const int32_t* const* octs, con
         if (e == cudaSuccess) e = upload(&A->d_corner, P.corner);
         if (e == cudaSuccess) e = upload(&A->d_leaf_cell, P.leaf_cell);
         if (e == cudaSuccess) e = upload(&A->d_coarse, P.coarse);
-        if (e == cudaSuccess) e = cudaMalloc((void**)&A->d_H, (size_t)A->h.ncells * 8 * sizeof(float));
+        if (e == cudaSuccess) e = device_alloc((void**)&A->d_H, (size_t)A->h.ncells * 8 * sizeof(float));
         if (e == cudaSuccess)
-            e = cudaMalloc((void**)&A->d_V, (size_t)std::max<int64_t>(A->nverts, 1) * 8 * sizeof(float));
+            e = device_alloc((void**)&A->d_V, (size_t)std::max<int64_t>(A->nverts, 1) * 8 * sizeof(float));
         st = status_of_cuda(e);
     }
     if (st != RR_OK) {

@@ -112,13 +112,13 @@ rr_status rr_batch_create(int32_t n, const rr_bundle_desc* bundles, rr_batch** o
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev);
     if (b->sms < 1) b->sms = 1;
-    cudaError_t e = cudaMallocHost(&b->h_args, sizeof(TraceArgs) * (size_t)n);
-    if (e == cudaSuccess) e = cudaMallocHost(&b->h_tiles, sizeof(int) * (size_t)(2 * n + 1));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_args, sizeof(TraceArgs) * (size_t)n);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_tiles, sizeof(int) * (size_t)(2 * n + 1));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_counter, sizeof(int));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_items, sizeof(ClearItem) * (size_t)n);
-    if (e == cudaSuccess) e = cudaMallocHost(&b->h_words, sizeof(HostWords) * (size_t)n);
+    cudaError_t e = pinned_alloc((void**)&b->h_args, sizeof(TraceArgs) * (size_t)n);
+    if (e == cudaSuccess) e = pinned_alloc((void**)&b->h_tiles, sizeof(int) * (size_t)(2 * n + 1));
+    if (e == cudaSuccess) e = device_alloc((void**)&b->d_args, sizeof(TraceArgs) * (size_t)n);
+    if (e == cudaSuccess) e = device_alloc((void**)&b->d_tiles, sizeof(int) * (size_t)(2 * n + 1));
+    if (e == cudaSuccess) e = device_alloc((void**)&b->d_counter, sizeof(int));
+    if (e == cudaSuccess) e = device_alloc((void**)&b->d_items, sizeof(ClearItem) * (size_t)n);
+    if (e == cudaSuccess) e = pinned_alloc((void**)&b->h_words, sizeof(HostWords) * (size_t)n);
     if (e == cudaSuccess) {
         std::vector<ClearItem> items((size_t)n);
         for (int i = 0; i < n; ++i) {

@@ -5,11 +5,11 @@
 // against 50 us for a 64-cell step of 128^2 rays).
 //
 // Bounds: at most kMostBytes and kMostBlocks are kept, the oldest are freed
-// first, a block larger than kMostBytes is freed at once, an allocation that
-// fails empties the pool and is tried again, and rr_release_cached empties it on
-// demand. A block is handed out on the device it was allocated on, to one holder
-// at a time (a mutex guards the list), and is given back only after the device
-// has finished with it, so any stream and thread may use it next.
+// first, a block larger than kMostBytes is freed at once, an allocation of the
+// library that fails empties the pool and is tried again, and rr_release_cached
+// empties it on demand. A block is handed out on the device it was allocated on,
+// to one holder at a time (a mutex guards the list), and is given back only after
+// the device has finished with it, so any stream and thread may use it next.
 #include <mutex>
 #include <vector>
 
@@ -46,6 +46,32 @@ void pool_clear()
     for (const Block& b : all) release(b);
 }
 
+namespace {
+
+template <class F>
+cudaError_t alloc_again(F alloc)
+{
+    cudaError_t e = alloc();
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();   // (or the next launch would report it)
+    pool_clear();
+    e = alloc();
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+    return e;
+}
+
+}  // namespace
+
+cudaError_t device_alloc(void** p, size_t bytes)
+{
+    return alloc_again([&] { return cudaMalloc(p, bytes); });
+}
+
+cudaError_t pinned_alloc(void** p, size_t bytes)
+{
+    return alloc_again([&] { return cudaMallocHost(p, bytes); });
+}
+
 cudaError_t pool_take(size_t bytes, Block* out)
 {
     int dev = 0;
@@ -69,14 +95,9 @@ cudaError_t pool_take(size_t bytes, Block* out)
     Block b;
     b.bytes = bytes;
     b.device = dev;
-    e = cudaMalloc(&b.dev, bytes);
-    if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        pool_clear();
-        e = cudaMalloc(&b.dev, bytes);
-    }
+    e = device_alloc(&b.dev, bytes);
     if (e != cudaSuccess) return e;
-    e = cudaMallocHost(&b.host, sizeof(HostWords));
+    e = pinned_alloc(reinterpret_cast<void**>(&b.host), sizeof(HostWords));
     if (e != cudaSuccess) {
         cudaFree(b.dev);
         return e;

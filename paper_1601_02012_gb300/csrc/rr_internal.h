@@ -58,6 +58,10 @@ cudaError_t pool_take(size_t bytes, Block* out);
 // idle: the device has finished with the block (it may be kept); otherwise it is freed.
 void pool_give(const Block& b, bool idle);
 void pool_clear();
+// Every allocation of the library: cudaMalloc and cudaMallocHost that, where
+// memory is short, give the pool's kept blocks back and try once more.
+cudaError_t device_alloc(void** p, size_t bytes);
+cudaError_t pinned_alloc(void** p, size_t bytes);
 
 struct StepRecord {
     rr_grid_desc grid;

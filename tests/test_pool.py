@@ -1,0 +1,121 @@
+"""The pool of context memory (pool.cu) on a made-up device of a few megabytes,
+without a GPU: pool.cu itself, compiled for the host against the CUDA calls that
+it makes."""
+import os
+import re
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1601_02012_gb300", "csrc")
+CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+
+DEVICE = r"""
+#include <stdio.h>
+#include <stdlib.h>
+#include <map>
+#include <new>
+#include "pool.cu"
+
+static size_t g_room = 8 << 20, g_pins = 8;      // what is left of the device's memory, and pinned blocks
+static cudaError_t g_last = cudaSuccess;
+static std::map<void*, size_t> g_dev, g_pin;
+static bool g_no_new = false;
+
+void* operator new(size_t n)
+{
+    if (g_no_new) throw std::bad_alloc();
+    return malloc(n);
+}
+void operator delete(void* p) noexcept { free(p); }
+void operator delete(void* p, size_t) noexcept { free(p); }
+
+extern "C" {
+cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
+cudaError_t cudaGetLastError() { const cudaError_t e = g_last; g_last = cudaSuccess; return e; }
+cudaError_t cudaMalloc(void** p, size_t n)
+{
+    if (n > g_room) return g_last = cudaErrorMemoryAllocation;
+    g_room -= n;
+    g_dev[*p = malloc(1)] = n;
+    return cudaSuccess;
+}
+cudaError_t cudaFree(void* p)
+{
+    if (!p) return cudaSuccess;
+    if (!g_dev.count(p)) return g_last = cudaErrorInvalidValue;
+    g_room += g_dev[p];
+    g_dev.erase(p);
+    return cudaSuccess;
+}
+cudaError_t cudaMallocHost(void** p, size_t)
+{
+    if (!g_pins) return g_last = cudaErrorMemoryAllocation;
+    --g_pins;
+    g_pin[*p = malloc(64)] = 1;
+    return cudaSuccess;
+}
+cudaError_t cudaFreeHost(void* p)
+{
+    if (!p) return cudaSuccess;
+    if (!g_pin.count(p)) return g_last = cudaErrorInvalidValue;
+    ++g_pins;
+    g_pin.erase(p);
+    return cudaSuccess;
+}
+}
+
+#define CHECK(x) do { if (!(x)) { fprintf(stderr, "line %d: %s\n", __LINE__, #x); exit(1); } } while (0)
+
+using namespace rr;
+"""
+
+
+@pytest.fixture
+def run(tmp_path):
+    def go(body):
+        src, exe = tmp_path / "pool_test.cpp", tmp_path / "pool_test"
+        src.write_text(DEVICE + "int main()\n{\n" + body + "\n}\n")
+        cmd = ["g++", "-std=c++17", "-O1", "-w", "-pthread", "-I" + os.path.join(ROOT, "include"), "-I" + CSRC,
+               "-I" + os.path.join(CUDA, "include"), str(src), "-o", str(exe)]
+        p = subprocess.run(cmd, capture_output=True, text=True)
+        assert p.returncode == 0, p.stderr[:3000]
+        p = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
+        assert p.returncode == 0, p.stderr
+    return go
+
+
+def test_short_memory_takes_the_kept_blocks(run):
+    run(r"""
+    Block a, b;
+    void* p = nullptr;
+    CHECK(pool_take(6 << 20, &a) == cudaSuccess);
+    pool_give(a, true);
+    CHECK(device_alloc(&p, 4 << 20) == cudaSuccess);             // does not fit beside the kept block
+    CHECK(g_dev.size() == 1 && cudaGetLastError() == cudaSuccess);
+    CHECK(device_alloc(&p, 5 << 20) == cudaErrorMemoryAllocation);
+    CHECK(cudaGetLastError() == cudaSuccess);                    // (no launch after it fails)
+    cudaFree(p);
+    // pinned memory, the pool's own words among it
+    g_pins = 1;
+    CHECK(pool_take(1 << 20, &a) == cudaSuccess && g_pins == 0);
+    pool_give(a, true);
+    CHECK(pinned_alloc(&p, 64) == cudaSuccess && g_dev.empty());
+    cudaFreeHost(p);
+    CHECK(pool_take(1 << 20, &a) == cudaSuccess);
+    pool_give(a, true);
+    CHECK(pool_take(4 << 20, &b) == cudaSuccess);
+    pool_give(b, true);
+    CHECK(g_dev.size() == 1 && g_pins == 0);
+    rr_release_cached();
+    CHECK(g_dev.empty() && g_pin.empty());
+    """)
+
+
+def test_every_allocation_can_take_them():
+    """No file but pool.cu asks the driver for memory itself."""
+    for name in sorted(os.listdir(CSRC)):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+        if name != "pool.cu":
+            assert not re.search(r"\bcuda(Malloc\w*|HostAlloc)\s*\(", text), name
