@@ -11,6 +11,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <memory>
 #include <new>
 #include <vector>
 
@@ -120,12 +121,16 @@ rr_status rr_batch_create(int32_t n, const rr_bundle_desc* bundles, rr_batch** o
     if (e == cudaSuccess) e = device_alloc((void**)&b->d_items, sizeof(ClearItem) * (size_t)n);
     if (e == cudaSuccess) e = pinned_alloc((void**)&b->h_words, sizeof(HostWords) * (size_t)n);
     if (e == cudaSuccess) {
-        std::vector<ClearItem> items((size_t)n);
+        std::unique_ptr<ClearItem[]> items(new (std::nothrow) ClearItem[(size_t)n]);
+        if (!items) {
+            free_batch(b);
+            return RR_ERR_OOM;
+        }
         for (int i = 0; i < n; ++i) {
             const rr_ctx* c = b->cones[(size_t)i];
             items[(size_t)i] = ClearItem{c->st, (long long)c->bundle.nx * c->bundle.ny};
         }
-        e = cudaMemcpy(b->d_items, items.data(), sizeof(ClearItem) * (size_t)n, cudaMemcpyHostToDevice);
+        e = cudaMemcpy(b->d_items, items.get(), sizeof(ClearItem) * (size_t)n, cudaMemcpyHostToDevice);
     }
     if (e != cudaSuccess) {
         free_batch(b);

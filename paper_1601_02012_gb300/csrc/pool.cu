@@ -11,7 +11,6 @@
 // to one holder at a time (a mutex guards the list), and is given back only after
 // the device has finished with it, so any stream and thread may use it next.
 #include <mutex>
-#include <vector>
 
 #include "rr_internal.h"
 
@@ -21,12 +20,21 @@ namespace {
 constexpr size_t kMostBytes = (size_t)1 << 30;
 constexpr size_t kMostBlocks = 64;
 
+// The kept blocks, oldest first. An array: a call that gives memory back may
+// not fail for want of memory.
+struct List {
+    Block b[kMostBlocks];
+    size_t n = 0;
+    Block remove(size_t i)
+    {
+        const Block r = b[i];
+        for (--n; i < n; ++i) b[i] = b[i + 1];
+        return r;
+    }
+};
+
 std::mutex g_mutex;
-std::vector<Block>& kept()
-{
-    static std::vector<Block>* v = new std::vector<Block>();   // never destroyed: outlives every context
-    return *v;
-}
+List g_kept;
 
 void release(const Block& b)
 {
@@ -38,12 +46,13 @@ void release(const Block& b)
 
 void pool_clear()
 {
-    std::vector<Block> all;
+    List all;
     {
         std::lock_guard<std::mutex> lock(g_mutex);
-        all.swap(kept());
+        all = g_kept;
+        g_kept.n = 0;
     }
-    for (const Block& b : all) release(b);
+    for (size_t i = 0; i < all.n; ++i) release(all.b[i]);
 }
 
 namespace {
@@ -79,16 +88,16 @@ cudaError_t pool_take(size_t bytes, Block* out)
     if (e != cudaSuccess) return e;
     {
         std::lock_guard<std::mutex> lock(g_mutex);
-        std::vector<Block>& v = kept();
-        size_t best = v.size();
+        const List& v = g_kept;
+        size_t best = v.n;
         // the smallest that fits and wastes no more than a quarter (or 1 MB)
-        for (size_t i = 0; i < v.size(); ++i)
-            if (v[i].device == dev && v[i].bytes >= bytes && v[i].bytes - bytes <= bytes / 4 + ((size_t)1 << 20) &&
-                (best == v.size() || v[i].bytes < v[best].bytes))
+        for (size_t i = 0; i < v.n; ++i)
+            if (v.b[i].device == dev && v.b[i].bytes >= bytes &&
+                v.b[i].bytes - bytes <= bytes / 4 + ((size_t)1 << 20) &&
+                (best == v.n || v.b[i].bytes < v.b[best].bytes))
                 best = i;
-        if (best < v.size()) {
-            *out = v[best];
-            v.erase(v.begin() + (long)best);
+        if (best < v.n) {
+            *out = g_kept.remove(best);
             return cudaSuccess;
         }
     }
@@ -109,28 +118,22 @@ cudaError_t pool_take(size_t bytes, Block* out)
 void pool_give(const Block& b, bool idle)
 {
     if (!b.dev) return;
-    if (!idle) {
+    if (!idle || b.bytes > kMostBytes) {
         release(b);
         return;
     }
-    std::vector<Block> old;
+    List old;
     {
         std::lock_guard<std::mutex> lock(g_mutex);
-        std::vector<Block>& v = kept();
         size_t total = b.bytes;
-        for (const Block& k : v) total += k.bytes;
-        if (b.bytes > kMostBytes) {
-            old.push_back(b);
-        } else {
-            while (!v.empty() && (total > kMostBytes || v.size() >= kMostBlocks)) {
-                total -= v.front().bytes;
-                old.push_back(v.front());
-                v.erase(v.begin());
-            }
-            v.push_back(b);
+        for (size_t i = 0; i < g_kept.n; ++i) total += g_kept.b[i].bytes;
+        while (g_kept.n && (total > kMostBytes || g_kept.n == kMostBlocks)) {
+            total -= g_kept.b[0].bytes;
+            old.b[old.n++] = g_kept.remove(0);
         }
+        g_kept.b[g_kept.n++] = b;
     }
-    for (const Block& k : old) release(k);
+    for (size_t i = 0; i < old.n; ++i) release(old.b[i]);
 }
 
 }  // namespace rr

@@ -113,6 +113,34 @@ def test_short_memory_takes_the_kept_blocks(run):
     """)
 
 
+def test_giving_back_takes_no_memory(run):
+    """A block is kept, an old one dropped and all released while the host has
+    no memory left (a C++ exception through the C interface otherwise)."""
+    run(r"""
+    g_pins = g_room = (size_t)1 << 40;
+    Block a[70];
+    for (Block& b : a) CHECK(pool_take(64, &b) == cudaSuccess);
+    g_no_new = true;
+    for (Block& b : a) pool_give(b, true);
+    CHECK(g_dev.size() == 64);                                   // the most that are kept
+    pool_clear();
+    CHECK(g_dev.empty());
+    g_no_new = false;
+    // the oldest go first, and the smallest that fits is taken
+    Block x, y, z;
+    CHECK(pool_take((size_t)600 << 20, &x) == cudaSuccess && pool_take((size_t)500 << 20, &y) == cudaSuccess);
+    pool_give(x, true);
+    pool_give(y, true);                                          // over 1 GiB together
+    CHECK(g_dev.size() == 1 && g_dev.count(y.dev));
+    CHECK(pool_take((size_t)450 << 20, &z) == cudaSuccess && z.dev == y.dev);
+    pool_give(z, false);                                         // not idle: freed
+    CHECK(g_dev.empty());
+    CHECK(pool_take((size_t)2 << 30, &z) == cudaSuccess);
+    pool_give(z, true);                                          // larger than what is kept
+    CHECK(g_dev.empty() && g_pin.empty());
+    """)
+
+
 def test_every_allocation_can_take_them():
     """No file but pool.cu asks the driver for memory itself."""
     for name in sorted(os.listdir(CSRC)):
