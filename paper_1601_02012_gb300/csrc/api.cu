@@ -332,7 +332,10 @@ static rr_status create_context(const rr_bundle_desc* bundle, int32_t y0, int32_
     e = launch_init_state(*bundle, s, 0, y0, y1 - y0);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
-        pool_give(ctx->block, false);
+        // kept, not freed: while a stream is captured, which refuses the launch
+        // or the wait, it refuses to free memory too. The block's next holder
+        // initialises it on the same stream, after what may still run here.
+        pool_give(ctx->block, true);
         delete ctx;
         return from_cuda(e);
     }

@@ -55,7 +55,8 @@ struct Block {
     int device = -1;
 };
 cudaError_t pool_take(size_t bytes, Block* out);
-// idle: the device has finished with the block (it may be kept); otherwise it is freed.
+// idle: nothing but the default stream still uses the block (it may be kept);
+// otherwise it is freed.
 void pool_give(const Block& b, bool idle);
 void pool_clear();
 // Every allocation of the library: cudaMalloc and cudaMallocHost that, where
