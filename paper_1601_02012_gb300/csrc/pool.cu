@@ -9,7 +9,12 @@
 // library that fails empties the pool and is tried again, and rr_release_cached
 // empties it on demand. A block is handed out on the device it was allocated on,
 // to one holder at a time (a mutex guards the list), and is given back only after
-// the device has finished with it, so any stream and thread may use it next.
+// the device has finished with it, so any stream and thread may use it next. A
+// block whose CUDA context is gone (cudaDeviceReset) went with it: it is neither
+// handed out nor freed.
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
 #include <mutex>
 
 #include "rr_internal.h"
@@ -36,10 +41,31 @@ struct List {
 std::mutex g_mutex;
 List g_kept;
 
+// The number of the current CUDA context, made current for device dev where the
+// thread has none (numbers are not used again; 0: the driver tells none).
+unsigned long long context_id(int dev)
+{
+    static const PFN_cuCtxGetId_v12000 get = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q);
+        return reinterpret_cast<PFN_cuCtxGetId_v12000>(e == cudaSuccess && q == cudaDriverEntryPointSuccess ? p : nullptr);
+    }();
+    unsigned long long id = 0;
+    if (!get || get(nullptr, &id) == CUDA_SUCCESS) return id;
+    return cudaSetDevice(dev) == cudaSuccess && get(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
 void release(const Block& b)
 {
-    cudaFree(b.dev);
-    cudaFreeHost(b.host);
+    int dev = b.device;
+    cudaGetDevice(&dev);
+    if (dev != b.device) cudaSetDevice(b.device);
+    if (context_id(b.device) == b.context) {
+        cudaFree(b.dev);
+        cudaFreeHost(b.host);
+    }
+    if (dev != b.device) cudaSetDevice(dev);
 }
 
 }  // namespace
@@ -86,13 +112,14 @@ cudaError_t pool_take(size_t bytes, Block* out)
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
+    const unsigned long long context = context_id(dev);
     {
         std::lock_guard<std::mutex> lock(g_mutex);
         const List& v = g_kept;
         size_t best = v.n;
         // the smallest that fits and wastes no more than a quarter (or 1 MB)
         for (size_t i = 0; i < v.n; ++i)
-            if (v.b[i].device == dev && v.b[i].bytes >= bytes &&
+            if (v.b[i].device == dev && v.b[i].context == context && v.b[i].bytes >= bytes &&
                 v.b[i].bytes - bytes <= bytes / 4 + ((size_t)1 << 20) &&
                 (best == v.n || v.b[i].bytes < v.b[best].bytes))
                 best = i;
@@ -104,6 +131,7 @@ cudaError_t pool_take(size_t bytes, Block* out)
     Block b;
     b.bytes = bytes;
     b.device = dev;
+    b.context = context;
     e = device_alloc(&b.dev, bytes);
     if (e != cudaSuccess) return e;
     e = pinned_alloc(reinterpret_cast<void**>(&b.host), sizeof(HostWords));
@@ -118,7 +146,7 @@ cudaError_t pool_take(size_t bytes, Block* out)
 void pool_give(const Block& b, bool idle)
 {
     if (!b.dev) return;
-    if (!idle || b.bytes > kMostBytes) {
+    if (!idle || b.bytes > kMostBytes || context_id(b.device) != b.context) {
         release(b);
         return;
     }

@@ -53,6 +53,7 @@ struct Block {
     size_t bytes = 0;
     HostWords* host = nullptr;
     int device = -1;
+    unsigned long long context = 0;   // the CUDA context both belong to
 };
 cudaError_t pool_take(size_t bytes, Block* out);
 // idle: nothing but the default stream still uses the block (it may be kept);

@@ -22,6 +22,7 @@ static size_t g_room = 8 << 20, g_pins = 8;      // what is left of the device's
 static cudaError_t g_last = cudaSuccess;
 static std::map<void*, size_t> g_dev, g_pin;
 static bool g_no_new = false;
+static unsigned long long g_context = 7;         // 0: none is current
 
 void* operator new(size_t n)
 {
@@ -33,6 +34,24 @@ void operator delete(void* p, size_t) noexcept { free(p); }
 
 extern "C" {
 cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
+static unsigned long long g_next = 8;
+cudaError_t cudaSetDevice(int)
+{
+    if (!g_context) g_context = g_next++;
+    return cudaSuccess;
+}
+static CUresult context(CUcontext, unsigned long long* id)
+{
+    *id = g_context;
+    return g_context ? CUDA_SUCCESS : CUDA_ERROR_INVALID_CONTEXT;
+}
+cudaError_t cudaGetDriverEntryPointByVersion(const char*, void** p, unsigned, unsigned long long,
+                                             cudaDriverEntryPointQueryResult* q)
+{
+    *p = (void*)context;
+    *q = cudaDriverEntryPointSuccess;
+    return cudaSuccess;
+}
 cudaError_t cudaGetLastError() { const cudaError_t e = g_last; g_last = cudaSuccess; return e; }
 cudaError_t cudaMalloc(void** p, size_t n)
 {
@@ -138,6 +157,28 @@ def test_giving_back_takes_no_memory(run):
     CHECK(pool_take((size_t)2 << 30, &z) == cudaSuccess);
     pool_give(z, true);                                          // larger than what is kept
     CHECK(g_dev.empty() && g_pin.empty());
+    """)
+
+
+def test_blocks_go_with_their_context(run):
+    """After a device reset the kept blocks are neither handed out nor freed (the
+    memory at their addresses is someone else's); a thread that has no context
+    current yet gets the device's own."""
+    run(r"""
+    Block a, b, c;
+    CHECK(pool_take(1 << 20, &a) == cudaSuccess && pool_take(1 << 20, &b) == cudaSuccess);
+    pool_give(a, true);
+    g_context = 0;
+    g_next = 7;                                                  // no context current in this thread
+    CHECK(pool_take(1 << 20, &c) == cudaSuccess && c.dev == a.dev);
+    pool_give(c, true);
+    g_context = 0;
+    g_next = 9;                                                  // the device was reset
+    CHECK(pool_take(1 << 20, &c) == cudaSuccess && c.dev != a.dev && c.dev != b.dev);
+    pool_give(b, true);                                          // of a context made before it
+    pool_give(c, true);
+    rr_release_cached();
+    CHECK(g_dev.size() == 2 && g_dev.count(a.dev) && g_dev.count(b.dev) && cudaGetLastError() == cudaSuccess);
     """)
 
 
