@@ -7,6 +7,8 @@ tensors into them. PyTorch only provides device memory and streams.
 """
 from __future__ import annotations
 
+import contextlib
+
 from . import _rr
 from ._rr import (RR_AT_CENTRES, RR_AT_VERTICES, RR_NGP, RR_TRILINEAR, RRError, bundle_desc, grid_desc,
                   rr_create, rr_create_band, rr_destroy, rr_finalize, rr_footprint_bbox, rr_reset, rr_segment_count,
@@ -461,15 +463,16 @@ def _cheaper(one, boxes):
     return _points(one) <= sum(_points(bb) for bb in boxes) + (len(boxes) - 1) * _LAUNCH_POINTS
 
 
+_AS_IT_IS = contextlib.nullcontext()
+
+
 def _on(stream):
     """A context in which torch allocates for ``stream`` (a torch stream, a raw
     handle, or None: the current one): memory freed by Python while work on
     ``stream`` still uses it then goes to later work on that stream alone."""
-    import contextlib
-
-    import torch
     if stream is None:
-        return contextlib.nullcontext()
+        return _AS_IT_IS
+    import torch
     if not isinstance(stream, torch.cuda.Stream):
         raw = stream if isinstance(stream, int) else int(stream.cuda_stream)
         stream = torch.cuda.ExternalStream(raw) if raw else torch.cuda.default_stream()
@@ -496,13 +499,14 @@ def _trace_pass(tr, grid, phi, steps, delta=None, footprint=True, stream=None, g
     if not steps:
         return
     n = [int(v) for v in grid.n]
+    cells = n[0] * n[1] * n[2]
     interp, flags = int(tr.desc.interp), int(tr.desc.flags)
     boxed = group > 1 and footprint and not (tr.method_a or tr.generic) and interp == RR_TRILINEAR and \
         (flags & _rr.RR_PERIODIC) and not (flags & _rr.RR_FP64_DDA)
     if boxed:
         boxes = [tr.footprint(grid, st.chi_a, st.chi_b, pad=1) for st in steps]
         boxed = all(bb[2 * a + 1] - bb[2 * a] < n[a] for bb in boxes for a in range(3)) and \
-            all(_points(bb) < 2 ** 31 for bb in boxes)
+            (cells < 2 ** 31 or all(_points(bb) < 2 ** 31 for bb in boxes))
     if boxed:
         i = 0
         while i < len(steps):
@@ -515,8 +519,10 @@ def _trace_pass(tr, grid, phi, steps, delta=None, footprint=True, stream=None, g
                 bbs, recs = [one] * len(bbs), [rec] * len(bbs)
             else:
                 # (as many steps as hold no more records than the whole grid)
-                while len(bbs) > 1 and sum(_points(bb) for bb in bbs) > n[0] * n[1] * n[2]:
+                points = [_points(bb) for bb in bbs]
+                while len(bbs) > 1 and sum(points) > cells:
                     bbs.pop()
+                    points.pop()
                 with _on(stream):
                     recs = [box_record_buffer(bb, device=phi.device) for bb in bbs]
                 for bb, rec in zip(bbs, recs):
