@@ -198,7 +198,7 @@ enum { kFormKahan = 0, kFormPlain = 1, kFormMoments = 2, kFormShear = 3, kFormMe
 enum { kAddrIndex = 0, kAddrPlanes = 1, kAddrFlat = 2, kAddrAuto = 3 };
 // flat: the caller has checked that no ray of the step comes within a cell of
 // the periodic seam and that the grid has fewer than 2^31 points (used by the
-// default FP32 trilinear periodic form only; ignored otherwise).
+// FP32 trilinear periodic forms; ignored otherwise).
 // wrapped: wrapped indices throughout instead of a choice per sub-step
 // (trilinear; seam_heavy).
 cudaError_t launch_trace(const TraceArgs& a, int interp, bool fp64_dda, cudaStream_t s, const TileCfg& t,

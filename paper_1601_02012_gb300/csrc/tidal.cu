@@ -275,8 +275,8 @@ __global__ void __launch_bounds__(NT, 3) tidal_kernel(const TidalArgs a, const _
     for (int k = 0; k < 2; ++k)
 #pragma unroll
         for (int q = 0; q < NC; ++q) prev[k][q] = 0.f;
-    // carried along x: the eight values of a plane that the next plane's stencils
-    // read as their neighbours below (b) and two planes of them (c: the current one)
+    // carried along x: the eight values of a plane that the stencils of the planes
+    // beside it read, of planes c - 1 (vb), c (va) and c + 1 (vc)
     const int om = o - RP, o1 = o + RP, op = o + 2 * RP;
     auto eight = [&](const float* P, float v[8]) {
         v[0] = P[om]; v[1] = P[o]; v[2] = P[o1]; v[3] = P[op];
@@ -293,22 +293,24 @@ __global__ void __launch_bounds__(NT, 3) tidal_kernel(const TidalArgs a, const _
         if (s2 == 0) par ^= 1u;
         float nxt2[LP];
         if (tma) {
-            // plane c + 3 into the slot of plane c - 2, read before the last barrier
+            // plane c + 4 into the slot of plane c - 2, last read before that plane's barrier
             if (threadIdx.x == 0 && c + 4 <= c_last + 1) {
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 issue(c + 4);
             }
             ok = mbar_wait(&mbar[s2], par) && ok;
         } else {
-            // plane c + 2 goes into the slot of plane c - 3 (read before the last
-            // barrier); plane c + 3 is fetched into registers, a whole plane of
-            // work ahead of its use
+            // plane c + 2 goes into the slot of plane c - 4 (last read before that
+            // plane's barrier); plane c + 3 is fetched into registers, a whole plane
+            // of work ahead of its use
             if (c + 3 <= c_last + 1) fetch(c + 3, nxt2);
             if (c + 2 <= c_last + 1) put(slot(c + 2), nxt);
         }
 
-        // the two stencils: rows r0 - 1 .. r0 + 2 of P1 at z - 1 .. z + 1, rows
-        // r0 - 1 .. r0 + 2 of P0 and P2 at z, rows r0, r0 + 1 of P0 and P2 at z +- 1
+        // the two stencils: rows r0 - 1 .. r0 + 2 of plane c at z - 1 .. z + 1, and
+        // of planes c - 1 and c + 1 rows r0 - 1 .. r0 + 2 at z, rows r0, r0 + 1 at
+        // z +- 1. vb, va and vc hold these eight values of planes c - 1, c and c + 1:
+        // read here are plane c + 1's and the four corners of plane c that va lacks
         eight(ring + s2 * SLOT, vc);
         s1 = s2;
         const float a_m0 = P1[om - 1], a_m1 = va[0], a_m2 = P1[om + 1];
