@@ -523,15 +523,16 @@ __device__ __forceinline__ void add_segment(const TraceArgs& A, const Walk<float
 // arithmetic. The loop holds crossings only; the segment that ends the
 // sub-step follows it, once for the whole warp, without the loads, the
 // projections and the corner shift that a crossing needs, and one test ends the
-// loop on the last segment and on the cap alike. Bound by issue slots (FMA pipes
-// 58 % and ALU 53 % busy at 74 % issue); production pass, trace kernels 22.62 ->
-// 21.52 ms without the last segment in the loop, 20.83 ms with one test, 20.33 ms
-// with the ray's constants hoisted (kHoist), 19.72 ms with the new corners
-// projected before the crossing's bookkeeping, 19.40 ms with the crossings of all
-// axes evaluated anew and the shift's selects ordered by the z face, the
-// commonest (one step of 256 cells 2.24 -> 2.13 ms, batch 8.91 -> 8.36 ms), and
-// 18.70 ms (batch 8.14 ms) with ray_consts' test for rates whose inverse
-// overflows (the same loop in other registers).
+// loop on the last segment and on the cap alike. Bound by issue slots and the
+// FP32 pipes (FMA 60 % and ALU 42 % busy at 72 % issue, 7.0 warp instructions a
+// segment); production pass, trace kernels 22.62 -> 21.52 ms without the last
+// segment in the loop, 20.83 ms with one test, 20.33 ms with the ray's constants
+// hoisted (kHoist), 19.72 ms with the new corners projected before the crossing's
+// bookkeeping, 19.40 ms with the crossings of all axes evaluated anew and the
+// shift's selects ordered by the z face, the commonest (one step of 256 cells
+// 2.24 -> 2.13 ms, batch 8.91 -> 8.36 ms), and 18.70 ms (batch 8.14 ms) with
+// ray_consts' test for rates whose inverse overflows, on which the loop compiles
+// to 8 % fewer instructions.
 // (B, D0, fd, SEAM: flat_start's; more: another sub-step follows; WIDE: a record in one 32-byte load)
 template <int INTERP, int FORM, bool SELECT, bool SEAM, bool WIDE = true>
 __device__ __forceinline__ void walk_flat(const TraceArgs& A, const float4* rec, const Walk<float>& W, const RayWeights& V, bool first,
