@@ -138,7 +138,8 @@ rr_status rr_create(const rr_bundle_desc* bundle, rr_ctx** out);
 /*
  * The library keeps the memory of destroyed contexts for later ones (at most
  * 1 GiB in at most 64 blocks per process; an allocation of its own that fails
- * frees it first). rr_release_cached gives all of it back now.
+ * frees it first). rr_release_cached gives all of it back now, for another
+ * allocator of the process that needs it.
  */
 rr_status rr_release_cached(void);
 
